@@ -558,9 +558,8 @@ int ftr_eval_appearance(ftr_ctx* ctx, int w, int h, const float* rendered_depth,
  * device allocation.  Every point gets the same accept / reject decision as
  * in ftr_solve (both follow the float64 quotient (X - b_min) / h - 1/2), and
  * the value matches ftr_solve's level within |dL| / (max A - min A) <= 1e-5,
- * but it is not bit-identical: the fractions are rounded from float64 rather
- * than through the ingest's float pair, and the partial sums are reduced in
- * a different tree (1024 points per CTA, then one warp).  The paper has no
+ * but it is not bit-identical: the partial sums are reduced in a different
+ * tree (whole multiples of 256 points per CTA, then one CTA).  The paper has no
  * counterpart: this entry point exists for callers that cannot allocate
  * device memory where they need the level -- a per-frame loop with a hard
  * latency budget (cudaMalloc/cudaFree may synchronise the device), or a host

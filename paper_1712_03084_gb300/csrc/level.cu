@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "ftr_internal.h"
+#include "node_pos.cuh"
 
 namespace ftr {
 namespace {
@@ -118,8 +119,8 @@ cudaError_t launch_level(ftr_ctx* c) {
 namespace ftr {
 namespace {
 
-constexpr int kNoAllocPointsPerCta = 1024;
-constexpr int kNoAllocMaxCtas = 4096;     // => at most 4,194,304 points per call
+constexpr int64_t kNoAllocMaxPoints = 4194304;
+constexpr int kNoAllocMaxCtas = 4096;
 // Partial (sum, count) per CTA plus (L, count) of the result: 64 KB + 16 B,
 // resident on every device that loads the library until the process exits.
 __device__ __align__(256) double g_noalloc_scratch[2 * kNoAllocMaxCtas + 2];
@@ -128,36 +129,50 @@ __device__ __align__(256) double g_noalloc_scratch[2 * kNoAllocMaxCtas + 2];
 std::mutex g_noalloc_mu;
 double* g_noalloc_ptr[64] = {};
 
-// t = (X - b_min) / h - 1/2 with every decision equal to the float64 quotient
-// (the same rule as the point ingest of the splat).
-__device__ __forceinline__ double noalloc_node_t(double x, double bmin, double h, double inv_h, double n) {
-    double t = (x - bmin) * inv_h - 0.5;
-    const double band = 1e-9 * (1.0 + fabs(t));
-    const double fr = t - floor(t);
-    if (fr < band || fr > 1.0 - band || fabs(t - 1.0) < band || fabs(t - (n - 2.0)) < band)
-        t = (x - bmin) / h - 0.5;
-    return t;
+// Points per CTA: 256 (one per thread) until the grid fills the chip once
+// (152 SMs x 8 CTAs of 256 threads), then whole multiples of 256 that keep it
+// to one wave; at the largest n that is 3584 points on 1171 CTAs.
+int noalloc_per_cta(int64_t n) {
+    constexpr int64_t kWave = 152 * 8;
+    const int64_t per = (n + kThreads * kWave - 1) / (kThreads * kWave);
+    return kThreads * (int)(per < 1 ? 1 : per);
 }
 
+// Per-CTA (sum, count) of trilinear A over the CTA's points.  The float64
+// quotient of every point decided this kernel's time (float64 runs at 1/64 of
+// the float32 rate: 42 us for 200,000 points of a 256^3 grid); the position is
+// taken from the float pair of node_t_pair instead, with float64 only within
+// 1e-6 of a decision, as in the ingest: the call with a host result went from
+// 77 to 39 us.  What is left is the latency of two dependent loads (the point,
+// then its eight nodes) and of the second launch, the copy and the wait.
 __global__ void __launch_bounds__(kThreads) k_level_noalloc_partial(GridDev g, const float* __restrict__ pts,
-                                                                    int64_t n, const float* __restrict__ A,
+                                                                    int64_t n, int per, const float* __restrict__ A,
                                                                     double* scratch) {
     __shared__ double sh[kThreads / 32];
+    __shared__ int shc[kThreads / 32];
     const int nx = g.n[0];
     const int64_t nxy = (int64_t)nx * g.n[1];
-    double sum = 0.0, cnt = 0.0;
-    const int64_t i0 = (int64_t)blockIdx.x * kNoAllocPointsPerCta;
-    for (int64_t i = i0 + threadIdx.x; i < i0 + kNoAllocPointsPerCta && i < n; i += kThreads) {
-        int b[3];
-        float f[3];
+    double sum = 0.0;
+    int cnt = 0;
+    const int64_t i0 = (int64_t)blockIdx.x * per;
+    for (int64_t i = i0 + threadIdx.x; i < i0 + per && i < n; i += kThreads) {
+        int b[3] = {0, 0, 0};
+        float f[3] = {0.f, 0.f, 0.f};
         bool ok = true;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double t = noalloc_node_t((double)pts[3 * i + c], g.bmin[c], g.h[c], g.inv_h[c], (double)g.n[c]);
-            ok = ok && (t >= 1.0) && (t < (double)g.n[c] - 2.0);
-            const double fl = ok ? floor(t) : 0.0;
-            b[c] = (int)fl;
-            f[c] = ok ? (float)(t - fl) : 0.f;
+            const float x = pts[3 * i + c];
+            bool up;
+            if (node_t_pair(x, g.bminf[c], g.inv_hf[c], g.inv_h_lo[c], b[c], f[c], up)) {
+                ok = ok && b[c] >= 1 && b[c] <= g.n[c] - 3;          // 1 <= t < n - 2
+            } else {
+                const double t = node_t((double)x, g.bmin[c], g.h[c], g.inv_h[c], (double)g.n[c]);
+                const bool in = (t >= 1.0) && (t < (double)g.n[c] - 2.0);   // false for NaN
+                ok = ok && in;
+                const double fl = in ? floor(t) : 0.0;
+                b[c] = (int)fl;
+                f[c] = in ? (float)(t - fl) : 0.f;
+            }
         }
         if (!ok) continue;
         const float* a0 = A + b[0] + (int64_t)nx * b[1] + nxy * b[2];
@@ -168,29 +183,45 @@ __global__ void __launch_bounds__(kThreads) k_level_noalloc_partial(GridDev g, c
         const float c0 = fmaf(f[1], c10 - c00, c00);
         const float c1 = fmaf(f[1], c11 - c01, c01);
         sum += (double)fmaf(f[2], c1 - c0, c0);
-        cnt += 1.0;
+        cnt += 1;
     }
-    const double s = block_sum(sum, sh);
-    const double c = block_sum(cnt, sh);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane == 0) {
+        sh[wid] = sum;
+        shc[wid] = cnt;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {          // every slot this call reads is written here first
+        double s = 0.0;
+        int c = 0;
+        for (int w = 0; w < kThreads / 32; ++w) {
+            s += sh[w];
+            c += shc[w];
+        }
         scratch[2 * blockIdx.x] = s;
-        scratch[2 * blockIdx.x + 1] = c;
+        scratch[2 * blockIdx.x + 1] = (double)c;
     }
 }
 
-__global__ void k_level_noalloc_final(double* scratch, int nblocks, double* level_dev) {
-    const int lane = threadIdx.x;
+// One CTA sums the partials in a fixed order.  Launched while the partial
+// kernel still runs (programmatic launch); it waits for that kernel's end.
+// (A last-CTA ticket would save this launch, but calls that overlap against
+// the contract could leave the ticket at a wrong value for good.)
+__global__ void __launch_bounds__(kThreads) k_level_noalloc_final(double* scratch, int nblocks, double* level_dev) {
+    pdl_wait();
+    __shared__ double sh[kThreads / 32];
     double s = 0.0, c = 0.0;
-    for (int b = lane; b < nblocks; b += 32) {
-        s += scratch[2 * b];
-        c += scratch[2 * b + 1];
+    for (int b = threadIdx.x; b < nblocks; b += kThreads) {
+        const double2 v = reinterpret_cast<const double2*>(scratch)[b];
+        s += v.x;
+        c += v.y;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_down_sync(0xffffffffu, s, o);
-        c += __shfl_down_sync(0xffffffffu, c, o);
-    }
-    if (lane == 0) {
+    s = block_sum(s, sh);
+    c = block_sum(c, sh);
+    if (threadIdx.x == 0) {
         const double L = c > 0.0 ? s / c : 0.0;
         scratch[2 * kNoAllocMaxCtas] = L;
         scratch[2 * kNoAllocMaxCtas + 1] = c;
@@ -212,7 +243,7 @@ extern "C" int ftr_iso_level_noalloc(const float* A, const int grid_n[3], const 
                                      int64_t n, double* level_out, void* stream) {
     using namespace ftr;
     if (!A || !grid_n || !bbox || !level_out || n < 0 || (n > 0 && !points)) return FTR_EINVAL;
-    if (n > (int64_t)kNoAllocPointsPerCta * kNoAllocMaxCtas) return FTR_EINVAL;   // beyond the static scratch
+    if (n > kNoAllocMaxPoints) return FTR_EINVAL;
     GridDev g{};
     for (int a = 0; a < 3; ++a) {
         if (!supported_axis(grid_n[a]) || !(bbox[3 + a] > bbox[a])) return FTR_EINVAL;
@@ -220,6 +251,9 @@ extern "C" int ftr_iso_level_noalloc(const float* A, const int grid_n[3], const 
         g.bmin[a] = (double)bbox[a];
         g.h[a] = ((double)bbox[3 + a] - (double)bbox[a]) / grid_n[a];
         g.inv_h[a] = 1.0 / g.h[a];
+        g.bminf[a] = bbox[a];
+        g.inv_hf[a] = (float)g.inv_h[a];
+        g.inv_h_lo[a] = (float)(g.inv_h[a] - (double)g.inv_hf[a]);
     }
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FTR_ECUDA;
@@ -249,11 +283,13 @@ extern "C" int ftr_iso_level_noalloc(const float* A, const int grid_n[3], const 
         if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return FTR_ECUDA;
         if (cs != cudaStreamCaptureStatusNone) return FTR_EINVAL;
     }
-    const int nblocks = n > 0 ? (int)((n + kNoAllocPointsPerCta - 1) / kNoAllocPointsPerCta) : 1;
-    k_level_noalloc_partial<<<nblocks, kThreads, 0, st>>>(g, points, n, A, scratch);
+    const int per = noalloc_per_cta(n);
+    const int nblocks = n > 0 ? (int)((n + per - 1) / per) : 1;
+    k_level_noalloc_partial<<<nblocks, kThreads, 0, st>>>(g, points, n, per, A, scratch);
     if (cudaGetLastError() != cudaSuccess) return FTR_ECUDA;
-    k_level_noalloc_final<<<1, 32, 0, st>>>(scratch, nblocks, out_on_device ? level_out : nullptr);
-    if (cudaGetLastError() != cudaSuccess) return FTR_ECUDA;
+    if (launch_pdl(k_level_noalloc_final, dim3(1), dim3(kThreads), 0, st, scratch, nblocks,
+                   out_on_device ? level_out : (double*)nullptr) != cudaSuccess)
+        return FTR_ECUDA;
     if (!out_on_device) {
         if (cudaMemcpyAsync(level_out, scratch + 2 * kNoAllocMaxCtas, sizeof(double), cudaMemcpyDeviceToHost, st) !=
             cudaSuccess)
