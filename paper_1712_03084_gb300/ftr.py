@@ -10,6 +10,7 @@ fallback.
 
 import ctypes
 import os
+import sys
 
 import numpy as np
 
@@ -59,6 +60,10 @@ class ftr_tex(ctypes.Structure):
 class ftr_point_set(ctypes.Structure):
     _fields_ = [("points", ctypes.c_void_p), ("normals", ctypes.c_void_p), ("weights", ctypes.c_void_p),
                 ("n", ctypes.c_int64)]
+
+
+_F9 = ctypes.c_float * 9
+_F12 = ctypes.c_float * 12
 
 
 class ftr_camera(ctypes.Structure):
@@ -170,6 +175,21 @@ def load():
     return lib
 
 
+_TORCH_NAMES = {np.float32: "float32", np.uint8: "uint8", np.int32: "int32"}
+_torch_dtypes = {}
+
+
+def _torch_dtype(dtype):
+    """The torch dtype of a numpy one (torch is loaded: a tensor is at hand)."""
+    want = _torch_dtypes.get(dtype)
+    if want is None:
+        torch = sys.modules.get("torch")
+        want = getattr(torch, _TORCH_NAMES[dtype], None)
+        if want is not None:
+            _torch_dtypes[dtype] = want
+    return want
+
+
 def _ptr(a, dtype=None):
     """Raw address of a numpy array or torch tensor (None -> NULL)."""
     if a is None:
@@ -183,14 +203,24 @@ def _ptr(a, dtype=None):
     if hasattr(a, "data_ptr"):
         if not a.is_contiguous():
             raise ValueError("tensor must be contiguous")
-        if dtype is not None:
-            want = {np.float32: "torch.float32", np.uint8: "torch.uint8", np.int32: "torch.int32"}[dtype]
-            if str(a.dtype) != want:
-                raise TypeError(f"expected {want}, got {a.dtype}")
+        # torch dtypes are singletons: the name is only built for the message
+        if dtype is not None and a.dtype is not _torch_dtype(dtype) and \
+                str(a.dtype) != f"torch.{_TORCH_NAMES[dtype]}":
+            raise TypeError(f"expected torch.{_TORCH_NAMES[dtype]}, got {a.dtype}")
         return a.data_ptr()
     if isinstance(a, int):
         return a
     raise TypeError(f"unsupported buffer type {type(a)}")
+
+
+def _floats(kind, m):
+    """A ctypes float array of ``kind`` from a matrix, copied whole (one numpy
+    conversion and one block copy: element by element, the four matrices of a
+    view took most of the host's share of a frame)."""
+    m = np.ascontiguousarray(m, dtype=np.float32)
+    if m.size != kind._length_:
+        raise ValueError(f"expected {kind._length_} values, got {m.size}")
+    return kind.from_buffer_copy(m)
 
 
 def _check(code, ctx=None):
@@ -275,11 +305,11 @@ def make_view(view):
     v.h, v.w = int(depth.shape[0]), int(depth.shape[1])
     if rgb is not None:
         v.rgb_h, v.rgb_w = int(rgb.shape[0]), int(rgb.shape[1])
-    v.K[:] = [float(x) for x in np.asarray(view["K"], dtype=np.float32).reshape(-1)]
-    v.world_to_cam[:] = [float(x) for x in np.asarray(view["world_to_cam"], dtype=np.float32).reshape(-1)]
+    v.K = _floats(_F9, view["K"])
+    v.world_to_cam = _floats(_F12, view["world_to_cam"])
     if "K_rgb" in view:
-        v.K_rgb[:] = [float(x) for x in np.asarray(view["K_rgb"], dtype=np.float32).reshape(-1)]
-        v.world_to_rgb[:] = [float(x) for x in np.asarray(view["world_to_rgb"], dtype=np.float32).reshape(-1)]
+        v.K_rgb = _floats(_F9, view["K_rgb"])
+        v.world_to_rgb = _floats(_F12, view["world_to_rgb"])
     v.depth = _ptr(depth, np.float32)
     v.conf = _ptr(conf, np.float32)
     v.rgb = _ptr(rgb, np.uint8)
@@ -300,8 +330,8 @@ def ftr_splat_depth(ctx, views, step=-1.0, noise=-1.0, radius=-1, conf_out=None,
 def make_camera(K, world_to_cam, w, h):
     cam = ftr_camera()
     cam.w, cam.h = int(w), int(h)
-    cam.K[:] = [float(x) for x in np.asarray(K, dtype=np.float32).reshape(-1)]
-    cam.world_to_cam[:] = [float(x) for x in np.asarray(world_to_cam, dtype=np.float32).reshape(-1)]
+    cam.K = _floats(_F9, K)
+    cam.world_to_cam = _floats(_F12, world_to_cam)
     return cam
 
 
