@@ -354,7 +354,9 @@ struct EvalScratch {
     float4* pts = nullptr;                // 2 x pixels: compacted sensor and rendered points (.w = pixel)
     float* d2 = nullptr;                  // pixels: squared closest-point distance per sensor pixel
     int64_t pix_cap = 0;
-    unsigned long long* cnt = nullptr;    // 8 counters (see evaluate.cu)
+    void* tiles = nullptr;                // per 16 x 16 pixel tile: box and place of its rendered points
+    int64_t tiles_cap = 0;
+    unsigned long long* cnt = nullptr;    // counters (see evaluate.cu)
     double* part = nullptr;               // per-block partial sums
     int64_t part_cap = 0;
     double* h_res = nullptr;              // pinned results
