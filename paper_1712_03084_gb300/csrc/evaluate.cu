@@ -24,12 +24,12 @@
 // Appearance (eq. (6)(7)), per scale j = 1..3:
 //   k_ap_luma / k_ap_down   luma planes and silhouette, then 2 x 2 block
 //                mean (silhouette: block AND) for the next scale;
-//   k_ap_ssim    16 x 16 pixels per CTA with an 11 x 11-window halo in shared
+//   k_ap_ssim    32 x 16 pixels per CTA with an 11 x 11-window halo in shared
 //                memory: per silhouette pixel the window means, then the
 //                second moments about those means (centred, so flat regions
 //                give exactly zero variance up to rounding of the mean),
 //                l, c, s and w(u); block partial sums in float64;
-//   k_sum_final  the partials in a fixed order.
+//   k_ap_final   the partials of every scale and term in a fixed order.
 // The host side combines the per-scale means into WMS3IM.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -44,9 +44,10 @@ namespace {
 
 constexpr int kNone = 1 << 28;      // column distance when the column holds no pixel of the set
 constexpr long long kFar = 0x7fffffffffffffffLL;   // no pixel of the set in the whole image
-constexpr int kTile = 16;           // appearance: output pixels per CTA side
+constexpr int kTile = 16;           // closest points: pixels per tile side
 constexpr int kR = 5;               // SSIM window radius (11 x 11)
-constexpr int kHalo = kTile + 2 * kR;
+constexpr int kSsimW = 32, kSsimH = 16;                                  // SSIM: output pixels per CTA
+constexpr int kHaloW = kSsimW + 2 * kR, kHaloH = kSsimH + 2 * kR;
 constexpr int kSumBlocks = 256;
 constexpr int kCpThreads = 64;      // closest points: small CTAs, so that one body's points reach every SM
 // counters of one geometry evaluation: |S_r|, |S_g|, |xor|, |or|, the two
@@ -370,22 +371,19 @@ __global__ void __launch_bounds__(256) k_sum(const T* __restrict__ v, int64_t n,
     if (threadIdx.x == 0) part[blockIdx.x] = s[0];
 }
 
-// out[c] = sum over blocks b of part[b * stride + c], c < comps, fixed order.
-__global__ void __launch_bounds__(256) k_sum_final(const double* __restrict__ part, int64_t nblocks, int comps,
-                                                   int stride, double* __restrict__ out) {
+// The block sums in a fixed order.
+__global__ void __launch_bounds__(256) k_sum_final(const double* __restrict__ part, int64_t nblocks,
+                                                   double* __restrict__ out) {
     __shared__ double s[256];
-    for (int c = 0; c < comps; ++c) {
-        double acc = 0.0;
-        for (int64_t b = threadIdx.x; b < nblocks; b += 256) acc += part[b * stride + c];
-        s[threadIdx.x] = acc;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[c] = s[0];
+    double acc = 0.0;
+    for (int64_t b = threadIdx.x; b < nblocks; b += 256) acc += part[b];
+    s[threadIdx.x] = acc;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
         __syncthreads();
     }
+    if (threadIdx.x == 0) out[0] = s[0];
 }
 
 __global__ void __launch_bounds__(256) k_ap_luma(const uint8_t* __restrict__ rr, const uint8_t* __restrict__ rg,
@@ -411,93 +409,225 @@ __global__ void __launch_bounds__(256) k_ap_down(const float* __restrict__ X, co
     S2[p] = S[a] & S[a + 1] & S[b] & S[b + 1];
 }
 
+// The SSIM terms of one pixel from its window moments, times the window's
+// silhouette count.
+struct SsimSums {
+    double l, c, s, w;
+};
+
+__device__ __forceinline__ void ssim_terms(float mx, float my, float vx, float vy, float cxy, int count, SsimSums& a) {
+    const float C1 = (0.01f * 255.f) * (0.01f * 255.f);
+    const float C2 = (0.03f * 255.f) * (0.03f * 255.f);
+    const float C3 = 0.5f * C2;
+    const float sgx = sqrtf(vx), sgy = sqrtf(vy);
+    const float l = (2.f * mx * my + C1) / (mx * mx + my * my + C1);
+    const float c = (2.f * sgx * sgy + C2) / (vx + vy + C2);
+    const float s = (cxy + C3) / (sgx * sgy + C3);
+    const double cw = (double)count;
+    a.l += cw * l;
+    a.c += cw * c;
+    a.s += cw * s;
+    a.w += cw;
+}
+
+// A thread takes two vertically adjacent pixels of a 32 x 16 tile.  The window
+// means are separable and keep the order of the direct sums: the row sums of
+// the 26 x 32 halo rows are formed once in shared memory and each pixel adds
+// its 11.  The second moments stay centred on each pixel's own mean (an
+// expansion about a common point would cancel in flat regions), so their 121
+// samples are read once for the two pixels.  A tile without silhouette pixels
+// ends after its loads; a tile that touches the image border takes the windows
+// cut at it.  (16 x 16 pixels with direct, bounds-tested 121-tap sums for the
+// means and the moments ran 182 + 137 + 57 us for the three scales of a 1920 x
+// 1080 view whose silhouette covers an eighth of it.)
 __global__ void __launch_bounds__(256) k_ap_ssim(const float* __restrict__ X, const float* __restrict__ Y,
-                                                 const uint8_t* __restrict__ S, int w, int h, Taps tp,
-                                                 double* __restrict__ part) {
-    __shared__ float sx[kHalo][kHalo + 1];
-    __shared__ float sy[kHalo][kHalo + 1];
-    __shared__ uint8_t ss[kHalo][kHalo + 1];
-    __shared__ double red[4][256];
-    const int bx = blockIdx.x * kTile - kR, by = blockIdx.y * kTile - kR;
-    for (int i = threadIdx.x; i < kHalo * kHalo; i += 256) {
-        const int ty = i / kHalo, tx = i % kHalo;
-        const int gx = bx + tx, gy = by + ty;
+                                                 const uint8_t* __restrict__ S, int w, int h,
+                                                 const __grid_constant__ Taps tp, double* __restrict__ part) {
+    __shared__ float sx[kHaloH][kHaloW];
+    __shared__ float sy[kHaloH][kHaloW];
+    __shared__ uint8_t ss[kHaloH][kHaloW + 2];
+    __shared__ float rowx[kHaloH][kSsimW];
+    __shared__ float rowy[kHaloH][kSsimW];
+    __shared__ int rown[kHaloH][kSsimW];
+    __shared__ double red[4][8];
+    const int bx = blockIdx.x * kSsimW - kR, by = blockIdx.y * kSsimH - kR;
+    const int tx = threadIdx.x % kSsimW, ty = 2 * (threadIdx.x / kSsimW);
+    const int x = blockIdx.x * kSsimW + tx, y = blockIdx.y * kSsimH + ty;
+    double* out = part + 4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x);
+    const bool in0 = x < w && y < h && S[(int64_t)y * w + x];
+    const bool in1 = x < w && y + 1 < h && S[(int64_t)(y + 1) * w + x];
+    if (!__syncthreads_or(in0 || in1)) {
+        if (threadIdx.x < 4) out[threadIdx.x] = 0.0;
+        return;
+    }
+    for (int i = threadIdx.x; i < kHaloH * kHaloW; i += 256) {
+        const int hy = i / kHaloW, hx = i % kHaloW;
+        const int gx = bx + hx, gy = by + hy;
         const bool in = gx >= 0 && gx < w && gy >= 0 && gy < h;
         const int64_t gi = (int64_t)gy * w + gx;
-        sx[ty][tx] = in ? X[gi] : 0.f;
-        sy[ty][tx] = in ? Y[gi] : 0.f;
-        ss[ty][tx] = in ? S[gi] : 0;
+        sx[hy][hx] = in ? X[gi] : 0.f;
+        sy[hy][hx] = in ? Y[gi] : 0.f;
+        ss[hy][hx] = in ? S[gi] : 0;
     }
     __syncthreads();
-    const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;
-    const int x = blockIdx.x * kTile + tx, y = blockIdx.y * kTile + ty;
-    double cl = 0.0, cc = 0.0, cs = 0.0, cw = 0.0;
-    if (x < w && y < h && ss[ty + kR][tx + kR]) {
-        const float C1 = (0.01f * 255.f) * (0.01f * 255.f);
-        const float C2 = (0.03f * 255.f) * (0.03f * 255.f);
-        const float C3 = 0.5f * C2;
-        // taps inside the image: i in [i0, i1], j in [j0, j1]
-        const int i0 = max(-kR, -x), i1 = min(kR, w - 1 - x);
-        const int j0 = max(-kR, -y), j1 = min(kR, h - 1 - y);
-        float gsx = 0.f, gsy = 0.f;
-        for (int i = i0; i <= i1; ++i) gsx += tp.g[i + kR];
-        for (int j = j0; j <= j1; ++j) gsy += tp.g[j + kR];
-        const float inv = 1.f / (gsx * gsy);
-        float mx = 0.f, my = 0.f;
-        int count = 0;
-        for (int j = j0; j <= j1; ++j) {
-            float rx = 0.f, ry = 0.f;
-            for (int i = i0; i <= i1; ++i) {
-                const float g = tp.g[i + kR];
-                rx += g * sx[ty + kR + j][tx + kR + i];
-                ry += g * sy[ty + kR + j][tx + kR + i];
-                count += ss[ty + kR + j][tx + kR + i];
-            }
-            mx += tp.g[j + kR] * rx;
-            my += tp.g[j + kR] * ry;
-        }
-        mx *= inv;
-        my *= inv;
-        float vx = 0.f, vy = 0.f, cxy = 0.f;
-        for (int j = j0; j <= j1; ++j) {
-            float ax = 0.f, ay = 0.f, axy = 0.f;
-            for (int i = i0; i <= i1; ++i) {
-                const float g = tp.g[i + kR];
-                const float ex = sx[ty + kR + j][tx + kR + i] - mx;
-                const float ey = sy[ty + kR + j][tx + kR + i] - my;
-                ax += g * ex * ex;
-                ay += g * ey * ey;
-                axy += g * ex * ey;
-            }
-            vx += tp.g[j + kR] * ax;
-            vy += tp.g[j + kR] * ay;
-            cxy += tp.g[j + kR] * axy;
-        }
-        vx *= inv;
-        vy *= inv;
-        cxy *= inv;
-        const float sgx = sqrtf(vx), sgy = sqrtf(vy);
-        const float l = (2.f * mx * my + C1) / (mx * mx + my * my + C1);
-        const float c = (2.f * sgx * sgy + C2) / (vx + vy + C2);
-        const float s = (cxy + C3) / (sgx * sgy + C3);
-        cw = (double)count;
-        cl = cw * l;
-        cc = cw * c;
-        cs = cw * s;
-    }
-    red[0][threadIdx.x] = cl;
-    red[1][threadIdx.x] = cc;
-    red[2][threadIdx.x] = cs;
-    red[3][threadIdx.x] = cw;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
+    const bool inner = bx >= 0 && by >= 0 && bx + kHaloW <= w && by + kHaloH <= h;   // block-uniform
+    for (int i = threadIdx.x; i < kHaloH * kSsimW; i += 256) {
+        const int hy = i / kSsimW, hx = i % kSsimW;
+        float rx = 0.f, ry = 0.f;
+        int n = 0;
+        if (inner) {
 #pragma unroll
-            for (int m = 0; m < 4; ++m) red[m][threadIdx.x] += red[m][threadIdx.x + o];
+            for (int k = 0; k <= 2 * kR; ++k) {
+                rx += tp.g[k] * sx[hy][hx + k];
+                ry += tp.g[k] * sy[hy][hx + k];
+                n += ss[hy][hx + k];
+            }
+        } else {
+            const int gx = blockIdx.x * kSsimW + hx;
+            for (int k = max(0, kR - gx); k <= min(2 * kR, kR + w - 1 - gx); ++k) {
+                rx += tp.g[k] * sx[hy][hx + k];
+                ry += tp.g[k] * sy[hy][hx + k];
+                n += ss[hy][hx + k];
+            }
         }
-        __syncthreads();
+        rowx[hy][hx] = rx;
+        rowy[hy][hx] = ry;
+        rown[hy][hx] = n;
     }
-    if (threadIdx.x < 4) part[4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) + threadIdx.x] = red[threadIdx.x][0];
+    __syncthreads();
+    SsimSums a = {0.0, 0.0, 0.0, 0.0};
+    if (inner) {
+        if (in0 || in1) {
+            float gsum = 0.f;
+#pragma unroll
+            for (int k = 0; k <= 2 * kR; ++k) gsum += tp.g[k];
+            const float inv = 1.f / (gsum * gsum);
+            float mx[2] = {0.f, 0.f}, my[2] = {0.f, 0.f};
+            int n[2] = {0, 0};
+#pragma unroll
+            for (int j = 0; j <= 2 * kR + 1; ++j) {
+                const float rx = rowx[ty + j][tx], ry = rowy[ty + j][tx];
+                const int rn = rown[ty + j][tx];
+                if (j <= 2 * kR) {
+                    mx[0] += tp.g[j] * rx;
+                    my[0] += tp.g[j] * ry;
+                    n[0] += rn;
+                }
+                if (j >= 1) {
+                    mx[1] += tp.g[j - 1] * rx;
+                    my[1] += tp.g[j - 1] * ry;
+                    n[1] += rn;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                mx[q] *= inv;
+                my[q] *= inv;
+            }
+            float vx[2] = {0.f, 0.f}, vy[2] = {0.f, 0.f}, cxy[2] = {0.f, 0.f};
+#pragma unroll 1
+            for (int j = 0; j <= 2 * kR + 1; ++j) {
+                float ax[2] = {0.f, 0.f}, ay[2] = {0.f, 0.f}, axy[2] = {0.f, 0.f};
+#pragma unroll
+                for (int k = 0; k <= 2 * kR; ++k) {
+                    const float g = tp.g[k], px = sx[ty + j][tx + k], py = sy[ty + j][tx + k];
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const float ex = px - mx[q], ey = py - my[q];
+                        ax[q] += g * ex * ex;
+                        ay[q] += g * ey * ey;
+                        axy[q] += g * ex * ey;
+                    }
+                }
+                if (j <= 2 * kR) {
+                    vx[0] += tp.g[j] * ax[0];
+                    vy[0] += tp.g[j] * ay[0];
+                    cxy[0] += tp.g[j] * axy[0];
+                }
+                if (j >= 1) {
+                    vx[1] += tp.g[j - 1] * ax[1];
+                    vy[1] += tp.g[j - 1] * ay[1];
+                    cxy[1] += tp.g[j - 1] * axy[1];
+                }
+            }
+            if (in0) ssim_terms(mx[0], my[0], vx[0] * inv, vy[0] * inv, cxy[0] * inv, n[0], a);
+            if (in1) ssim_terms(mx[1], my[1], vx[1] * inv, vy[1] * inv, cxy[1] * inv, n[1], a);
+        }
+    } else {
+        for (int q = 0; q < 2; ++q) {
+            if (!(q ? in1 : in0)) continue;
+            // taps inside the image: columns i0..i1, rows j0..j1 of the window
+            const int yq = y + q, tq = ty + q;
+            const int i0 = max(0, kR - x), i1 = min(2 * kR, kR + w - 1 - x);
+            const int j0 = max(0, kR - yq), j1 = min(2 * kR, kR + h - 1 - yq);
+            float gsx = 0.f, gsy = 0.f;
+            for (int i = i0; i <= i1; ++i) gsx += tp.g[i];
+            for (int j = j0; j <= j1; ++j) gsy += tp.g[j];
+            const float inv = 1.f / (gsx * gsy);
+            float mx = 0.f, my = 0.f;
+            int n = 0;
+            for (int j = j0; j <= j1; ++j) {
+                mx += tp.g[j] * rowx[tq + j][tx];
+                my += tp.g[j] * rowy[tq + j][tx];
+                n += rown[tq + j][tx];
+            }
+            mx *= inv;
+            my *= inv;
+            float vx = 0.f, vy = 0.f, cxy = 0.f;
+            for (int j = j0; j <= j1; ++j) {
+                float ax = 0.f, ay = 0.f, axy = 0.f;
+                for (int i = i0; i <= i1; ++i) {
+                    const float g = tp.g[i];
+                    const float ex = sx[tq + j][tx + i] - mx, ey = sy[tq + j][tx + i] - my;
+                    ax += g * ex * ex;
+                    ay += g * ey * ey;
+                    axy += g * ex * ey;
+                }
+                vx += tp.g[j] * ax;
+                vy += tp.g[j] * ay;
+                cxy += tp.g[j] * axy;
+            }
+            ssim_terms(mx, my, vx * inv, vy * inv, cxy * inv, n, a);
+        }
+    }
+    double v[4] = {a.l, a.c, a.s, a.w};
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[m] += __shfl_xor_sync(0xffffffffu, v[m], o);
+        if ((threadIdx.x & 31) == 0) red[m][threadIdx.x >> 5] = v[m];
+    }
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        double t = 0.0;
+        for (int k = 0; k < 8; ++k) t += red[threadIdx.x][k];
+        out[threadIdx.x] = t;
+    }
+}
+
+// The twelve sums of the three scales, one CTA each: CTA 4 j + m adds term m of
+// scale j over that scale's tiles in a fixed order.
+struct ApScales {
+    int64_t at[3], n[3];      // first partial (of 4 terms) and number of tiles per scale
+};
+
+__global__ void __launch_bounds__(256) k_ap_final(const double* __restrict__ part, ApScales sc,
+                                                  double* __restrict__ out) {
+    __shared__ double s[8];
+    const int j = blockIdx.x >> 2, m = blockIdx.x & 3;
+    const double* p = part + 4 * sc.at[j] + m;
+    double acc = 0.0;
+#pragma unroll 8
+    for (int64_t b = threadIdx.x; b < sc.n[j]; b += 256) acc += p[4 * b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int k = 0; k < 8; ++k) t += s[k];
+        out[blockIdx.x] = t;
+    }
 }
 
 bool dev_ptr(const void* p) {
@@ -640,7 +770,7 @@ int ftr_eval_geometry(ftr_ctx* c, const ftr_camera* cam, const float* rendered_d
     // the list sizes stay on the device: CTAs past the sensor points end at once
     k_ev_cp<<<(unsigned)((npx + kCpThreads - 1) / kCpThreads), kCpThreads, 0, st>>>(ptsG, ptsR, tiles, rendered_depth, ev->cnt, d2);
     k_sum<float><<<kSumBlocks, 256, 0, st>>>(d2, npx, ev->part);
-    k_sum_final<<<1, 256, 0, st>>>(ev->part, kSumBlocks, 1, 1, reinterpret_cast<double*>(ev->cnt + 9));
+    k_sum_final<<<1, 256, 0, st>>>(ev->part, kSumBlocks, reinterpret_cast<double*>(ev->cnt + 9));
     c->launches += 6;
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "ftr_eval_geometry: kernels");
     unsigned long long* hc = reinterpret_cast<unsigned long long*>(ev->h_res);
@@ -688,8 +818,8 @@ int ftr_eval_appearance(ftr_ctx* c, int w, int h, const float* rendered_depth, c
         ws[j] = j ? ws[j - 1] / 2 : w;
         hs[j] = j ? hs[j - 1] / 2 : h;
         off[j + 1] = off[j] + (int64_t)ws[j] * hs[j];
-        gx[j] = (unsigned)((ws[j] + kTile - 1) / kTile);
-        gy[j] = (unsigned)((hs[j] + kTile - 1) / kTile);
+        gx[j] = (unsigned)((ws[j] + kSsimW - 1) / kSsimW);
+        gy[j] = (unsigned)((hs[j] + kSsimH - 1) / kSsimH);
         boff[j + 1] = boff[j] + (int64_t)gx[j] * gy[j];
     }
     const double nan = std::numeric_limits<double>::quiet_NaN();
@@ -730,11 +860,16 @@ int ftr_eval_appearance(ftr_ctx* c, int w, int h, const float* rendered_depth, c
         if ((int64_t)gx[j] * gy[j] > 0) {
             k_ap_ssim<<<dim3(gx[j], gy[j]), 256, 0, st>>>(X + off[j], Y + off[j], S + off[j], ws[j], hs[j], tp,
                                                          ev->part + 4 * boff[j]);
-            k_sum_final<<<1, 256, 0, st>>>(ev->part + 4 * boff[j], boff[j + 1] - boff[j], 4, 4,
-                                           ev->part + 4 * boff[3] + 4 * j);
-            c->launches += 2;
+            c->launches++;
         }
     }
+    ApScales sc;
+    for (int j = 0; j < 3; ++j) {
+        sc.at[j] = boff[j];
+        sc.n[j] = boff[j + 1] - boff[j];
+    }
+    k_ap_final<<<12, 256, 0, st>>>(ev->part, sc, ev->part + 4 * boff[3]);
+    c->launches++;
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "ftr_eval_appearance: kernels");
     if ((e = cudaMemcpyAsync(ev->h_res, ev->part + 4 * boff[3], 12 * sizeof(double), cudaMemcpyDeviceToHost, st)) !=
             cudaSuccess ||

@@ -5,7 +5,8 @@ the SSIM tiles, dense and sparse silhouettes, overlapping and far apart.
 Bars: counts, VRE and the Hausdorff distance exact (integers).  Closest-point
 distances: each back-projected coordinate is rounded to float32, so a distance
 moves by at most 2 sqrt(3) 2^-24 z per axis ratio r = max |X| / z of the view;
-with |X| <= 2 z and z <= 4 m that is 2.8e-6 m.
+with |X| <= 2 z and z <= 4 m that is 2.8e-6 m.  WMS3IM and its terms within
+1e-4 (float32 luma and window moments), as in the other appearance tests.
 """
 
 import numpy as np
@@ -66,3 +67,25 @@ def test_geometry_sizes(w, h, kind):
     step = max(1, len(Xg) // 3000)
     ref = np.sqrt(oev.closest_sq(Xg[::step], Xr))
     assert np.max(np.abs(np.sqrt(d[gd > 0])[::step] - ref)) <= 2.8e-6
+
+
+@pytest.mark.parametrize("w,h", [(9, 11), (32, 16), (33, 17), (42, 26), (43, 27), (75, 53), (128, 96), (131, 77)])
+def test_appearance_sizes(w, h):
+    torch = G.require_gpu()
+    from paper_1712_03084_gb300 import ftr
+    rng = np.random.default_rng(w * 31 + h)
+    v, u = np.mgrid[0:h, 0:w]
+    a = (120 + 60 * np.sin(0.2 * u + 0.1 * v)[..., None] + rng.uniform(-30, 30, (h, w, 3))).astype(np.uint8)
+    b = np.clip(a.astype(float) * 0.8 + rng.uniform(-20, 40, (h, w, 3)), 0, 255).astype(np.uint8)
+    rd = np.where((u - w / 2) ** 2 / w ** 2 + (v - h / 2) ** 2 / h ** 2 < 0.3, 2.0, 0.0).astype(np.float32)
+    ctx = ftr.Context((32, 32, 32), (0, 0, 0, 1, 1, 1))
+    got = ftr.ftr_eval_appearance(ctx.h, torch.from_numpy(rd).cuda(), torch.from_numpy(a).cuda(),
+                                  torch.from_numpy(b).cuda())
+    none = ftr.ftr_eval_appearance(ctx.h, torch.zeros((h, w), device="cuda"), torch.from_numpy(a).cuda(),
+                                   torch.from_numpy(b).cuda())
+    ctx.close()
+    ref, L, C, S = oev.wms3im(rd, a, b)
+    assert abs(got["wms3im"] - ref) <= 1e-4
+    for x, y in ((got["l"], L), (got["c"], C), (got["s"], S)):
+        assert np.max(np.abs(np.array(x) - np.array(y))) <= 1e-4
+    assert np.isnan(none["wms3im"])
