@@ -712,6 +712,7 @@ void eval_free(ftr_ctx* c) {
     if (!ev) return;
     if (ev->zkey) cudaFree(ev->zkey);
     if (ev->big) cudaFree(ev->big);
+    if (ev->proj) cudaFree(ev->proj);
     if (ev->col) cudaFree(ev->col);
     if (ev->pts) cudaFree(ev->pts);
     if (ev->d2) cudaFree(ev->d2);

@@ -350,6 +350,8 @@ struct EvalScratch {
     int64_t zkey_cap = 0;
     int* big = nullptr;                   // large triangles for the shared-pixel pass, then their count
     int64_t big_cap = 0;
+    void* proj = nullptr;                 // per vertex: camera coordinates and projection; ray slopes
+    size_t proj_cap = 0;
     int* col = nullptr;                   // 2 x pixels: column distances to the sensor / rendered silhouette
     float4* pts = nullptr;                // 2 x pixels: compacted sensor and rendered points (.w = pixel)
     float* d2 = nullptr;                  // pixels: squared closest-point distance per sensor pixel
