@@ -5,8 +5,8 @@
 // per-vertex weights and UVs (multitexture blend).  No graphics API is used:
 //
 //   k_project  one thread per vertex: its camera coordinates in float64 and
-//              its projection in float32 with an error bound; the ray slopes
-//              of every pixel column and row (float64);
+//              its projection to 1e-7 pixels; the ray slopes of every pixel
+//              column and row (float64);
 //   k_raster   128 triangles per CTA: walk the pixel centres of the screen
 //              bounding box, test coverage with the three edge functions,
 //              intersect the pixel's ray with the triangle's plane and keep
@@ -30,9 +30,8 @@
 // float32 wherever its error bound allows and in float64 only where it does not
 // (an edge function within its bound of zero), and the float64 work left (a
 // depth per covered pixel that is not behind the surface already there) is
-// queued per CTA so that it runs on full warps.  A triangle whose float32
-// projection is useless (error above 1/20 pixel, or not finite) takes the
-// float64 path throughout.
+// queued per CTA so that it runs on full warps.  A triangle projected more
+// than 2^20 pixels away, or not to a number, takes the float64 path throughout.
 // The colours are float32 (they only feed the final rounding to u8).
 #include <cuda_runtime.h>
 #include <math.h>
@@ -136,11 +135,33 @@ __device__ __forceinline__ void tri_pixel(const CamDev& cam, const TriSetup& s, 
     atomicMin(zkey + (int64_t)py * cam.w + (int64_t)px, key);
 }
 
-// Per vertex: uvez = float32 projection (u, v), a bound e on its error in pixels
-// (-1: nearer than kZNear, its triangles are not drawn) and z; xy = camera x
-// and y; vd = the camera coordinates in float64.
+// Per vertex: at = the projection rounded to whole pixels (int bits) and the
+// rest in float32; xyz = camera coordinates in float32 and how to treat the
+// vertex; vd = the camera coordinates in float64.
+//
+// The rest is good to 1e-7 pixels at any image position, so that few coverage
+// decisions are left open: x / z = a + da with a the float32 quotient and da
+// from the exact remainder x - a z (one float64 operation), and every product
+// and sum that follows keeps its float32 rounding error as a second term.
+// (Plain float32 projections, 1e-3 pixels, left one fragment in sixteen open
+// and with it a float64 coverage test in every warp: 97 us instead of 32 for
+// the 1920 x 1080 raster below.)
+constexpr float kVertSkip = -1.f, kVertExact = 0.f, kVertFast = 1.f;
+
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return s;
+}
+
+__device__ __forceinline__ float two_prod(float a, float b, float& err) {
+    const float p = __fmul_rn(a, b);
+    err = __fmaf_rn(a, b, -p);
+    return p;
+}
+
 __global__ void __launch_bounds__(256) k_project(CamDev cam, const float* __restrict__ verts, int64_t nv,
-                                                 float4* __restrict__ uvez, float2* __restrict__ xy,
+                                                 float4* __restrict__ at, float4* __restrict__ xyz,
                                                  double* __restrict__ vd, double* __restrict__ slope) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < nv) {
@@ -150,12 +171,21 @@ __global__ void __launch_bounds__(256) k_project(CamDev cam, const float* __rest
         for (int r = 0; r < 3; ++r) vd[3 * i + r] = xc[r];
         const float x = (float)xc[0], y = (float)xc[1], z = (float)xc[2];
         const float a = x / z, b = y / z;
-        const float ua = cam.Kf[0] * a, ub = cam.Kf[1] * b, va = cam.Kf[4] * b;
-        // four roundings of at most 2^-24 each on every term, and the sums
-        const float e = 5e-7f * (fabsf(ua) + fabsf(ub) + fabsf(cam.Kf[2]) + fabsf(va) + fabsf(cam.Kf[5]));
-        const bool drawn = xc[2] >= kZNear;
-        uvez[i] = make_float4(ua + ub + cam.Kf[2], va + cam.Kf[5], drawn ? e : -1.f, z);
-        xy[i] = make_float2(x, y);
+        const float ar = (float)__fma_rn(-(double)a, xc[2], xc[0]) / z, br = (float)__fma_rn(-(double)b, xc[2], xc[1]) / z;
+        float e1, e2, e3, e4, e5, e6;
+        const float ua = two_prod(cam.Kf[0], a, e1), ub = two_prod(cam.Kf[1], b, e2);
+        const float us = two_sum(two_sum(ua, ub, e3), cam.Kf[2], e4);
+        const float ul = ((e1 + e2) + (e3 + e4)) + (cam.Kf[0] * ar + cam.Kf[1] * br);
+        const float va = two_prod(cam.Kf[4], b, e5), vs = two_sum(va, cam.Kf[5], e6);
+        const float vl = (e5 + e6) + cam.Kf[4] * br;
+        const float ui = rintf(us), vi = rintf(vs);
+        // the second terms are below 2^-23 of the sums they belong to, their own
+        // errors below 2^-45: what counts is the rounding of the rest (at most half a
+        // pixel), 2^-25, so 4e-8 covers it while the sums stay below 2^20
+        const float size = fabsf(ua) + fabsf(ub) + fabsf(cam.Kf[2]) + fabsf(va) + fabsf(cam.Kf[5]);
+        const float how = !(xc[2] >= kZNear) ? kVertSkip : (size < 1048576.f ? kVertFast : kVertExact);
+        at[i] = make_float4(__int_as_float((int)ui), __int_as_float((int)vi), (us - ui) + ul, (vs - vi) + vl);
+        xyz[i] = make_float4(x, y, z, how);
     } else {
         // slope[x] = (x - K02) / K00 (rays without skew), slope[w + y] = (y - K12) / K11
         const int64_t k = i - nv;
@@ -244,10 +274,11 @@ constexpr int kRasterThreads = 128;
 constexpr int kQueue = 2048;        // fragments per CTA that wait for their float64 depth (8 KB)
 
 // Measured on 152,000 triangles of a body-sized mesh: 88 us at 512 x 424 and
-// 213 us at 1920 x 1080 with one float64 thread per triangle and pixel walk.
+// 213 us at 1920 x 1080 with one float64 thread per triangle and pixel walk,
+// 18 and 32 us now.
 __global__ void __launch_bounds__(kRasterThreads) k_raster(
     CamDev cam, const float* __restrict__ verts, const int32_t* __restrict__ tris, int64_t nt, int64_t nv,
-    const float4* __restrict__ uvez, const float2* __restrict__ xy, const double* __restrict__ vd,
+    const float4* __restrict__ at, const float4* __restrict__ xyz, const double* __restrict__ vd,
     const double* __restrict__ slope, unsigned long long* __restrict__ zkey, int* __restrict__ big,
     int* __restrict__ nbig) {
     __shared__ unsigned s_q[kQueue];                 // triangle of the CTA | y - y0 | x - x0 | open coverage
@@ -260,7 +291,7 @@ __global__ void __launch_bounds__(kRasterThreads) k_raster(
     __syncthreads();
     bool any = false;
     int id[3] = {0, 0, 0};
-    float4 P[3];
+    float4 C[3];
     bool draw = t < nt;
     if (draw) {
 #pragma unroll
@@ -269,52 +300,61 @@ __global__ void __launch_bounds__(kRasterThreads) k_raster(
             draw = draw && id[m] >= 0 && id[m] < nv;
         }
     }
-    float e = 0.f;
-    bool wild = false;
+    bool exact = false;
     if (draw) {
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-            P[m] = uvez[id[m]];
-            draw = draw && !(P[m].z < 0.f);          // a NaN bound is not negative: the float64 path decides
-            wild = wild || !(P[m].z < 0.05f) || !isfinite(P[m].x) || !isfinite(P[m].y);
-            e = fmaxf(e, P[m].z);
+            C[m] = xyz[id[m]];
+            draw = draw && C[m].w != kVertSkip;
+            exact = exact || C[m].w != kVertFast;
         }
     }
-    if (draw && wild) {
+    if (draw && exact) {
         raster_exact(cam, verts, tris, t, nv, zkey, big, nbig);
         draw = false;
     }
     if (draw) {
-        // pixel centres the box can hold, widened by the projection's error
-        const float xmin = fminf(fminf(P[0].x, P[1].x), P[2].x) - 1.5f * e, xmax = fmaxf(fmaxf(P[0].x, P[1].x), P[2].x) + 1.5f * e;
-        const float ymin = fminf(fminf(P[0].y, P[1].y), P[2].y) - 1.5f * e, ymax = fmaxf(fmaxf(P[0].y, P[1].y), P[2].y) + 1.5f * e;
-        const int x0 = (int)fmaxf(ceilf(xmin), 0.f), x1 = (int)fminf(floorf(xmax), (float)(cam.w - 1));
-        const int y0 = (int)fmaxf(ceilf(ymin), 0.f), y1 = (int)fminf(floorf(ymax), (float)(cam.h - 1));
-        if (xmax >= 0.f && ymax >= 0.f && x1 >= x0 && y1 >= y0) {
+        // positions relative to the whole pixel of vertex 0
+        float X[3], Y[3];
+        const float4 P0 = at[id[0]], P1 = at[id[1]], P2 = at[id[2]];
+        const int ox = __float_as_int(P0.x), oy = __float_as_int(P0.y);
+        X[0] = P0.z;
+        Y[0] = P0.w;
+        X[1] = (float)(__float_as_int(P1.x) - ox) + P1.z;
+        Y[1] = (float)(__float_as_int(P1.y) - oy) + P1.w;
+        X[2] = (float)(__float_as_int(P2.x) - ox) + P2.z;
+        Y[2] = (float)(__float_as_int(P2.y) - oy) + P2.w;
+        const float xlo = fminf(fminf(X[0], X[1]), X[2]), xhi = fmaxf(fmaxf(X[0], X[1]), X[2]);
+        const float ylo = fminf(fminf(Y[0], Y[1]), Y[2]), yhi = fmaxf(fmaxf(Y[0], Y[1]), Y[2]);
+        const float D = fmaxf(fmaxf(xhi, yhi), -fminf(xlo, ylo)) + 1.f;      // > every coordinate used below
+        const float e = 1e-7f * D;          // > the error of X, Y: 4e-8 of the vertex + 2^-24 D of the sum
+        // pixel centres the box can hold, widened by that error
+        const int x0 = max(ox + (int)ceilf(xlo - 2.f * e), 0), x1 = min(ox + (int)floorf(xhi + 2.f * e), cam.w - 1);
+        const int y0 = max(oy + (int)ceilf(ylo - 2.f * e), 0), y1 = min(oy + (int)floorf(yhi + 2.f * e), cam.h - 1);
+        if (x1 >= x0 && y1 >= y0) {
             if ((int64_t)(x1 - x0 + 1) * (y1 - y0 + 1) > kBigPx) {
                 big[atomicAdd(nbig, 1)] = (int)t;
             } else {
-                const float X1 = P[1].x - P[0].x, Y1 = P[1].y - P[0].y, X2 = P[2].x - P[0].x, Y2 = P[2].y - P[0].y;
-                // |edge function error| <= tol: its factors are below D + 1 and
-                // carry errors of at most 2 e each; the products round once more
-                const float D = fmaxf(xmax - xmin, ymax - ymin) + 1.f;
-                const float tol = 8.f * e * (D + e) + 1e-6f * D * D;
+                const float X1 = X[1] - X[0], Y1 = Y[1] - Y[0], X2 = X[2] - X[0], Y2 = Y[2] - Y[0];
+                // |edge function error| <= tol: its factors are at most 2 D and off
+                // by at most 7 e after their differences (44 e D for the two
+                // products), and products and difference round (10 e D)
+                const float tol = 64.f * e * D;
                 // nothing nearer than the nearest vertex is hit, unless the plane
                 // is seen edge-on or the triangle is a sliver
                 float zlow = -1.f;
                 {
-                    const float2 c0 = xy[id[0]], c1 = xy[id[1]], c2 = xy[id[2]];
-                    const float ax = c1.x - c0.x, ay = c1.y - c0.y, az = P[1].w - P[0].w;
-                    const float bx = c2.x - c0.x, by = c2.y - c0.y, bz = P[2].w - P[0].w;
+                    const float ax = C[1].x - C[0].x, ay = C[1].y - C[0].y, az = C[1].z - C[0].z;
+                    const float bx = C[2].x - C[0].x, by = C[2].y - C[0].y, bz = C[2].z - C[0].z;
                     const float nx = ay * bz - az * by, ny = az * bx - ax * bz, nz = ax * by - ay * bx;
                     const float nn = nx * nx + ny * ny + nz * nz;
                     const float l2 = fmaxf(ax * ax + ay * ay + az * az, bx * bx + by * by + bz * bz);
-                    const float r2 = fmaxf(fmaxf(c0.x * c0.x + c0.y * c0.y + P[0].w * P[0].w,
-                                                 c1.x * c1.x + c1.y * c1.y + P[1].w * P[1].w),
-                                           c2.x * c2.x + c2.y * c2.y + P[2].w * P[2].w);
-                    const float d = nx * c0.x + ny * c0.y + nz * P[0].w;
+                    float r2 = 0.f;
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) r2 = fmaxf(r2, C[m].x * C[m].x + C[m].y * C[m].y + C[m].z * C[m].z);
+                    const float d = nx * C[0].x + ny * C[0].y + nz * C[0].z;
                     if (nn >= 1e-4f * l2 * l2 && l2 >= 1e-6f * r2 && d * d >= 0.01f * nn * r2)
-                        zlow = fminf(fminf(P[0].w, P[1].w), P[2].w) * (1.f - 1e-5f);
+                        zlow = fminf(fminf(C[0].z, C[1].z), C[2].z) * (1.f - 1e-5f);
                 }
                 s_zlow[tid] = zlow;
                 s_x0[tid] = x0;
@@ -322,9 +362,9 @@ __global__ void __launch_bounds__(kRasterThreads) k_raster(
 #pragma unroll
                 for (int m = 0; m < 3; ++m) s_id[m][tid] = id[m];
                 for (int py = y0; py <= y1; ++py) {
-                    const float qy = (float)py - P[0].y;
+                    const float qy = (float)(py - oy) - Y[0];
                     for (int px = x0; px <= x1; ++px) {
-                        const float qx = (float)px - P[0].x;
+                        const float qx = (float)(px - ox) - X[0];
                         const float f0 = X1 * qy - Y1 * qx;
                         const float f1 = (X2 - X1) * (qy - Y1) - (Y2 - Y1) * (qx - X1);
                         const float f2 = Y2 * (qx - X2) - X2 * (qy - Y2);
@@ -335,9 +375,9 @@ __global__ void __launch_bounds__(kRasterThreads) k_raster(
                             if (cur != 0xffffffffu && zlow > __uint_as_float(cur)) continue;
                         }
                         const unsigned open = !(lo > tol || hi < -tol);
-                        const int at = atomicAdd(&s_n, 1);
-                        if (at < kQueue) {
-                            s_q[at] = ((unsigned)tid << 21) | ((unsigned)(py - y0) << 11) | ((unsigned)(px - x0) << 1) | open;
+                        const int slot = atomicAdd(&s_n, 1);
+                        if (slot < kQueue) {
+                            s_q[slot] = ((unsigned)tid << 21) | ((unsigned)(py - y0) << 11) | ((unsigned)(px - x0) << 1) | open;
                             any = true;
                         } else if (!open || covered_exact(cam, vd, id[0], id[1], id[2], px, py)) {
                             double n[4];
@@ -578,9 +618,9 @@ int ftr_render(ftr_ctx* c, const ftr_render_src* src, const ftr_camera* cam, flo
         int* nbig = ev->big + src->n_tris;
         if ((e = cudaMemsetAsync(nbig, 0, sizeof(int), c->stream)) != cudaSuccess)
             return cuda_fail(c, e, "ftr_render: clear");
-        // scratch: vd (3 doubles per vertex), slopes (w + h doubles), uvez, xy
+        // scratch: at, xyz, vd (3 doubles per vertex), slopes (w + h doubles)
         const int64_t nv = src->n_vertices, nslope = (int64_t)cam->w + cam->h;
-        const size_t need = (size_t)nv * (24 + 16 + 8) + (size_t)nslope * 8 + 16;
+        const size_t need = (size_t)nv * (16 + 16 + 24) + (size_t)nslope * 8;
         if (need > ev->proj_cap) {
             cudaStreamSynchronize(c->stream);
             if (ev->proj) cudaFree(ev->proj);
@@ -589,14 +629,15 @@ int ftr_render(ftr_ctx* c, const ftr_render_src* src, const ftr_camera* cam, flo
             if ((e = cudaMalloc(&ev->proj, need)) != cudaSuccess) return cuda_fail(c, e, "ftr_render: vertices");
             ev->proj_cap = need;
         }
-        float4* uvez = static_cast<float4*>(ev->proj);
-        double* vd = reinterpret_cast<double*>(uvez + nv);
+        float4* at = static_cast<float4*>(ev->proj);
+        float4* xyz = at + nv;
+        double* vd = reinterpret_cast<double*>(xyz + nv);
         double* slope = vd + 3 * nv;
-        float2* xy = reinterpret_cast<float2*>(slope + nslope);
-        k_project<<<(unsigned)((nv + nslope + 255) / 256), 256, 0, c->stream>>>(cd, src->vertices, nv, uvez, xy, vd, slope);
+        k_project<<<(unsigned)((nv + nslope + 255) / 256), 256, 0, c->stream>>>(cd, src->vertices, nv, at, xyz, vd,
+                                                                                          slope);
         c->launches++;
         k_raster<<<(unsigned)((src->n_tris + kRasterThreads - 1) / kRasterThreads), kRasterThreads, 0, c->stream>>>(
-            cd, src->vertices, src->tris, src->n_tris, nv, uvez, xy, vd, slope, ev->zkey, ev->big, nbig);
+            cd, src->vertices, src->tris, src->n_tris, nv, at, xyz, vd, slope, ev->zkey, ev->big, nbig);
         k_raster_big<<<2 * 152, 256, 0, c->stream>>>(cd, src->vertices, src->tris, src->n_vertices, ev->zkey, ev->big,
                                                      nbig);
         c->launches += 2;
