@@ -16,8 +16,8 @@
 //                are contiguous; the order of the tiles does not matter) and
 //                records the box of the tile's rendered points;
 //   k_ev_cp      per sensor point the squared distance to the closest rendered
-//                point, float32: only tiles whose box can hold a closer point
-//                than the best so far are searched;
+//                point, float32: only 8 x 8 pixel blocks whose box can hold a
+//                closer point than the best so far are searched;
 //   k_sum / k_sum_final  the float64 sum of those distances in pixel order,
 //                fixed blocks and a fixed tree (deterministic).
 //
@@ -52,8 +52,9 @@ constexpr int kSumBlocks = 256;
 constexpr int kCpThreads = 64;      // closest points: small CTAs, so that one body's points reach every SM
 // counters of one geometry evaluation: |S_r|, |S_g|, |xor|, |or|, the two
 // squared Hausdorff maxima, the list sizes I and J, the tiles with rendered
-// points, and the float64 sum of the closest-point distances
-constexpr int kCounters = 10;
+// points, the float64 sum of the closest-point distances, and the entries of
+// the sensor list (whole warps)
+constexpr int kCounters = 11;
 // Sec. III-E3: exponents of the three scales (luminance, contrast, structure)
 constexpr double kAlpha[3] = {0.0, 0.0, 0.1333};
 constexpr double kBeta[3] = {0.0448, 0.3001, 0.1333};
@@ -80,7 +81,7 @@ __device__ __forceinline__ int col_distance(unsigned m, int i, int base, int pre
 // segments): the segment's rows are loaded at once and kept as one bit per row
 // and set, so the column is read once and its distances need no second sweep.
 // (A thread per column walking all rows twice ran 4 CTAs for a 512-pixel row
-// and took 380 us at 512 x 424, all of it dependent loads.)  Shared memory:
+// and took 380 us at 512 x 424, all of it dependent loads; now 12.)  Shared memory:
 // masks [set][segment][column], 256 bytes per segment.
 __global__ void __launch_bounds__(512) k_ev_cols(const float* __restrict__ rd, const float* __restrict__ gd, int w,
                                                  int h, int nseg, int* __restrict__ colG, int* __restrict__ colR,
@@ -95,11 +96,20 @@ __global__ void __launch_bounds__(512) k_ev_cols(const float* __restrict__ rd, c
         unsigned mg = 0, mr = 0;
         if (x < w) {
             const int64_t at = (int64_t)s * 32 * w + x;
-#pragma unroll 16
-            for (int i = 0; i < 32; ++i) {
-                if (s * 32 + i >= h) break;
-                mg |= (unsigned)(gd[at + (int64_t)i * w] > 0.f) << i;
-                mr |= (unsigned)(rd[at + (int64_t)i * w] > 0.f) << i;
+            const int rows = h - s * 32;            // all loads of 16 rows in flight at once
+#pragma unroll
+            for (int i0 = 0; i0 < 32; i0 += 16) {
+                float vg[16], vr[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    vg[i] = i0 + i < rows ? gd[at + (int64_t)(i0 + i) * w] : 0.f;
+                    vr[i] = i0 + i < rows ? rd[at + (int64_t)(i0 + i) * w] : 0.f;
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    mg |= (unsigned)(vg[i] > 0.f) << (i0 + i);
+                    mr |= (unsigned)(vr[i] > 0.f) << (i0 + i);
+                }
             }
         }
         s_g[s * 32 + lane] = mg;
@@ -123,6 +133,7 @@ __global__ void __launch_bounds__(512) k_ev_cols(const float* __restrict__ rd, c
                 if (s_r[t * 32 + lane]) qr = t * 32 + __ffs(s_r[t * 32 + lane]) - 1;
             const unsigned mg = s_g[s * 32 + lane], mr = s_r[s * 32 + lane];
             const int rows = min(32, h - s * 32);
+#pragma unroll 4
             for (int i = 0; i < rows; ++i) {
                 const int64_t at = (int64_t)(s * 32 + i) * w + x;
                 colG[at] = col_distance(mg, i, s * 32, pg, qg);
@@ -191,28 +202,43 @@ struct Intr {
     double K[9];
 };
 
-// Rendered points of one 16 x 16 pixel tile: their bounding box and their
-// place in the list.
-struct PointTile {
+// Rendered points of one 8 x 8 pixel block: their bounding box and their place
+// in the list.  A 16 x 16 pixel tile holds four of them and the box of all.
+struct PointBox {
     float lo[3];
     int start;
     float hi[3];
     int count;
 };
+struct PointTile {
+    PointBox all, part[4];
+};
 
+// A warp takes 8 x 4 pixels and a pair of warps one 8 x 8 block, so that a
+// block's points are near one another.  The sensor points of a warp that has
+// any keep a whole warp's entries (the rest repeat one of them, tag -1): a warp
+// of k_ev_cp then never holds the points of two distant patches.  tile_of: per
+// image tile its record, -1 without rendered points.
 __global__ void __launch_bounds__(256) k_ev_points(const float* __restrict__ rd, const float* __restrict__ gd,
                                                    int w, int h, Intr in, float4* __restrict__ ptsG,
                                                    float4* __restrict__ ptsR, PointTile* __restrict__ tiles,
-                                                   float* __restrict__ d2, unsigned long long* __restrict__ cnt) {
+                                                   int* __restrict__ tile_of, float* __restrict__ d2,
+                                                   unsigned long long* __restrict__ cnt) {
     __shared__ int s_ng[8], s_nr[8], s_base[3];
-    __shared__ float s_box[6][8];
-    const int x = blockIdx.x * kTile + (threadIdx.x & (kTile - 1)), y = blockIdx.y * kTile + threadIdx.x / kTile;
+    __shared__ float s_box[8][6];
+    const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int x = blockIdx.x * kTile + ((wid >> 1) & 1) * 8 + (lane & 7);
+    const int y = blockIdx.y * kTile + (wid >> 2) * 8 + (wid & 1) * 4 + (lane >> 3);
     const bool live = x < w && y < h;
     const int64_t p = (int64_t)y * w + x;
     const float zg = live ? gd[p] : 0.f, zr = live ? rd[p] : 0.f;
     const bool g = zg > 0.f, r = zr > 0.f;
+    int* own = tile_of + (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
     if (live) d2[p] = g ? __uint_as_float(0x7f800000u) : 0.f;
-    if (!__syncthreads_or(g || r)) return;
+    if (!__syncthreads_or(g || r)) {
+        if (threadIdx.x == 0) *own = -1;
+        return;
+    }
     double dx = 0.0, dy = 0.0;
     if (g || r) {
         const double py = (double)y, px = (double)x;
@@ -232,7 +258,6 @@ __global__ void __launch_bounds__(256) k_ev_points(const float* __restrict__ rd,
         b[4] = fmaxf(-inf, P.y);
         b[5] = fmaxf(-inf, P.z);
     }
-    const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const unsigned bg = __ballot_sync(0xffffffffu, g), br = __ballot_sync(0xffffffffu, r);
 #pragma unroll
@@ -247,112 +272,184 @@ __global__ void __launch_bounds__(256) k_ev_points(const float* __restrict__ rd,
         s_ng[wid] = __popc(bg);
         s_nr[wid] = __popc(br);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) s_box[c][wid] = b[c];
+        for (int c = 0; c < 6; ++c) s_box[wid][c] = b[c];
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        int ng = 0, nr = 0;
+        int ng = 0, nr = 0, slots = 0;
         for (int k = 0; k < 8; ++k) {
             ng += s_ng[k];
             nr += s_nr[k];
+            slots += s_ng[k] ? 32 : 0;
         }
-        s_base[0] = ng ? (int)atomicAdd(cnt + 6, (unsigned long long)ng) : 0;
+        if (ng) atomicAdd(cnt + 6, (unsigned long long)ng);
+        s_base[0] = ng ? (int)atomicAdd(cnt + 10, (unsigned long long)slots) : 0;
         s_base[1] = nr ? (int)atomicAdd(cnt + 7, (unsigned long long)nr) : 0;
-        if (nr) {
-            PointTile t;
-            t.start = s_base[1];
-            t.count = nr;
-            for (int c = 0; c < 3; ++c) {
-                float lo = s_box[c][0], hi = s_box[3 + c][0];
-                for (int k = 1; k < 8; ++k) {
-                    lo = fminf(lo, s_box[c][k]);
-                    hi = fmaxf(hi, s_box[3 + c][k]);
-                }
-                t.lo[c] = lo;
-                t.hi[c] = hi;
-            }
-            tiles[atomicAdd(cnt + 8, 1ull)] = t;
-        }
+        s_base[2] = nr ? (int)atomicAdd(cnt + 8, 1ull) : -1;
+        *own = s_base[2];
     }
     __syncthreads();
+    if (s_base[2] >= 0 && threadIdx.x < 5) {      // the tile's record: thread 4 the whole, 0..3 the blocks
+        const int k0 = threadIdx.x == 4 ? 0 : 2 * threadIdx.x, k1 = threadIdx.x == 4 ? 8 : k0 + 2;
+        PointBox t;
+        t.start = s_base[1];
+        for (int k = 0; k < k0; ++k) t.start += s_nr[k];
+        t.count = 0;
+        for (int c = 0; c < 3; ++c) {
+            t.lo[c] = inf;
+            t.hi[c] = -inf;
+        }
+        for (int k = k0; k < k1; ++k) {
+            t.count += s_nr[k];
+            for (int c = 0; c < 3; ++c) {
+                t.lo[c] = fminf(t.lo[c], s_box[k][c]);
+                t.hi[c] = fmaxf(t.hi[c], s_box[k][3 + c]);
+            }
+        }
+        if (threadIdx.x == 4)
+            tiles[s_base[2]].all = t;
+        else
+            tiles[s_base[2]].part[threadIdx.x] = t;
+    }
     int og = s_base[0], orr = s_base[1];
     for (unsigned k = 0; k < wid; ++k) {
-        og += s_ng[k];
+        og += s_ng[k] ? 32 : 0;
         orr += s_nr[k];
     }
-    if (g) {
-        const double z = zg;
-        ptsG[og + __popc(bg & lt)] = make_float4((float)(z * dx), (float)(z * dy), zg, __int_as_float((int)p));
+    if (bg) {
+        float4 Q = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (g) {
+            const double z = zg;
+            Q = make_float4((float)(z * dx), (float)(z * dy), zg, 0.f);
+        }
+        const int first = __ffs(bg) - 1;
+        const float fx = __shfl_sync(0xffffffffu, Q.x, first), fy = __shfl_sync(0xffffffffu, Q.y, first),
+                    fz = __shfl_sync(0xffffffffu, Q.z, first);
+        ptsG[og + lane] = g ? make_float4(Q.x, Q.y, Q.z, __int_as_float((int)p))
+                            : make_float4(fx, fy, fz, __int_as_float(-1));
     }
     if (r) ptsR[orr + __popc(br & lt)] = P;
 }
 
+// Squared distance from a box (or a point, lo = hi) to a box, not above that of
+// any two points in them (differences and sums of float32 are monotonic; the
+// factor covers the order the sum is rounded in).
+__device__ __forceinline__ float box_gap2(const float lo[3], const float hi[3], const PointBox& b) {
+    float s = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const float d = fmaxf(fmaxf(b.lo[c] - hi[c], lo[c] - b.hi[c]), 0.f);
+        s += d * d;
+    }
+    return s * 0.9999f;
+}
+
 // Per sensor point the squared distance to the closest rendered point: the
-// minimum over all of them, found by searching only the tiles whose box can
-// hold a closer point.  `bound` starts from the rendered point of the same
-// pixel (the two differ along the ray only), else from the farthest corner of
-// the nearest tile, both widened by more than the float32 error of a
-// distance; a box's distance is shrunk by the same, so no tile that holds the
-// minimum is skipped and the result is that of the full search.  A warp holds
-// points of neighbouring pixels and searches a tile together when any of its
-// lanes wants it.  The full search (every pair, 28,000 x 28,000 points at
-// 512 x 424) took 107 us; this does about 1/30 of the pairs.
+// minimum over all of them, found by searching only the blocks whose box can
+// hold a closer point, so the result is that of the full search.  A warp holds
+// the points of one 8 x 4 pixel patch and searches together: its own tile
+// first, which leaves most lanes with the distance to the surface (where that
+// is empty, the tile whose farthest corner is nearest); then its lanes test 32
+// tile boxes at a time against the box of the warp's points, and the blocks of
+// those that remain per lane.  28,000 x 28,000 points of a 512 x 424 view: 107
+// us for all pairs, 94 with 16 x 16 tiles tested lane by lane in list order, 55
+// now; the last warps, whose patch lies off the rendered silhouette, decide it.
 __global__ void __launch_bounds__(kCpThreads) k_ev_cp(const float4* __restrict__ G, const float4* __restrict__ R,
-                                               const PointTile* __restrict__ tiles, const float* __restrict__ rd,
-                                               const unsigned long long* __restrict__ cnt, float* __restrict__ d2) {
-    __shared__ PointTile s[kCpThreads];
-    const int64_t I = (int64_t)cnt[6];
+                                                      const PointTile* __restrict__ tiles,
+                                                      const int* __restrict__ tile_of, int w,
+                                                      const unsigned long long* __restrict__ cnt,
+                                                      float* __restrict__ d2) {
     const int nt = (int)cnt[8];
     const int64_t gi = (int64_t)blockIdx.x * kCpThreads + threadIdx.x;
-    if ((int64_t)blockIdx.x * kCpThreads >= I) return;
-    const bool live = gi < I;
+    if (gi >= (int64_t)cnt[10]) return;                    // whole warps
+    const unsigned lane = threadIdx.x & 31;
     const float inf = __uint_as_float(0x7f800000u);
-    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 q = G[gi];
+    const int tag = __float_as_int(q.w);                   // pixel, -1: a repeated point
     float best = inf, bound = inf;
-    if (live) {
-        q = G[gi];
-        const float zr = rd[__float_as_int(q.w)];
-        if (zr > 0.f) {
-            const float ratio = zr / q.z;
-            const float d = sqrtf(q.x * q.x + q.y * q.y + q.z * q.z) * (fabsf(1.f - ratio) + 2e-6f * (1.f + ratio));
-            bound = d * d * 1.0001f;
-            if (!(bound >= 0.f)) bound = inf;
+    auto search = [&](const PointBox& b) {
+        const float4* pr = R + b.start;
+#pragma unroll 8
+        for (int k = 0; k < b.count; ++k) {
+            const float4 c = __ldg(pr + k);
+            const float ex = q.x - c.x, ey = q.y - c.y, ez = q.z - c.z;
+            best = fminf(best, ex * ex + ey * ey + ez * ez);
+        }
+    };
+    const float ql[3] = {q.x, q.y, q.z};
+    auto visit = [&](const PointTile& t) {                 // warp-uniform
+        for (int s = 0; s < 4; ++s) {
+            const bool want = !(box_gap2(ql, ql, t.part[s]) > fminf(best, bound));
+            if (t.part[s].count > 0 && __any_sync(0xffffffffu, want)) search(t.part[s]);
+        }
+    };
+    // the tile of the warp's points
+    const int p0 = __reduce_max_sync(0xffffffffu, tag);
+    const int own = tile_of[(int64_t)(p0 / w / kTile) * ((w + kTile - 1) / kTile) + (p0 % w) / kTile];
+    if (own >= 0) visit(tiles[own]);
+    float lo[3], hi[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) lo[c] = hi[c] = ql[c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            lo[c] = fminf(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
+            hi[c] = fmaxf(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
         }
     }
-    const bool far = __syncthreads_or(live && bound == inf);
-    for (int pass = far ? 0 : 1; pass < 2; ++pass) {
-        for (int tb = 0; tb < nt; tb += kCpThreads) {
-            __syncthreads();
-            if (tb + (int)threadIdx.x < nt) s[threadIdx.x] = tiles[tb + threadIdx.x];
-            __syncthreads();
-            const int n = min(kCpThreads, nt - tb);
-            for (int j = 0; j < n; ++j) {
-                const PointTile& t = s[j];
-                const float ax = t.lo[0] - q.x, ay = t.lo[1] - q.y, az = t.lo[2] - q.z;
-                const float bx = q.x - t.hi[0], by = q.y - t.hi[1], bz = q.z - t.hi[2];
-                if (pass == 0) {
-                    const float fx = fmaxf(fabsf(ax), fabsf(bx)), fy = fmaxf(fabsf(ay), fabsf(by)),
-                                fz = fmaxf(fabsf(az), fabsf(bz));
-                    bound = fminf(bound, (fx * fx + fy * fy + fz * fz) * 1.0001f);
-                    continue;
-                }
-                const float cx = fmaxf(fmaxf(ax, bx), 0.f), cy = fmaxf(fmaxf(ay, by), 0.f),
-                            cz = fmaxf(fmaxf(az, bz), 0.f);
-                const float lb = (cx * cx + cy * cy + cz * cz) * 0.9999f;
-                const bool want = live && !(lb > fminf(best, bound));
-                if (!__any_sync(0xffffffffu, want)) continue;
-                const float4* pr = R + t.start;
-                const int m = t.count;
-#pragma unroll 8
-                for (int k = 0; k < m; ++k) {
-                    const float4 c = __ldg(pr + k);
-                    const float ex = q.x - c.x, ey = q.y - c.y, ez = q.z - c.z;
-                    best = fminf(best, ex * ex + ey * ey + ez * ez);
-                }
+    float reach;                                           // no lane looks farther
+    auto update_reach = [&]() {
+        reach = fminf(best, bound);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) reach = fmaxf(reach, __shfl_xor_sync(0xffffffffu, reach, o));
+    };
+    update_reach();
+    if (reach == inf) {
+        float far = inf;                                   // farthest corners of the two boxes
+        int at = -1;
+        for (int j = lane; j < nt; j += 32) {
+            const PointBox b = tiles[j].all;
+            float s = 0.f;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float d = fmaxf(fabsf(b.hi[c] - lo[c]), fabsf(hi[c] - b.lo[c]));
+                s += d * d;
+            }
+            if (s * 1.0001f < far) {
+                far = s * 1.0001f;
+                at = j;
             }
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float of = __shfl_xor_sync(0xffffffffu, far, o);
+            const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+            if (of < far || (of == far && oa > at)) {      // the same choice in every lane
+                far = of;
+                at = oa;
+            }
+        }
+        bound = far;
+        if (at >= 0) visit(tiles[at]);
+        update_reach();
     }
-    if (live) d2[__float_as_int(q.w)] = best;
+    for (int jb = 0; jb < nt; jb += 32) {
+        const int j = jb + (int)lane;
+        bool want = false;
+        if (j < nt && j != own) {
+            const PointBox b = tiles[j].all;
+            want = !(box_gap2(lo, hi, b) > reach);
+        }
+        unsigned m = __ballot_sync(0xffffffffu, want);
+        while (m) {
+            const int k = jb + __ffs(m) - 1;
+            m &= m - 1;
+            visit(tiles[k]);
+        }
+        update_reach();
+    }
+    if (tag >= 0) d2[tag] = best;
 }
 
 // float64 sums of n values in a fixed order: block b takes the indices
@@ -663,22 +760,22 @@ cudaError_t grow_pixels(ftr_ctx* c, EvalScratch* ev, int64_t npx) {
     ev->pix_cap = 0;
     cudaError_t e;
     if ((e = cudaMalloc((void**)&ev->col, (size_t)npx * 2 * sizeof(int))) != cudaSuccess) return e;
-    if ((e = cudaMalloc((void**)&ev->pts, (size_t)npx * 2 * sizeof(float4))) != cudaSuccess) return e;
+    if ((e = cudaMalloc((void**)&ev->pts, (size_t)npx * sizeof(float4))) != cudaSuccess) return e;
     if ((e = cudaMalloc((void**)&ev->d2, (size_t)npx * sizeof(float))) != cudaSuccess) return e;
     ev->pix_cap = npx;
     return cudaSuccess;
 }
 
-// The tile records of a w x h image (its tile count is not bounded by the
-// pixels of another shape).
+// The sensor points (whole warps of every tile), tile records and tile map of a
+// w x h image (its tile count is not bounded by the pixels of another shape).
 cudaError_t grow_tiles(ftr_ctx* c, EvalScratch* ev, int64_t n) {
     if (ev->tiles && ev->tiles_cap >= n) return cudaSuccess;
     cudaStreamSynchronize(c->stream);
-    PointTile* t = nullptr;
+    void* t = nullptr;
     if (ev->tiles) cudaFree(ev->tiles);
     ev->tiles = nullptr;
     ev->tiles_cap = 0;
-    cudaError_t e = cudaMalloc((void**)&t, (size_t)n * sizeof(PointTile));
+    cudaError_t e = cudaMalloc(&t, (size_t)n * (256 * sizeof(float4) + sizeof(PointTile) + sizeof(int)));
     if (e == cudaSuccess) {
         ev->tiles = t;
         ev->tiles_cap = n;
@@ -748,12 +845,13 @@ int ftr_eval_geometry(ftr_ctx* c, const ftr_camera* cam, const float* rendered_d
     float* d2 = cp_d2_out ? cp_d2_out : ev->d2;
     int* colG = ev->col;
     int* colR = ev->col + npx;
-    float4* ptsG = ev->pts;
-    float4* ptsR = ev->pts + npx;
+    float4* ptsR = ev->pts;
     const int tx = (w + kTile - 1) / kTile, ty = (h + kTile - 1) / kTile;
     if ((e = grow_tiles(c, ev, (int64_t)tx * ty)) != cudaSuccess)
         return cuda_fail(c, e, "ftr_eval_geometry: scratch");
-    PointTile* tiles = static_cast<PointTile*>(ev->tiles);
+    float4* ptsG = static_cast<float4*>(ev->tiles);
+    PointTile* tiles = reinterpret_cast<PointTile*>(ptsG + 256 * (int64_t)tx * ty);
+    int* tile_of = reinterpret_cast<int*>(tiles + (int64_t)tx * ty);
     if ((e = cudaMemsetAsync(ev->cnt, 0, kCounters * sizeof(unsigned long long), st)) != cudaSuccess)
         return cuda_fail(c, e, "ftr_eval_geometry");
     const int nseg = (h + 31) / 32;
@@ -767,9 +865,10 @@ int ftr_eval_geometry(ftr_ctx* c, const ftr_camera* cam, const float* rendered_d
     Intr in;
     for (int j = 0; j < 9; ++j) in.K[j] = cam->K[j];
     k_ev_points<<<dim3((unsigned)tx, (unsigned)ty), 256, 0, st>>>(rendered_depth, sensor_depth, w, h, in, ptsG, ptsR,
-                                                                 tiles, d2, ev->cnt);
+                                                                 tiles, tile_of, d2, ev->cnt);
     // the list sizes stay on the device: CTAs past the sensor points end at once
-    k_ev_cp<<<(unsigned)((npx + kCpThreads - 1) / kCpThreads), kCpThreads, 0, st>>>(ptsG, ptsR, tiles, rendered_depth, ev->cnt, d2);
+    k_ev_cp<<<(unsigned)((int64_t)tx * ty * (256 / kCpThreads)), kCpThreads, 0, st>>>(ptsG, ptsR, tiles, tile_of, w,
+                                                                                          ev->cnt, d2);
     k_sum<float><<<kSumBlocks, 256, 0, st>>>(d2, npx, ev->part);
     k_sum_final<<<1, 256, 0, st>>>(ev->part, kSumBlocks, reinterpret_cast<double*>(ev->cnt + 9));
     c->launches += 6;

@@ -353,10 +353,10 @@ struct EvalScratch {
     void* proj = nullptr;                 // per vertex: camera coordinates and projection; ray slopes
     size_t proj_cap = 0;
     int* col = nullptr;                   // 2 x pixels: column distances to the sensor / rendered silhouette
-    float4* pts = nullptr;                // 2 x pixels: compacted sensor and rendered points (.w = pixel)
+    float4* pts = nullptr;                // pixels: compacted rendered points (.w = pixel)
     float* d2 = nullptr;                  // pixels: squared closest-point distance per sensor pixel
     int64_t pix_cap = 0;
-    void* tiles = nullptr;                // per 16 x 16 pixel tile: box and place of its rendered points
+    void* tiles = nullptr;                // per 16 x 16 pixel tile: sensor points, boxes of its rendered points
     int64_t tiles_cap = 0;
     unsigned long long* cnt = nullptr;    // counters (see evaluate.cu)
     double* part = nullptr;               // per-block partial sums
