@@ -375,7 +375,7 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
     ALLOC(c->d_brick_cursor, c->n_bricks);
     ALLOC(c->d_brick_slot, c->n_bricks);
     ALLOC(c->d_active, c->n_bricks);
-    ALLOC(c->d_meta, 8);
+    ALLOC(c->d_meta, kMetaInts);
     ALLOC(c->d_kerr, 1);
     ALLOC(c->d_tile, (c->n_bricks + kBrickScanTile - 1) / kBrickScanTile + 1);
     ALLOC(c->d_unit_off, c->n_bricks + 1);
@@ -445,7 +445,7 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
     cudaMemsetAsync(c->d_brick_slot, 0xff, sizeof(int) * c->n_bricks, c->stream);
     {
         // no brick touched yet: an empty live z-slab (max brick z = -1)
-        const int meta0[8] = {0, 0, 0, -1, 0, 0, 0, 0};
+        const int meta0[kMetaInts] = {0, 0, 0, -1};   // and no live rows
         cudaMemcpyAsync(c->d_meta, meta0, sizeof(meta0), cudaMemcpyHostToDevice, c->stream);
     }
     cudaMemsetAsync(c->d_wild, 0, sizeof(int), c->stream);
@@ -1482,7 +1482,9 @@ int ftr_autotune(ftr_ctx* c, float* report) {
     // rewrites these values
     if (!c->solved) {
         const int meta[4] = {c->n_bricks, 0, 0, c->g.nb[2] - 1};
-        if ((e = cudaMemcpyAsync(c->d_meta, meta, sizeof(meta), cudaMemcpyHostToDevice, c->stream)) != cudaSuccess)
+        if ((e = cudaMemcpyAsync(c->d_meta, meta, sizeof(meta), cudaMemcpyHostToDevice, c->stream)) != cudaSuccess ||
+            (e = cudaMemsetAsync(c->d_meta + kMetaRows, 0xff, sizeof(int) * (kMetaInts - kMetaRows), c->stream)) !=
+                cudaSuccess)
             return cuda_fail(c, e, "ftr_autotune");
     }
     cudaEvent_t t0, t1;

@@ -25,6 +25,8 @@
 #include <set>
 #include <utility>
 
+#include "ftr_internal.h"
+
 namespace ftr {
 
 // W_96^j = exp(-2 pi i j / 96), a constant table of each translation unit,
@@ -260,6 +262,15 @@ __device__ __forceinline__ void live_z_range(const int* __restrict__ meta, int& 
     }
     zl = (bmin * 8) & ~15;
     zh = ((bmax + 1) * 8 + 15) & ~15;
+}
+
+// Which 16-row groups of z-plane z hold non-zero V: bit y / 16 (meta[kMetaRows +
+// z / 8], set by the splat per touched brick).  Rows outside them transform to
+// zero along x: the x pass neither computes nor writes their spectra and the y
+// pass takes zeros in their place.  A body in its box touches about 45 % of the
+// (y, z) rows inside its live slab.
+__device__ __forceinline__ unsigned live_rows(const int* __restrict__ meta, int z) {
+    return (unsigned)meta[kMetaRows + (z >> 3)];
 }
 
 // Ask L2 to fetch the 128-byte line holding p (no register is written, so

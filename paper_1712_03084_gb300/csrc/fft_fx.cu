@@ -22,7 +22,8 @@ constexpr int kLines = 24;
 template <int N>
 __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
     k_fx(GridDev g, const int* __restrict__ slot_tab, const float* __restrict__ vpool, float2* __restrict__ s0,
-         int64_t Mh, const float2* __restrict__ tw, float wx_scale, const int* __restrict__ meta) {
+         int64_t Mh, const float2* __restrict__ tw, float wx_scale, const int* __restrict__ meta,
+         int fill) {
     pdl_wait();
     using X = Xchg<N, kLines>;
     constexpr int NB = N / kBrick;
@@ -35,11 +36,13 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
     const int y0 = blockIdx.x * kRows;
     const int z = blockIdx.y;
     const int tid = threadIdx.x;
-    // z-planes outside the 16-aligned slab of touched bricks are never read
-    // by the later passes: nothing to write there
+    // z-planes outside the 16-aligned slab of touched bricks and, unless `fill`
+    // (a y pass that reads every row), 16-row groups without a touched brick are
+    // never read by the later passes: nothing to write there
     int zl, zh;
     live_z_range(meta, zl, zh);
     if (z < zl || z >= zh) return;
+    if (!fill && !((live_rows(meta, z) >> blockIdx.x) & 1u)) return;
     if (tid == 0) s_any = 0;
     __syncthreads();
     const int bz = z >> 3;
@@ -131,7 +134,7 @@ cudaError_t run_fx(ftr_ctx* c) {
     dim3 grid(c->g.n[1] / kRows, c->g.n[2]);
     const float wx_scale = (float)(2.0 * 3.14159265358979323846 / (c->g.n[0] * c->g.h[0]));
     launch_pdl(k_fx<N>, grid, kLines * X::NT, smem, c->stream, c->g, c->d_brick_slot, c->d_vpool, c->d_s0, c->Mh,
-                                                       c->d_tw[0], wx_scale, c->d_meta);
+                                                       c->d_tw[0], wx_scale, c->d_meta, c->fused == 2 ? 1 : 0);
     c->launches++;
     return cudaGetLastError();
 }

@@ -1,7 +1,7 @@
 // Forward pass along y, with the x and y terms of the filter combined.
 //
 // Input: the x-pass half spectra [c][k_x][z][y] (j w_x already applied to
-// c = x).  Each CTA transforms 16 contiguous y lines (z0..z0+15 at one k_x)
+// c = x), written only where a 16-row group holds a touched brick.  Each CTA transforms 16 contiguous y lines (z0..z0+15 at one k_x)
 // of the three components.  Because the integration filter of Sec. III-B is
 // j (w . V^) / |w|^2 and w_y depends only on k_y, the x and y components can
 // be summed as soon as both are transformed along y:
@@ -15,14 +15,18 @@
 namespace ftr {
 namespace {
 
-// Load line f's elements y = N2 n1 + r (contiguous) and run step 1.
+// Load line f's elements y = N2 n1 + r (contiguous) and run step 1; rows whose
+// 16-row group is not in `rows` are zero and not read (N2 divides 16, so the
+// group of an element does not depend on r).
 template <int N, int F>
 __device__ __forceinline__ void load_step1(const float2* __restrict__ src, int r, int f, float2* smem,
-                                           const float2* __restrict__ tw, uint64_t pol) {
+                                           const float2* __restrict__ tw, uint64_t pol, unsigned rows) {
     using X = Xchg<N, F>;
+    static_assert(16 % X::N2 == 0, "an element's 16-row group is n1's");
     float2 v[X::N1];
 #pragma unroll
-    for (int n1 = 0; n1 < X::N1; ++n1) v[n1] = ld_l2hint(src + X::N2 * n1 + r, pol);
+    for (int n1 = 0; n1 < X::N1; ++n1)
+        v[n1] = (rows >> (X::N2 * n1 / 16)) & 1u ? ld_l2hint(src + X::N2 * n1 + r, pol) : make_float2(0.f, 0.f);
     fft_step1<N, F, -1>(v, f, r, smem, tw);
 }
 
@@ -53,18 +57,20 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
     // the transformed x component waits in shared memory (line index fastest)
     float2* stash = smem + X::SIZE;
     const float2* line = s0 + (size_t)N * (z0 + f1 + (size_t)nz * kx);
+    const unsigned rows = live_rows(meta, z0 + f1);
     // the y and z components' lines go to L2 while the x component is
     // transformed (one prefetch per 128-byte line per thread)
     if (r1 < X::N2 && (r1 & 15) == 0) {
 #pragma unroll
         for (int n1 = 0; n1 < X::N1; ++n1) {
+            if (!((rows >> (X::N2 * n1 / 16)) & 1u)) continue;
             prefetch_l2(line + Mh + X::N2 * n1 + r1);
             prefetch_l2(line + 2 * Mh + X::N2 * n1 + r1);
         }
     }
     const uint64_t pin = l2_evict_first(), pout = l2_evict_last();
     // x component: transform along y and park it (line index fastest)
-    if (r1 < X::N2) load_step1<N, F>(line, r1, f1, smem, tw, pin);
+    if (r1 < X::N2) load_step1<N, F>(line, r1, f1, smem, tw, pin, rows);
     __syncthreads();
     float2 o[X::N2];
     if (i2 < X::N1) fft_step2<N, F, -1>(o, f2, i2, smem);
@@ -74,7 +80,7 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
         for (int k2 = 0; k2 < X::N2; ++k2) stash[f2 + (F + 1) * (i2 + X::N1 * k2)] = o[k2];
     }
     // y component: transform, then W = x + j w_y y goes out as field 0
-    if (r1 < X::N2) load_step1<N, F>(line + Mh, r1, f1, smem, tw, pin);
+    if (r1 < X::N2) load_step1<N, F>(line + Mh, r1, f1, smem, tw, pin, rows);
     __syncthreads();
     if (i2 < X::N1) fft_step2<N, F, -1>(o, f2, i2, smem);
     __syncthreads();
@@ -88,7 +94,7 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
         }
     }
     // z component: transform and write as field 1
-    if (r1 < X::N2) load_step1<N, F>(line + 2 * Mh, r1, f1, smem, tw, pin);
+    if (r1 < X::N2) load_step1<N, F>(line + 2 * Mh, r1, f1, smem, tw, pin, rows);
     __syncthreads();
     if (i2 < X::N1) {
         fft_step2<N, F, -1>(o, f2, i2, smem);
@@ -97,8 +103,8 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
     }
 }
 
-// The same pass with the CTA's three component tiles (16 lines each, one
-// contiguous block per component) fetched by bulk asynchronous copies at
+// The same pass with the CTA's three component tiles (16 lines each, per line
+// the span of its live 16-row groups) fetched by bulk asynchronous copies at
 // the start, so that all of its input is in flight at once; each tile's
 // buffer then serves as that component's exchange buffer, and the x
 // component's as the stash.  Waits are bounded (a timeout sets *err).
@@ -110,7 +116,6 @@ __global__ void __launch_bounds__(16 * Xchg<N, 16>::NT, 2)
     constexpr int F = 16;
     using X = Xchg<N, F>;
     constexpr int BUF = cmax(X::SIZE, (F + 1) * N);
-    constexpr uint32_t kBytes = F * N * sizeof(float2);
     extern __shared__ __align__(16) float2 smem[];
     __shared__ uint64_t mbar[3];
     const int nz = g.n[2];
@@ -121,18 +126,28 @@ __global__ void __launch_bounds__(16 * Xchg<N, 16>::NT, 2)
     live_z_range(meta, zl, zh);
     if (z0 + F <= zl || z0 >= zh) return;
     const size_t tile = (size_t)N * ((size_t)z0 + (size_t)nz * kx);
-    if (tid == 0) {
-        for (int c = 0; c < 3; ++c) tc::mbar_init(&mbar[c], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        for (int c = 0; c < 3; ++c) {
-            tc::mbar_expect_tx(&mbar[c], kBytes);
-            tc::bulk_g2s(smem + c * BUF, s0 + (size_t)c * Mh + tile, kBytes, &mbar[c]);
+    if (tid < 32) {
+        // lane l < 16: line l's span [y0, y1) of live rows (multiples of 16)
+        const unsigned m = tid < F ? live_rows(meta, z0 + tid) : 0u;
+        const int y0 = m ? 16 * (__ffs(m) - 1) : 0, y1 = m ? min(16 * (32 - __clz(m)), N) : 0;
+        const uint32_t bytes = (uint32_t)(y1 - y0) * (uint32_t)sizeof(float2);
+        const uint32_t all = __reduce_add_sync(0xffffffffu, bytes);
+        if (tid == 0) {
+            for (int c = 0; c < 3; ++c) tc::mbar_init(&mbar[c], 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            for (int c = 0; c < 3; ++c) tc::mbar_expect_tx(&mbar[c], all);
         }
+        __syncwarp();
+        if (bytes > 0)
+            for (int c = 0; c < 3; ++c)
+                tc::bulk_g2s(smem + c * BUF + N * tid + y0, s0 + (size_t)c * Mh + tile + (size_t)N * tid + y0, bytes,
+                             &mbar[c]);
     }
     __syncthreads();
     const int f1 = tid / X::NT, r1 = tid % X::NT;
     const int f2 = tid % F, i2 = tid / F;
     const size_t out_base = (size_t)(z0 + f2) + (size_t)nz * ((size_t)N * kx);
+    const unsigned rows = live_rows(meta, z0 + f1);
     float2* stash = smem;                      // the x component's buffer, once its exchange is done
     float2 o[X::N2];
     for (int c = 0; c < 3; ++c) {
@@ -141,7 +156,8 @@ __global__ void __launch_bounds__(16 * Xchg<N, 16>::NT, 2)
         float2 v[X::N1];
         if (r1 < X::N2) {
 #pragma unroll
-            for (int n1 = 0; n1 < X::N1; ++n1) v[n1] = B[f1 * N + X::N2 * n1 + r1];
+            for (int n1 = 0; n1 < X::N1; ++n1)
+                v[n1] = (rows >> (X::N2 * n1 / 16)) & 1u ? B[f1 * N + X::N2 * n1 + r1] : make_float2(0.f, 0.f);
         }
         __syncthreads();                       // the staged lines are in registers: B becomes the exchange
         if (r1 < X::N2) fft_step1<N, F, -1>(v, f1, r1, B, tw);

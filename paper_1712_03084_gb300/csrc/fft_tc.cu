@@ -348,6 +348,7 @@ __global__ void __launch_bounds__(kFxLines * Plan<N>::N1)
     int zl, zh;
     live_z_range(meta, zl, zh);
     if (z < zl || z >= zh) return;
+    if (!((live_rows(meta, z) >> blockIdx.x) & 1u)) return;   // zero rows: the y pass does not read them
     if (tid == 0) s_any = 0;
     __syncthreads();
     const int bz = z >> 3;
@@ -471,11 +472,14 @@ __global__ void __launch_bounds__(TcLines<N>::value * Plan<N>::N1, TcLines<N>::v
     const int f2 = tid % F, i2 = tid / F;
     const size_t out_base = (size_t)(z0 + f2) + (size_t)nz * ((size_t)N * kx);
     const float2* line = s0 + (size_t)N * (z0 + f1 + (size_t)nz * kx);
+    static_assert(16 % N2 == 0, "an element's 16-row group is n1's");
+    const unsigned rows = live_rows(meta, z0 + f1);
     float2 v[N1], o[N2];
     for (int c = 0; c < 3; ++c) {
         if (act) {
 #pragma unroll
-            for (int n1 = 0; n1 < N1; ++n1) v[n1] = line[(size_t)c * Mh + N2 * n1 + r1];
+            for (int n1 = 0; n1 < N1; ++n1)
+                v[n1] = (rows >> (N2 * n1 / 16)) & 1u ? line[(size_t)c * Mh + N2 * n1 + r1] : make_float2(0.f, 0.f);
         }
         e.template dft<N1, N2, -1, true>(v, act, f1, r1, o);
         if (c == 0) {

@@ -20,6 +20,11 @@ constexpr int kMcThreads = 256;           // CTA size of the inside-bit pass (8 
 constexpr int kMaxTrisPerCase = 5;
 constexpr int kSplatChunk = 1024;          // (point, brick) pairs per accumulation work unit
 
+// d_meta: the frame's scalars (see ftr_ctx), then per brick layer along z the
+// 16-row groups along y that hold a touched brick (bit y / 16).
+constexpr int kMetaRows = 8;
+constexpr int kMetaInts = kMetaRows + 64;
+
 enum Stage {
     ST_INGEST = 0,
     ST_SPLAT_BIN,
@@ -114,7 +119,8 @@ struct ftr_ctx {
     int* d_brick_slot = nullptr;
     int* d_active = nullptr;
     int* d_meta = nullptr;     // [0] active bricks, [1] entries, [2] min bz, [3] max bz, [4] accumulation
-                               // ticket, [5] accumulation chunks, [6] heavy bricks
+                               // ticket, [5] accumulation chunks, [6] heavy bricks,
+                               // [kMetaRows + bz] live 16-row groups of brick layer bz
     int4* d_tile = nullptr;    // per-tile sums / offsets of the brick scan (pairs, touched, chunks, heavy)
     int* d_unit_off = nullptr; // per touched brick: first accumulation chunk; [touched] = all chunks
     int* d_heavy_idx = nullptr;  // per touched brick: index of its global accumulator, -1 for one chunk

@@ -264,12 +264,13 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_sums(const int* __restric
             meta[3] = -1;
         }
     }
+    if (blockIdx.x == 0 && threadIdx.x < kMetaInts - kMetaRows) meta[kMetaRows + threadIdx.x] = 0;   // live rows: or-ed
 }
 
 // Per tile: its exclusive offset is the sum of the (few) tile sums before it,
 // summed by every CTA itself (no separate scan launch); CTA 0 also writes the
 // totals.  Then the tile's bricks get their offsets, slots and chunk ranges.
-__global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restrict__ cnt, int nb, int nbxy,
+__global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restrict__ cnt, int nb, int nbx, int nbxy,
                                                              const int4* __restrict__ tile_sum, int ntiles, int* off,
                                                              int* cursor, int* slot, int* active, int* meta,
                                                              int* unit_off, int* heavy_idx, int* unit_slot) {
@@ -321,6 +322,9 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restri
                 const int bz = b / nbxy;
                 zmin = min(zmin, bz);
                 zmax = max(zmax, bz);
+                // its pair of brick rows = 16 grid rows; the first brick of a run along x sets the bit
+                const int by = (b - bz * nbxy) / nbx;
+                if (b % nbx == 0 || cnt[b - 1] == 0) atomicOr(&meta[kMetaRows + bz], 1 << (by >> 1));
             } else {
                 slot[b] = -1;
             }
@@ -611,7 +615,7 @@ cudaError_t launch_splat(ftr_ctx* c) {
     // the per-brick point counts were taken by the ingest
     const int ntiles = (c->n_bricks + kTile - 1) / kTile;
     launch_pdl(k_brick_tile_sums, ntiles, kScanT, 0, c->stream, c->d_brick_cnt, c->n_bricks, c->d_tile, c->d_meta);
-    launch_pdl(k_brick_tile_write, ntiles, kScanT, 0, c->stream, c->d_brick_cnt, c->n_bricks, c->g.nb[0] * c->g.nb[1],
+    launch_pdl(k_brick_tile_write, ntiles, kScanT, 0, c->stream, c->d_brick_cnt, c->n_bricks, c->g.nb[0], c->g.nb[0] * c->g.nb[1],
                c->d_tile, ntiles, c->d_brick_off, c->d_brick_cursor, c->d_brick_slot, c->d_active, c->d_meta,
                c->d_unit_off, c->d_heavy_idx, c->d_unit_slot);
     c->launches += 2;
@@ -637,6 +641,8 @@ cudaError_t launch_load_dense_V(ftr_ctx* c, const float* V_dev) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int meta[4] = {c->n_bricks, 0, 0, c->g.nb[2] - 1};
+    if ((e = cudaMemsetAsync(c->d_meta + kMetaRows, 0xff, sizeof(int) * (kMetaInts - kMetaRows), c->stream)) != cudaSuccess)
+        return e;
     return cudaMemcpyAsync(c->d_meta, meta, sizeof(meta), cudaMemcpyHostToDevice, c->stream);
 }
 
