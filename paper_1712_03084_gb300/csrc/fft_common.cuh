@@ -158,11 +158,13 @@ template <> struct Plan<512> { static constexpr int N1 = 32, N2 = 16; };
 __host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 
 // Minimum resident CTAs per SM requested from the register allocator for the
-// 16-line passes: three (24 warps) while the transform still fits in 80
-// registers without spilling (n <= 256), one above.
+// 16-line passes: what 80 registers per thread allow while the transform still
+// fits in them (a spill of a few values at 384 points): three (24 warps) up to
+// 256, two (24 warps) at 384, where the y and z pass otherwise take 121-145
+// registers and run 12 warps (156 + 204 us, now 119 + 171); one above.
 template <int N>
 struct MinCtas {
-    static constexpr int value = N <= 256 ? 3 : 1;
+    static constexpr int value = N <= 256 ? 3 : (N <= 384 ? 2 : 1);
 };
 // The same register budget per thread for other tile heights F (lines per
 // CTA): F = 8 asks for twice the CTAs of F = 16, F = 32 half (at least one).
@@ -212,9 +214,13 @@ __device__ __forceinline__ void fft_step1(float2 (&v)[Plan<N>::N1], int f, int j
     Dft<X::N1, SIGN>::run(v);
 #pragma unroll
     for (int k1 = 0; k1 < X::N1; ++k1) {
-        float2 w = (k1 == 0 || j == 0) ? make_float2(1.f, 0.f) : __ldg(&tw[N + k1 * X::N2 + j]);
+        if (k1 == 0) {
+            xs[X::idx(f, j, 0)] = v[0];
+            continue;
+        }
+        float2 w = __ldg(&tw[N + k1 * X::N2 + j]);      // W^0 = 1 - 0 i for j = 0
         if (SIGN > 0) w.y = -w.y;
-        xs[X::idx(f, j, k1)] = (k1 == 0) ? v[k1] : cmul(v[k1], w);
+        xs[X::idx(f, j, k1)] = cmul(v[k1], w);
     }
 }
 
@@ -237,9 +243,13 @@ __device__ __forceinline__ void fft_step1_swapped(float2 (&v)[Plan<N>::N2], int 
     Dft<X::N2, SIGN>::run(v);
 #pragma unroll
     for (int k1 = 0; k1 < X::N2; ++k1) {
-        float2 w = (k1 == 0 || j == 0) ? make_float2(1.f, 0.f) : __ldg(&tw[2 * N + k1 * X::N1 + j]);
+        if (k1 == 0) {
+            xs[X::idxr(f, j, 0)] = v[0];
+            continue;
+        }
+        float2 w = __ldg(&tw[2 * N + k1 * X::N1 + j]);
         if (SIGN > 0) w.y = -w.y;
-        xs[X::idxr(f, j, k1)] = (k1 == 0) ? v[k1] : cmul(v[k1], w);
+        xs[X::idxr(f, j, k1)] = cmul(v[k1], w);
     }
 }
 

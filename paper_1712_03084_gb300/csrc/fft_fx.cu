@@ -19,8 +19,10 @@ namespace {
 constexpr int kRows = 16;
 constexpr int kLines = 24;
 
+// 56 registers per thread at 256 and 384 points: three and two CTAs per SM (at
+// 384 one CTA of 18 warps left its barriers and loads uncovered: 96 us, now 87).
 template <int N>
-__global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
+__global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT, N == 256 ? 3 : (N == 384 ? 2 : 1))
     k_fx(GridDev g, const int* __restrict__ slot_tab, const float* __restrict__ vpool, float2* __restrict__ s0,
          int64_t Mh, const float2* __restrict__ tw, float wx_scale, const int* __restrict__ meta,
          int fill) {
