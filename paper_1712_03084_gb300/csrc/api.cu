@@ -198,8 +198,8 @@ cudaError_t grow_entries(ftr_ctx* c, int64_t need) {
     // chunks: one per touched brick plus at most cap / chunk more
     const int64_t units = (int64_t)c->n_bricks + cap / kSplatChunk + 2;
     if (units > c->cap_units) {
-        dfree(c->d_unit_slot);
-        if ((e = dalloc(&c->d_unit_slot, (size_t)units)) != cudaSuccess) return e;
+        dfree(c->d_units);
+        if ((e = dalloc(&c->d_units, (size_t)units)) != cudaSuccess) return e;
         c->cap_units = units;
     }
     return e;
@@ -242,7 +242,7 @@ void free_all(ftr_ctx* c) {
     dfree(c->d_meta);
     dfree(c->d_tile);
     dfree(c->d_unit_off);
-    dfree(c->d_unit_slot);
+    dfree(c->d_units);
     dfree(c->d_heavy_idx);
     dfree(c->d_heavy_acc);
     dfree(c->d_heavy_done);
@@ -1483,7 +1483,7 @@ int ftr_autotune(ftr_ctx* c, float* report) {
     if (!c->solved) {
         const int meta[4] = {c->n_bricks, 0, 0, c->g.nb[2] - 1};
         if ((e = cudaMemcpyAsync(c->d_meta, meta, sizeof(meta), cudaMemcpyHostToDevice, c->stream)) != cudaSuccess ||
-            (e = cudaMemsetAsync(c->d_meta + kMetaRows, 0xff, sizeof(int) * (kMetaInts - kMetaRows), c->stream)) !=
+            (e = cudaMemsetAsync(c->d_meta + kMetaRows, 0xff, sizeof(int) * (kMetaClasses - kMetaRows), c->stream)) !=
                 cudaSuccess)
             return cuda_fail(c, e, "ftr_autotune");
     }
@@ -1620,7 +1620,7 @@ int64_t context_bytes(const int n[3], const Caps& k) {
     b += k.stage + k.tex_stage;
     b += nb * (int64_t)sizeof(int) * 5 + (nb / kBrickScanTile + 1) * (int64_t)sizeof(int4) + 64;
     b += k.entries * (int64_t)sizeof(int);
-    b += k.units * (int64_t)sizeof(int);
+    b += k.units * (int64_t)sizeof(int4);
     b += k.heavy * (4 * kBrickVox * 8 + 4) + nb * 8;   // heavy-brick accumulators, chunk offsets
     b += nb * 3 * kBrickVox * (int64_t)sizeof(float);
     b += 5 * Mh * (int64_t)sizeof(float2) + M * (int64_t)sizeof(float);

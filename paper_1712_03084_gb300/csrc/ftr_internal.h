@@ -21,9 +21,13 @@ constexpr int kMaxTrisPerCase = 5;
 constexpr int kSplatChunk = 1024;          // (point, brick) pairs per accumulation work unit
 
 // d_meta: the frame's scalars (see ftr_ctx), then per brick layer along z the
-// 16-row groups along y that hold a touched brick (bit y / 16).
+// 16-row groups along y that hold a touched brick (bit y / 16), then the number
+// of accumulation units per size class and the units placed so far (both zero
+// between frames).
+constexpr int kSizeClasses = 32;
 constexpr int kMetaRows = 8;
-constexpr int kMetaInts = kMetaRows + 64;
+constexpr int kMetaClasses = kMetaRows + 64;
+constexpr int kMetaInts = kMetaClasses + 2 * kSizeClasses;
 
 enum Stage {
     ST_INGEST = 0,
@@ -107,7 +111,7 @@ struct ftr_ctx {
     int64_t points_in = 0;             // -1: the count is on the device only (ftr_splat_depth_async)
     bool depth_async = false;          // the frame's points come from ftr_splat_depth_async
     unsigned long long* d_dropped = nullptr;
-    int* d_wild = nullptr;     // set when some accepted weight lies outside [0, 1]
+    int* d_wild = nullptr;     // bit 0: some accepted weight lies outside [0, 1], bit 1: a normal component beyond 3.9
     void* d_stage = nullptr;   // staging for host inputs
     size_t stage_cap = 0;
 
@@ -124,7 +128,7 @@ struct ftr_ctx {
     int4* d_tile = nullptr;    // per-tile sums / offsets of the brick scan (pairs, touched, chunks, heavy)
     int* d_unit_off = nullptr; // per touched brick: first accumulation chunk; [touched] = all chunks
     int* d_heavy_idx = nullptr;  // per touched brick: index of its global accumulator, -1 for one chunk
-    int* d_unit_slot = nullptr;  // per accumulation chunk: its touched brick
+    int4* d_units = nullptr;     // per accumulation chunk: brick, slot, first pair, pairs
     int64_t cap_units = 0;
     unsigned long long* d_heavy_acc = nullptr;   // 4 x 512 int64 per heavy brick (zero between frames)
     int* d_heavy_done = nullptr; // chunks finished per heavy brick (zero between frames)

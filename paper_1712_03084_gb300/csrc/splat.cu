@@ -15,7 +15,7 @@
 //           brick and the accumulation chunks (no single-CTA scan)
 //   fill    per point, append its index to each overlapped brick's list
 //   accum   persistent CTAs take work units (up to 1024 (point, brick) pairs
-//           of one touched brick) from a per-frame ticket: 64 lanes per point
+//           of one touched brick): 64 lanes per point
 //           evaluate the stencil nodes inside the brick and add the
 //           contributions to shared-memory fixed-point accumulators (value *
 //           2^40 as 32-bit hi/lo halves, exact and order-independent, so the
@@ -51,21 +51,49 @@ __device__ __forceinline__ bool stencil_bricks(const int4 b, int mode, int lo[3]
     return true;
 }
 
-// n_dev (nullable): the point count on the device; n then only bounds it.
+// Runs of equal b over the lanes of a full warp: the first lane of this lane's
+// run and the run's length.  Consecutive points are neighbouring pixels, mostly
+// in the same bricks, so one atomic per run serves almost as few addresses as
+// one per distinct value, for a shuffle and a ballot (a match over the warp
+// takes a step per distinct value: 8 of them were half of this stage).
+struct Run {
+    int first, len;
+};
+__device__ __forceinline__ Run run_of(int b, int lane) {
+    const int prev = __shfl_up_sync(0xffffffffu, b, 1);
+    const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || prev != b);
+    const unsigned upto = heads & (0xffffffffu >> (31 - lane)), after = heads & ~(0xffffffffu >> (31 - lane));
+    Run r;
+    r.first = 31 - __clz(upto);
+    r.len = (after ? __ffs(after) - 1 : 32) - r.first;
+    return r;
+}
+
 // One point: t per axis with every decision equal to the float64 one, the
 // acceptance test, and the point record at slot `dst`.
 // An accepted point also counts itself into every brick its stencil overlaps
 // (cnt: per-brick point counts of the frame, zeroed when the frame starts).
-__device__ __forceinline__ void ingest_one(const float* p, const float* q, const float* wp, int64_t dst, const GridDev& g,
+// Called by whole warps; lanes without a point have live = false.
+__device__ __forceinline__ void ingest_one(bool live, const float* p, const float* q, const float* wp, int64_t dst, const GridDev& g,
                                            int4* pbase, float4* pfrac, float4* pnrm, unsigned long long* dropped,
                                            int* wild_weights, int* cnt) {
-    bool ok = true;
+    bool ok = live;
     int fl[3] = {0, 0, 0};
     float fr[3] = {0.f, 0.f, 0.f};
+    float x3[3] = {0.f, 0.f, 0.f}, q3[3] = {0.f, 0.f, 0.f}, wi = 1.f;
+    if (live) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            x3[c] = p[c];
+            q3[c] = q[c];
+        }
+        if (wp) wi = *wp;
+    }
     int up = 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const float x = p[c];
+        if (!live) break;
+        const float x = x3[c];
         int fli;
         float r;
         bool u;
@@ -90,14 +118,13 @@ __device__ __forceinline__ void ingest_one(const float* p, const float* q, const
         }
     }
     if (!ok) {
-        atomicAdd(dropped, 1ull);
+        if (live) atomicAdd(dropped, 1ull);
         fl[0] = fl[1] = fl[2] = 0;
     }
     const int4 rec = make_int4(fl[0], fl[1], fl[2], ok ? (1 | (up << 1)) : 0);
-    pbase[dst] = rec;
-    // per brick slot k of the at most 2 x 2 x 2 bricks the stencil overlaps,
-    // the lanes counting into the same brick add their number with one atomic
-    const unsigned act = __activemask();
+    // per brick slot k of the at most 2 x 2 x 2 bricks the stencil overlaps, a
+    // run of lanes counting into the same brick adds its length with one atomic
+    const int lane = threadIdx.x & 31;
     int lo[3] = {0, 0, 0}, hi[3] = {-1, -1, -1};
     const bool any = stencil_bricks(rec, g.mode, lo, hi);
 #pragma unroll
@@ -105,26 +132,33 @@ __device__ __forceinline__ void ingest_one(const float* p, const float* q, const
         const int bx = lo[0] + (k & 1), by = lo[1] + ((k >> 1) & 1), bz = lo[2] + (k >> 2);
         const bool valid = any && bx <= hi[0] && by <= hi[1] && bz <= hi[2];
         const int b = valid ? bx + g.nb[0] * (by + g.nb[1] * bz) : -1;
-        const unsigned peers = __match_any_sync(act, b);
-        if (valid && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&cnt[b], __popc(peers));
+        const Run r = run_of(b, lane);
+        if (valid && lane == r.first) atomicAdd(&cnt[b], r.len);
     }
-    const float wi = wp ? *wp : 1.0f;
-    if (ok && !(wi >= 0.f && wi <= 1.f)) atomicOr(wild_weights, 1);   // outside the fast path's range
+    if (!live) return;
+    pbase[dst] = rec;
+    // outside the range of the accumulation's 32-bit halves (bit 0) or of its
+    // conversions by magic addition (bit 1)
+    const bool wild_w = !(wi >= 0.f && wi <= 1.f);
+    const bool wild_n = !(fabsf(q3[0]) < 3.9f && fabsf(q3[1]) < 3.9f && fabsf(q3[2]) < 3.9f);
+    if (ok && (wild_w || wild_n)) atomicOr(wild_weights, (wild_w ? 1 : 0) | (wild_n ? 2 : 0));
     pfrac[dst] = make_float4(fr[0], fr[1], fr[2], wi);
-    pnrm[dst] = make_float4(q[0], q[1], q[2], 0.f);
+    pnrm[dst] = make_float4(q3[0], q3[1], q3[2], 0.f);
 }
 
+// n_dev (nullable): the point count on the device; n then only bounds it.
 __global__ void k_ingest(const float* __restrict__ pts, const float* __restrict__ nrm,
                          const float* __restrict__ w, int64_t n, int64_t base, GridDev g, int4* pbase,
                          float4* pfrac, float4* pnrm, unsigned long long* dropped, int* wild_weights,
                          int64_t* npts_dev, const int* __restrict__ n_dev, int* cnt) {
     pdl_wait();
     if (n_dev) n = min(n, (int64_t)*n_dev);
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) *npts_dev = base + n;   // points stored so far: later kernels read the count here
-    if (i >= n) return;
-    ingest_one(pts + 3 * i, nrm + 3 * i, w ? w + i : nullptr, base + i, g, pbase, pfrac, pnrm, dropped, wild_weights,
-               cnt);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *npts_dev = base + n;   // points stored so far: later kernels read it here
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n; i0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = i0 + threadIdx.x;
+        ingest_one(i < n, pts + 3 * i, nrm + 3 * i, w ? w + i : nullptr, base + i, g, pbase, pfrac, pnrm, dropped,
+                   wild_weights, cnt);
+    }
 }
 
 // Several point sets in one launch: thread i ingests point i of the
@@ -134,11 +168,10 @@ __global__ void k_ingest_sets(IngestSets S, GridDev g, int4* pbase, float4* pfra
     pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) *npts_dev = S.base + S.off[S.k];
-    if (i >= S.off[S.k]) return;
     int s = 0;
     while (s + 1 < S.k && i >= S.off[s + 1]) ++s;
     const int64_t j = i - S.off[s];
-    ingest_one(S.pts[s] + 3 * j, S.nrm[s] + 3 * j, S.w[s] ? S.w[s] + j : nullptr, S.base + i, g, pbase, pfrac, pnrm,
+    ingest_one(i < S.off[S.k], S.pts[s] + 3 * j, S.nrm[s] + 3 * j, S.w[s] ? S.w[s] + j : nullptr, S.base + i, g, pbase, pfrac, pnrm,
                dropped, wild_weights, cnt);
 }
 
@@ -146,8 +179,10 @@ __global__ void k_ingest_sets(IngestSets S, GridDev g, int4* pbase, float4* pfra
 // launch does not depend on it.
 // A warp takes 32 consecutive points (neighbouring pixels of one camera,
 // mostly the same bricks): per brick slot k of the at most 2 x 2 x 2 bricks
-// a stencil overlaps, the lanes that append to the same brick reserve their
-// places with one atomic (the lowest lane's) and write at their rank.
+// a stencil overlaps, a run of lanes that append to the same brick reserves its
+// places with one atomic (the first lane's) and each writes at its rank.  The
+// atomics of the eight slots are all issued before the first place is used:
+// one after another, their round trips made this pass 7-12 us.
 __global__ void k_brick_fill(const int4* __restrict__ pbase, const int64_t* __restrict__ npts, GridDev g,
                              int* cursor, int* entries) {
     pdl_wait();
@@ -159,19 +194,22 @@ __global__ void k_brick_fill(const int4* __restrict__ pbase, const int64_t* __re
         const int64_t i = i0 + lane;
         int lo[3] = {0, 0, 0}, hi[3] = {-1, -1, -1};
         const bool ok = i < n && stencil_bricks(pbase[i], g.mode, lo, hi);
+        Run run[8];
+        int pos[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int bx = lo[0] + (k & 1), by = lo[1] + ((k >> 1) & 1), bz = lo[2] + (k >> 2);
             const bool valid = ok && bx <= hi[0] && by <= hi[1] && bz <= hi[2];
             const int b = valid ? bx + g.nb[0] * (by + g.nb[1] * bz) : -1;
-            const unsigned peers = __match_any_sync(0xffffffffu, b);
-            if (valid) {
-                const int leader = __ffs(peers) - 1;
-                int pos = 0;
-                if (lane == leader) pos = atomicAdd(&cursor[b], __popc(peers));
-                pos = __shfl_sync(peers, pos, leader) + __popc(peers & ((1u << lane) - 1u));
-                entries[pos] = (int)i;
-            }
+            run[k] = run_of(b, lane);
+            pos[k] = 0;
+            if (valid && lane == run[k].first) pos[k] = atomicAdd(&cursor[b], run[k].len);
+            if (!valid) run[k].len = 0;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int at = __shfl_sync(0xffffffffu, pos[k], run[k].first);
+            if (run[k].len) entries[at + lane - run[k].first] = (int)i;
         }
     }
 }
@@ -188,6 +226,7 @@ static_assert(kTile % kScanT == 0, "a tile is a whole number of block scans");
 // pairs, one chunk per CTA at a time; the 32-bit hi/lo accumulators stay exact
 // for up to 2047 contributions per voxel.
 constexpr int kChunk = kSplatChunk;
+constexpr int kHeavyUnit = 1 << 30;   // the unit's brick has more than one chunk
 
 // Block-wide exclusive scan of four ints per thread (kScanT threads).
 __device__ __forceinline__ int4 block_scan4(int4 v, int4& total, int4* sh) {
@@ -240,10 +279,16 @@ __device__ __forceinline__ int4 brick_counts(int c) {
     return make_int4(c, c > 0, ch, ch > 1);
 }
 
+// Size class of a unit of n pairs: 32 pairs wide (the last: 993 to kChunk).
+__device__ __forceinline__ int size_class(int n) { return min((n - 1) >> 5, kSizeClasses - 1); }
+
 __global__ void __launch_bounds__(kScanT) k_brick_tile_sums(const int* __restrict__ cnt, int nb, int4* tile_sum,
                                                             int* meta) {
     pdl_wait();
     __shared__ int4 sh[kScanT / 32];
+    __shared__ int s_class[kSizeClasses];
+    if (threadIdx.x < kSizeClasses) s_class[threadIdx.x] = 0;
+    __syncthreads();
     int4 v = make_int4(0, 0, 0, 0);
     for (int k = 0; k < kTile / kScanT; ++k) {
         const int b = blockIdx.x * kTile + k * kScanT + threadIdx.x;
@@ -253,10 +298,14 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_sums(const int* __restric
             v.y += q.y;
             v.z += q.z;
             v.w += q.w;
+            if (q.z > 1) atomicAdd(&s_class[kSizeClasses - 1], q.z - 1);   // full chunks
+            if (q.z > 0) atomicAdd(&s_class[size_class(q.x - (q.z - 1) * kChunk)], 1);
         }
     }
     int4 tot;
     block_scan4(v, tot, sh);
+    if (threadIdx.x < kSizeClasses && s_class[threadIdx.x])
+        atomicAdd(&meta[kMetaClasses + threadIdx.x], s_class[threadIdx.x]);
     if (threadIdx.x == 0) {
         tile_sum[blockIdx.x] = tot;
         if (blockIdx.x == 0) {       // the z range is min/max-reduced by the write kernel
@@ -264,7 +313,7 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_sums(const int* __restric
             meta[3] = -1;
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x < kMetaInts - kMetaRows) meta[kMetaRows + threadIdx.x] = 0;   // live rows: or-ed
+    if (blockIdx.x == 0 && threadIdx.x < kMetaClasses - kMetaRows) meta[kMetaRows + threadIdx.x] = 0;   // live rows: or-ed
 }
 
 // Per tile: its exclusive offset is the sum of the (few) tile sums before it,
@@ -273,9 +322,14 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_sums(const int* __restric
 __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restrict__ cnt, int nb, int nbx, int nbxy,
                                                              const int4* __restrict__ tile_sum, int ntiles, int* off,
                                                              int* cursor, int* slot, int* active, int* meta,
-                                                             int* unit_off, int* heavy_idx, int* unit_slot) {
+                                                             int* unit_off, int* heavy_idx, int4* units) {
     pdl_wait();
     __shared__ int4 sh[kScanT / 32];
+    // units of this tile per size class, then where they go: after the larger
+    // classes' units and the units of its class that other tiles placed first
+    __shared__ int s_class[kSizeClasses];
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < kSizeClasses) s_class[threadIdx.x] = 0;
     int4 pre = make_int4(0, 0, 0, 0), all = make_int4(0, 0, 0, 0);
     for (int i = threadIdx.x; i < ntiles; i += kScanT) {
         const int4 v = tile_sum[i];
@@ -302,13 +356,31 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restri
         meta[5] = total.z;             // chunks in all
         meta[6] = total.w;             // heavy bricks
     }
+    static_assert(kTile == kScanT, "a thread per brick");
     int zmin = 0x7fffffff, zmax = -1;
-    for (int k = 0; k < kTile / kScanT; ++k) {
-        const int b = blockIdx.x * kTile + k * kScanT + threadIdx.x;
+    {
+        const int b = blockIdx.x * kTile + threadIdx.x;
         const int c = b < nb ? cnt[b] : 0;
         const int4 q = brick_counts(c);
+        // rank of the brick's full chunks and of its last chunk in their classes
+        const int nlast = c - (q.z - 1) * kChunk;
+        int rfull = 0, rlast = 0;
+        if (q.z > 1) rfull = atomicAdd(&s_class[kSizeClasses - 1], q.z - 1);
+        if (q.z > 0) rlast = atomicAdd(&s_class[size_class(nlast)], 1);
         int4 tot;
         const int4 ex = block_scan4(q, tot, sh);
+        if (threadIdx.x < kSizeClasses) {
+            const int mine = s_class[lane], count = meta[kMetaClasses + lane];
+            const int at = mine ? atomicAdd(&meta[kMetaClasses + kSizeClasses + lane], mine) : 0;
+            int larger = count;                      // inclusive sum over the classes from this one up
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_down_sync(0xffffffffu, larger, o);
+                if (lane + o < 32) larger += v;
+            }
+            s_class[lane] = larger - count + at;
+        }
+        __syncthreads();
         if (b < nb) {
             off[b] = run.x + ex.x;
             cursor[b] = run.x + ex.x;
@@ -317,11 +389,14 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restri
                 slot[b] = s;
                 active[s] = b;
                 unit_off[s] = run.z + ex.z;
-                for (int j = 0; j < q.z; ++j) unit_slot[run.z + ex.z + j] = s;
+                // per chunk all that its CTA needs: brick, slot, first pair, pairs (| kHeavyUnit)
+                const int hv = q.w ? kHeavyUnit : 0;
+                for (int j = 0; j + 1 < q.z; ++j)
+                    units[s_class[kSizeClasses - 1] + rfull + j] = make_int4(b, s, run.x + ex.x + j * kChunk, kChunk | hv);
+                units[s_class[size_class(nlast)] + rlast] = make_int4(b, s, run.x + ex.x + (q.z - 1) * kChunk, nlast | hv);
                 heavy_idx[s] = q.w ? run.w + ex.w : -1;
                 const int bz = b / nbxy;
-                zmin = min(zmin, bz);
-                zmax = max(zmax, bz);
+                zmin = zmax = bz;
                 // its pair of brick rows = 16 grid rows; the first brick of a run along x sets the bit
                 const int by = (b - bz * nbxy) / nbx;
                 if (b % nbx == 0 || cnt[b - 1] == 0) atomicOr(&meta[kMetaRows + bz], 1 << (by >> 1));
@@ -329,10 +404,6 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restri
                 slot[b] = -1;
             }
         }
-        run.x += tot.x;
-        run.y += tot.y;
-        run.z += tot.z;
-        run.w += tot.w;
     }
     if (zmax >= 0) {
         atomicMin(&meta[2], zmin);
@@ -340,7 +411,7 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restri
     }
 }
 
-constexpr int kAccThreads = 512;
+constexpr int kAccThreads = 256;
 
 // round(v * 2^40) as int64 without a 64-bit conversion (those run on the slow
 // double-precision pipe): with x = v 2^9, hi = trunc(x) and r = x - hi (exact:
@@ -375,10 +446,29 @@ __device__ __forceinline__ void fix40_split(float v, int& hi, int& lo) {
     lo = __float2int_rn(fmaf(hf, -9.5367431640625e-07f, v) * 1099511627776.0f);
 }
 
-// Persistent CTAs take work units from a per-frame ticket: a unit is one
-// chunk of at most kChunk (point, brick) pairs of one touched brick.  64
-// lanes per point evaluate the stencil nodes that fall inside the brick and
-// add the fixed-point contributions to shared-memory accumulators.  Integer
+// The same for |v| < 4: adding 1.5 2^23 rounds to an integer (ties to even) and
+// leaves it in the low mantissa bits.  The three conversions per component of
+// fix40_split run on a unit with a quarter of the rate; these run at full rate.
+__device__ __forceinline__ void fix40_split_magic(float v, int& hi, int& lo) {
+    constexpr float kMagic = 12582912.0f;
+    const float f = __fmaf_rn(v, 1048576.0f, kMagic);
+    hi = __float_as_int(f) - __float_as_int(kMagic);
+    const float r = __fmaf_rn(__fsub_rn(f, kMagic), -9.5367431640625e-07f, v);
+    lo = __float_as_int(__fmaf_rn(r, 1099511627776.0f, kMagic)) - __float_as_int(kMagic);
+}
+
+// Accumulator index of brick node li = x + 8 y + 64 z: planes 68 apart, so that
+// the 4 x 4 nodes of two adjacent planes that a warp adds to fall on 32
+// different banks.
+constexpr int kPlane = 68;
+constexpr int kAccVox = 8 * kPlane;
+__device__ __forceinline__ int acc_of(int li) { return (li & 63) + kPlane * (li >> 6); }
+
+// Persistent CTAs take work units: a unit is one chunk of at most kChunk
+// (point, brick) pairs of one touched brick, described by one record.  A warp
+// takes a pair: 4 x 4 nodes of two stencil planes per step, over the planes
+// that fall inside the brick (2.9 of 4 on average), and adds the fixed-point
+// contributions to shared-memory accumulators.  Integer
 // sums are exact and order-independent, so V is bit-reproducible.  32-bit
 // atomics on the (hi, lo) parts, exact while a voxel receives fewer than 2^11
 // contributions of magnitude <= 1 (a chunk has at most kChunk points; weights
@@ -387,101 +477,123 @@ __device__ __forceinline__ void fix40_split(float v, int& hi, int& lo) {
 // of a heavier brick add their exact sums into its int64 accumulator in
 // global memory, and the chunk that completes last (a per-brick counter)
 // writes V and clears the accumulator for the next frame.
-__global__ void __launch_bounds__(kAccThreads) k_splat_accum(GridDev g, const int* __restrict__ active,
-                                                             const int* __restrict__ meta,
-                                                             const int* __restrict__ off,
-                                                             const int* __restrict__ entries,
-                                                             const int4* __restrict__ pbase,
-                                                             const float4* __restrict__ pfrac,
-                                                             const float4* __restrict__ pnrm,
-                                                             const int* __restrict__ wild_weights,
-                                                             float* __restrict__ vpool, int* __restrict__ ticket,
-                                                             const int* __restrict__ unit_off,
-                                                             const int* __restrict__ unit_slot,
-                                                             const int* __restrict__ heavy_idx,
-                                                             unsigned long long* __restrict__ heavy_acc,
-                                                             int* __restrict__ heavy_done) {
+//
+// Bricks differ in size by a factor of a hundred, and an SM holds only about
+// seven of a 256^3 frame's: in grid order one SM ran 2.4 times the mean.  The
+// binning therefore lists the units by size, largest first: unit u < gridDim.x
+// belongs to CTA u, so that each SM starts with one of every size, and the
+// ticket (zeroed by the binning) gives out the small rest, drawn while the
+// current unit runs (256^3 frame: 43 us, now 34).  (Without atomics, each warp owning two planes of the
+// brick, the work was less evenly spread within a CTA and took longer.)
+template <bool WEIGHTED>
+__global__ void __launch_bounds__(kAccThreads, 6) k_splat_accum(GridDev g, int* __restrict__ meta,
+                                                                const int4* __restrict__ units,
+                                                                const int* __restrict__ entries,
+                                                                const int4* __restrict__ pbase,
+                                                                const float4* __restrict__ pfrac,
+                                                                const float4* __restrict__ pnrm,
+                                                                const int* __restrict__ wild_weights,
+                                                                float* __restrict__ vpool,
+                                                                const int* __restrict__ unit_off,
+                                                                const int* __restrict__ heavy_idx,
+                                                                unsigned long long* __restrict__ heavy_acc,
+                                                                int* __restrict__ heavy_done) {
     pdl_wait();
-    __shared__ __align__(16) unsigned acc[8][kBrickVox];   // fast: [c] hi, [4 + c] lo; slow: 4 x int64
-    __shared__ int4 s_base[kStage];
-    __shared__ float4 s_frac[kStage];
-    __shared__ float4 s_nrm[kStage];
-    unsigned long long* acc64 = reinterpret_cast<unsigned long long*>(&acc[0][0]);
-    const int tid = threadIdx.x;
-    const int o = tid & 63;
-    const int ox = o & 3, oy = (o >> 2) & 3, oz = o >> 4;
-    const int pl = tid >> 6;
-    const bool weights_ok = wild_weights[0] == 0;
-    const int nunits = meta[5];
-    __shared__ int s_unit, s_slot;
+    __shared__ __align__(16) unsigned acc[8][kAccVox];   // fast: [c] hi, [4 + c] lo; slow: 4 x int64
+    __shared__ float4 s_frac[kStage];    // frac + 1 per axis (weighted), W
+    __shared__ float4 s_nrm[kStage];     // N, stencil corner in the brick as packed bytes
+    __shared__ int s_next;
     __shared__ bool s_last;
-    for (;;) {
-        if (tid == 0) {
-            const int u = atomicAdd(ticket, 1);
-            s_unit = u;
-            s_slot = u < nunits ? unit_slot[u] : 0;   // the touched brick whose chunks hold unit u
-        }
-        __syncthreads();
-        const int unit = s_unit, s = s_slot;
-        if (unit >= nunits) break;                                      // block-uniform
-        const int b = active[s];
+    const int tid = threadIdx.x;
+    const int lane = tid & 31, warp = tid >> 5;
+    const int ox = lane & 3, oy = (lane >> 2) & 3;
+    unsigned long long* acc64 = reinterpret_cast<unsigned long long*>(&acc[0][0]);
+    const float fox = (float)ox, foy = (float)oy;
+    // packed node coordinates: fields at bits 0, 12 and 24, biased by 8, so that
+    // a coordinate lies in the brick iff bit 3 is set and bit 4 clear
+    const unsigned lane_off = (unsigned)(ox | (oy << 12));
+    const int wild = wild_weights[0];
+    const bool fast = !(wild & 1), magic = wild == 0;                   // block-uniform
+    const int nunits = meta[5];
+    if (blockIdx.x == 0 && tid < 2 * kSizeClasses) meta[kMetaClasses + tid] = 0;   // for the next frame's binning
+    for (int unit = blockIdx.x; unit < nunits;) {
+        if (tid == 0) s_next = (int)gridDim.x + atomicAdd(meta + 4, 1);   // needed after this unit
+        const int4 U = units[unit];
+        const int b = U.x, s = U.y, e0 = U.z, e1 = U.z + (U.w & (kHeavyUnit - 1));
+        const bool heavy = (U.w & kHeavyUnit) != 0;
         const int bx = b % g.nb[0], by = (b / g.nb[0]) % g.nb[1], bz = b / (g.nb[0] * g.nb[1]);
         const int orgx = bx * kBrick, orgy = by * kBrick, orgz = bz * kBrick;
-        const int nchunks = unit_off[s + 1] - unit_off[s];
-        const int e0 = off[b] + (unit - unit_off[s]) * kChunk;
-        const int e1 = min(off[b + 1], e0 + kChunk);
-        const bool fast = weights_ok;                                   // block-uniform
-        for (int k = tid; k < 8 * kBrickVox; k += kAccThreads) (&acc[0][0])[k] = 0u;
+        for (int k = tid; k < 8 * kAccVox / 4; k += kAccThreads)
+            reinterpret_cast<uint4*>(&acc[0][0])[k] = make_uint4(0u, 0u, 0u, 0u);
         for (int eb = e0; eb < e1; eb += kStage) {
             const int nbatch = min(kStage, e1 - eb);
-            __syncthreads();
+            if (eb != e0) __syncthreads();       // the previous batch is done with
             if (tid < nbatch) {
                 const int i = entries[eb + tid];
-                s_base[tid] = pbase[i];
-                s_frac[tid] = pfrac[i];
-                s_nrm[tid] = pnrm[i];
+                const int4 pb = pbase[i];
+                const float4 fr = pfrac[i], nr = pnrm[i];
+                unsigned pk;
+                if (WEIGHTED) {
+                    // corner of the 4^3 stencil relative to the brick: -3 .. 7 per axis
+                    pk = (unsigned)(pb.x - 1 - orgx + 8) | (unsigned)(pb.y - 1 - orgy + 8) << 12 |
+                         (unsigned)(pb.z - 1 - orgz + 8) << 24;
+                    // X - p(q) = (t - q) h with t - q = frac + 1 - offset
+                    s_frac[tid] = make_float4(fr.x + 1.0f, fr.y + 1.0f, fr.z + 1.0f, fr.w);
+                } else {
+                    // the nearest node: inside the brick
+                    pk = (unsigned)(pb.x + ((pb.w >> 1) & 1) - orgx) | (unsigned)(pb.y + ((pb.w >> 2) & 1) - orgy) << 3 |
+                         (unsigned)(pb.z + ((pb.w >> 3) & 1) - orgz) << 6;
+                }
+                s_nrm[tid] = make_float4(nr.x, nr.y, nr.z, __uint_as_float(pk));
             }
             __syncthreads();
-            if (g.mode == FTR_SPLAT_WEIGHTED) {
-                for (int p = pl; p < nbatch; p += kAccThreads / 64) {
-                    const int4 pb = s_base[p];
-                    const int lx = pb.x - 1 + ox - orgx;
-                    const int ly = pb.y - 1 + oy - orgy;
-                    const int lz = pb.z - 1 + oz - orgz;
-                    if ((unsigned)lx >= kBrick || (unsigned)ly >= kBrick || (unsigned)lz >= kBrick) continue;
-                    const float4 fr = s_frac[p];
-                    const float4 nr = s_nrm[p];
-                    // X - p(q) = (t - q) h with t - q = frac + 1 - offset
-                    const float dx = (fr.x + 1.0f - (float)ox) * g.hf[0];
-                    const float dy = (fr.y + 1.0f - (float)oy) * g.hf[1];
-                    const float dz = (fr.z + 1.0f - (float)oz) * g.hf[2];
-                    const float r2 = dx * dx + dy * dy + dz * dz;
-                    const float e1v = expf(-r2 * g.inv_s1sq) * fr.w;   // sigma1 * g1 * W
-                    const float e2v = expf(-r2 * g.inv_s2sq) * fr.w;   // sigma2 * g2 * W
-                    const int li = lx + kBrick * (ly + kBrick * lz);
-                    const float val[4] = {e1v * nr.x, e1v * nr.y, e1v * nr.z, e2v};
-                    if (fast) {
+            if (WEIGHTED) {
+                for (int p = warp; p < nbatch; p += kAccThreads / 32) {
+                    const float4 nr = s_nrm[p], fr = s_frac[p];
+                    const unsigned pk = __float_as_uint(nr.w), q = pk + lane_off;
+                    const bool in_xy = (q & 0x18018u) == 0x08008u;
+                    const int zc = (int)(pk >> 24) - 8;                 // first stencil plane, warp-uniform
+                    const int z1 = min(3, 7 - zc);                      // last one in the brick
+                    const float dx = (fr.x - fox) * g.hf[0];
+                    const float dy = (fr.y - foy) * g.hf[1];
+                    const float rxy = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
+                    const int lxy = (int)((q & 7u) | ((q >> 9) & 0x38u));
+                    for (int zb = max(0, -zc); zb <= z1; zb += 2) {
+                        const int oz = zb + (lane >> 4);
+                        if (!in_xy || oz > z1) continue;
+                        const float dz = (fr.z - (float)oz) * g.hf[2];
+                        const float r2 = __fmaf_rn(dz, dz, rxy);
+                        const float e1v = expf(-r2 * g.inv_s1sq) * fr.w;   // sigma1 * g1 * W
+                        const float e2v = expf(-r2 * g.inv_s2sq) * fr.w;   // sigma2 * g2 * W
+                        const int li = lxy + kPlane * (zc + oz);
+                        const float val[4] = {e1v * nr.x, e1v * nr.y, e1v * nr.z, e2v};
+                        if (magic) {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            int hi, lo;
-                            fix40_split(val[c], hi, lo);
-                            atomicAdd(reinterpret_cast<int*>(&acc[c][li]), hi);
-                            atomicAdd(reinterpret_cast<int*>(&acc[4 + c][li]), lo);
+                            for (int c = 0; c < 4; ++c) {
+                                int hi, lo;
+                                fix40_split_magic(val[c], hi, lo);
+                                atomicAdd(reinterpret_cast<int*>(&acc[c][li]), hi);
+                                atomicAdd(reinterpret_cast<int*>(&acc[4 + c][li]), lo);
+                            }
+                        } else if (fast) {
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                int hi, lo;
+                                fix40_split(val[c], hi, lo);
+                                atomicAdd(reinterpret_cast<int*>(&acc[c][li]), hi);
+                                atomicAdd(reinterpret_cast<int*>(&acc[4 + c][li]), lo);
+                            }
+                        } else {
+#pragma unroll
+                            for (int c = 0; c < 4; ++c)
+                                atomicAdd(&acc64[c * kAccVox + li], (unsigned long long)fix40(val[c]));
                         }
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            atomicAdd(&acc64[c * kBrickVox + li], (unsigned long long)fix40(val[c]));
                     }
                 }
             } else {
                 for (int p = tid; p < nbatch; p += kAccThreads) {
-                    const int4 pb = s_base[p];
-                    const int lx = pb.x + ((pb.w >> 1) & 1) - orgx;
-                    const int ly = pb.y + ((pb.w >> 2) & 1) - orgy;
-                    const int lz = pb.z + ((pb.w >> 3) & 1) - orgz;
                     const float4 nr = s_nrm[p];
-                    const int li = lx + kBrick * (ly + kBrick * lz);
+                    const int li = acc_of((int)__float_as_uint(nr.w));
                     const float val[3] = {nr.x, nr.y, nr.z};
                     if (fast) {
 #pragma unroll
@@ -495,59 +607,71 @@ __global__ void __launch_bounds__(kAccThreads) k_splat_accum(GridDev g, const in
                     } else {
 #pragma unroll
                         for (int c = 0; c < 3; ++c)
-                            atomicAdd(&acc64[c * kBrickVox + li], (unsigned long long)fix40(val[c]));
-                        atomicAdd(&acc64[3 * kBrickVox + li], 1ull << 40);
+                            atomicAdd(&acc64[c * kAccVox + li], (unsigned long long)fix40(val[c]));
+                        atomicAdd(&acc64[3 * kAccVox + li], 1ull << 40);
                     }
                 }
             }
         }
         __syncthreads();
+        const int next = s_next;
         float* out = vpool + (size_t)s * 3 * kBrickVox;
+        auto own_sums = [&](int a, long long (&u)[4]) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                u[c] = fast ? (long long)(int)acc[c][a] * (1ll << 20) + (long long)(int)acc[4 + c][a]
+                            : (long long)acc64[c * kAccVox + a];
+        };
+        bool write = true;
         unsigned long long* gacc = nullptr;
-        if (nchunks > 1) {
+        if (heavy) {
             // add this chunk's exact sums to the brick's global accumulator
-            gacc = heavy_acc + (size_t)heavy_idx[s] * 4 * kBrickVox;
+            const int h = heavy_idx[s], nchunks = unit_off[s + 1] - unit_off[s];
+            gacc = heavy_acc + (size_t)h * 4 * kBrickVox;
             for (int li = tid; li < kBrickVox; li += kAccThreads) {
+                long long u[4];
+                own_sums(acc_of(li), u);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const long long v = fast ? (long long)(int)acc[c][li] * (1ll << 20) + (long long)(int)acc[4 + c][li]
-                                             : (long long)acc64[c * kBrickVox + li];
-                    if (v != 0) atomicAdd(&gacc[c * kBrickVox + li], (unsigned long long)v);
-                }
+                for (int c = 0; c < 4; ++c)
+                    if (u[c] != 0) atomicAdd(&gacc[c * kBrickVox + li], (unsigned long long)u[c]);
             }
             __threadfence();
             __syncthreads();
-            if (tid == 0) s_last = atomicAdd(&heavy_done[heavy_idx[s]], 1) == nchunks - 1;
+            if (tid == 0) {
+                s_last = atomicAdd(&heavy_done[h], 1) == nchunks - 1;
+                if (s_last) heavy_done[h] = 0;                          // cleared for the next frame
+            }
             __syncthreads();
-            if (!s_last) continue;                                      // block-uniform; next unit
+            write = s_last;                                             // block-uniform
             __threadfence();
         }
-        for (int li = tid; li < kBrickVox; li += kAccThreads) {
-            long long u[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
+        if (write) {
+            for (int li = tid; li < kBrickVox; li += kAccThreads) {
+                long long u[4];
                 if (gacc) {
-                    u[c] = (long long)__ldcg(&gacc[c * kBrickVox + li]);
-                    gacc[c * kBrickVox + li] = 0ull;                    // cleared for the next frame
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        u[c] = (long long)__ldcg(&gacc[c * kBrickVox + li]);
+                        gacc[c * kBrickVox + li] = 0ull;                // cleared for the next frame
+                    }
                 } else {
-                    u[c] = fast ? (long long)(int)acc[c][li] * (1ll << 20) + (long long)(int)acc[4 + c][li]
-                                : (long long)acc64[c * kBrickVox + li];
+                    own_sums(acc_of(li), u);
+                }
+                if (u[3] > 0) {
+                    // exact integer sums, one float32 quotient per voxel
+                    const float sc = g.v_scale_f / fix_to_float(u[3]);
+                    out[li] = fix_to_float(u[0]) * sc;
+                    out[kBrickVox + li] = fix_to_float(u[1]) * sc;
+                    out[2 * kBrickVox + li] = fix_to_float(u[2]) * sc;
+                } else {
+                    out[li] = 0.f;
+                    out[kBrickVox + li] = 0.f;
+                    out[2 * kBrickVox + li] = 0.f;
                 }
             }
-            if (u[3] > 0) {
-                // exact integer sums, one float32 quotient per voxel
-                const float sc = g.v_scale_f / fix_to_float(u[3]);
-                out[li] = fix_to_float(u[0]) * sc;
-                out[kBrickVox + li] = fix_to_float(u[1]) * sc;
-                out[2 * kBrickVox + li] = fix_to_float(u[2]) * sc;
-            } else {
-                out[li] = 0.f;
-                out[kBrickVox + li] = 0.f;
-                out[2 * kBrickVox + li] = 0.f;
-            }
         }
-        if (gacc && tid == 0) heavy_done[heavy_idx[s]] = 0;
-        __syncthreads();
+        unit = next;
+        __syncthreads();                        // accumulators and s_next are free again
     }
 }
 
@@ -589,8 +713,11 @@ inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t
 cudaError_t launch_ingest(ftr_ctx* c, const float* pts, const float* nrm, const float* w, int64_t n,
                           const int* n_dev) {
     if (n == 0) return cudaSuccess;
-    // small CTAs spread the few float64 operations per point over every SM
-    launch_pdl(k_ingest, blocks_for(n, 32), 32, 0, c->stream, pts, nrm, w, n, c->n_pts, c->g, c->pts.base, c->pts.frac,
+    // small CTAs spread the few float64 operations per point over every SM; with
+    // the count on the device (n = every depth pixel) they stride over it: a CTA
+    // per 32 pixels ran 40,704 CTAs for 65,000 points, 24 us
+    const unsigned blocks = n_dev ? (unsigned)min((int64_t)152 * 32, (int64_t)blocks_for(n, 32)) : blocks_for(n, 32);
+    launch_pdl(k_ingest, blocks, 32, 0, c->stream, pts, nrm, w, n, c->n_pts, c->g, c->pts.base, c->pts.frac,
                                                        c->pts.nrm, c->d_dropped, c->d_wild, c->d_npts, n_dev,
                                                        c->d_brick_cnt);
     c->launches++;
@@ -617,7 +744,7 @@ cudaError_t launch_splat(ftr_ctx* c) {
     launch_pdl(k_brick_tile_sums, ntiles, kScanT, 0, c->stream, c->d_brick_cnt, c->n_bricks, c->d_tile, c->d_meta);
     launch_pdl(k_brick_tile_write, ntiles, kScanT, 0, c->stream, c->d_brick_cnt, c->n_bricks, c->g.nb[0], c->g.nb[0] * c->g.nb[1],
                c->d_tile, ntiles, c->d_brick_off, c->d_brick_cursor, c->d_brick_slot, c->d_active, c->d_meta,
-               c->d_unit_off, c->d_heavy_idx, c->d_unit_slot);
+               c->d_unit_off, c->d_heavy_idx, c->d_units);
     c->launches += 2;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     launch_pdl(k_brick_fill, sms * 2, 256, 0, c->stream, c->pts.base, c->d_npts, c->g, c->d_brick_cursor, c->d_entries);
@@ -625,10 +752,10 @@ cudaError_t launch_splat(ftr_ctx* c) {
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     prof_end(c, ST_SPLAT_BIN);
     prof_begin(c, ST_SPLAT_ACC);
-    const int grid = sms * 4;
-    launch_pdl(k_splat_accum, grid, kAccThreads, 0, c->stream, c->g, c->d_active, c->d_meta, c->d_brick_off, c->d_entries,
-               c->pts.base, c->pts.frac, c->pts.nrm, c->d_wild, c->d_vpool, c->d_meta + 4, c->d_unit_off,
-               c->d_unit_slot, c->d_heavy_idx, c->d_heavy_acc, c->d_heavy_done);
+    const int grid = sms * 6;
+    launch_pdl(c->g.mode == FTR_SPLAT_WEIGHTED ? k_splat_accum<true> : k_splat_accum<false>, grid, kAccThreads, 0,
+               c->stream, c->g, c->d_meta, c->d_units, c->d_entries, c->pts.base, c->pts.frac, c->pts.nrm, c->d_wild,
+               c->d_vpool, c->d_unit_off, c->d_heavy_idx, c->d_heavy_acc, c->d_heavy_done);
     c->launches++;
     prof_end(c, ST_SPLAT_ACC);
     return cudaGetLastError();
@@ -641,7 +768,7 @@ cudaError_t launch_load_dense_V(ftr_ctx* c, const float* V_dev) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int meta[4] = {c->n_bricks, 0, 0, c->g.nb[2] - 1};
-    if ((e = cudaMemsetAsync(c->d_meta + kMetaRows, 0xff, sizeof(int) * (kMetaInts - kMetaRows), c->stream)) != cudaSuccess)
+    if ((e = cudaMemsetAsync(c->d_meta + kMetaRows, 0xff, sizeof(int) * (kMetaClasses - kMetaRows), c->stream)) != cudaSuccess)
         return e;
     return cudaMemcpyAsync(c->d_meta, meta, sizeof(meta), cudaMemcpyHostToDevice, c->stream);
 }
