@@ -38,21 +38,11 @@ int cuda_fail(ftr_ctx* c, cudaError_t e, const char* what) {
 // After a stream synchronisation: FTR_ETIMEOUT if a tensor-core completion
 // wait of the split-precision passes gave up since the last check.
 int tc_check(ftr_ctx* c, const char* who) {
-    // the flags reached c->h_flags with the frame's last copy (see launch_flags)
-    if (!c->h_flags || (!c->h_flags[0] && !c->h_flags[1])) return FTR_OK;
-    c->h_flags[0] = c->h_flags[1] = 0;
-    if (c->d_tc_err) cudaMemsetAsync(c->d_tc_err, 0, sizeof(int), c->stream);
-    if (c->d_kerr) cudaMemsetAsync(c->d_kerr, 0, sizeof(int), c->stream);
+    // the kernels raise the flags in page-locked host memory
+    volatile int* f = c->h_flags;
+    if (!f || (!f[0] && !f[1])) return FTR_OK;
+    f[0] = f[1] = 0;
     return set_err(c, FTR_ETIMEOUT, "%s: a device completion wait timed out", who);
-}
-
-// Enqueue the copy of the device wait flags into pinned host memory.
-cudaError_t launch_flags(ftr_ctx* c) {
-    cudaError_t e = cudaSuccess;
-    if (c->d_tc_err) e = cudaMemcpyAsync(&c->h_flags[0], c->d_tc_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess && c->d_kerr)
-        e = cudaMemcpyAsync(&c->h_flags[1], c->d_kerr, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    return e;
 }
 
 void prof_begin(ftr_ctx* c, int st) {
@@ -230,9 +220,6 @@ void free_all(ftr_ctx* c) {
     dfree(c->pts.base);
     dfree(c->pts.frac);
     dfree(c->pts.nrm);
-    dfree(c->d_dropped);
-    dfree(c->d_npts);
-    dfree(c->d_wild);
     if (c->d_stage) cudaFree(c->d_stage);
     dfree(c->d_brick_cnt);
     dfree(c->d_brick_off);
@@ -258,8 +245,6 @@ void free_all(ftr_ctx* c) {
     dfree(c->d_raw_tiles);
     dfree(c->d_raw_total);
     if (c->h_raw_total) cudaFreeHost(c->h_raw_total);
-    dfree(c->d_tc_err);
-    dfree(c->d_kerr);
     dfree(c->d_ring);
     dfree(c->d_yz_sync);
     dfree(c->d_level);
@@ -271,8 +256,7 @@ void free_all(ftr_ctx* c) {
     dfree(c->d_rowmm);
     dfree(c->d_mc_word);
     dfree(c->d_mc_off);
-    if (c->h_mc_tot) cudaFreeHost(c->h_mc_tot);
-    if (c->h_flags) cudaFreeHost(c->h_flags);
+    if (c->h_page) cudaFreeHost(c->h_page);
     dfree(c->d_mc_nodes);
     dfree(c->d_verts);
     dfree(c->d_vnrm);
@@ -367,16 +351,18 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
         delete c;                                           \
         return FTR_ENOMEM;                                  \
     }
-    ALLOC(c->d_dropped, 1);
-    ALLOC(c->d_npts, 1);
-    ALLOC(c->d_wild, 1);
-    ALLOC(c->d_brick_cnt, c->n_bricks);
+    // what ftr_reset clears, in one block and one memset: the brick counts, the
+    // point count, the dropped points and the wild flags (n_bricks is even)
+    ALLOC(c->d_brick_cnt, c->n_bricks + 6);
+    c->d_npts = reinterpret_cast<int64_t*>(c->d_brick_cnt + c->n_bricks);
+    c->d_dropped = reinterpret_cast<unsigned long long*>(c->d_npts + 1);
+    c->d_wild = reinterpret_cast<int*>(c->d_dropped + 1);
+    c->reset_bytes = sizeof(int) * ((size_t)c->n_bricks + 6);
     ALLOC(c->d_brick_off, c->n_bricks + 1);
     ALLOC(c->d_brick_cursor, c->n_bricks);
     ALLOC(c->d_brick_slot, c->n_bricks);
     ALLOC(c->d_active, c->n_bricks);
     ALLOC(c->d_meta, kMetaInts);
-    ALLOC(c->d_kerr, 1);
     ALLOC(c->d_tile, (c->n_bricks + kBrickScanTile - 1) / kBrickScanTile + 1);
     ALLOC(c->d_unit_off, c->n_bricks + 1);
     ALLOC(c->d_heavy_idx, c->n_bricks);
@@ -401,12 +387,18 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
     ALLOC(c->d_mc_off, 3 * (c->mc_blocks + 1) + 3);
     ALLOC(c->d_rowmm, c->mc_blocks);
 #undef ALLOC
-    if ((e = cudaMallocHost((void**)&c->h_mc_tot, 4 * sizeof(int))) != cudaSuccess ||
-        (e = cudaMallocHost((void**)&c->h_flags, 2 * sizeof(int))) != cudaSuccess) {
+    // results that kernels write straight into page-locked memory, so that no
+    // copy follows them: the level, the mesh totals and the wait flags
+    if ((e = cudaMallocHost((void**)&c->h_page, 64)) != cudaSuccess) {
         free_all(c);
         delete c;
         return FTR_ENOMEM;
     }
+    memset(c->h_page, 0, 64);
+    c->h_level = reinterpret_cast<double*>(c->h_page);
+    c->h_mc_tot = reinterpret_cast<int*>(c->h_page) + 4;
+    c->h_flags = reinterpret_cast<int*>(c->h_page) + 8;
+    c->d_kerr = c->h_flags + 1;
     // W_n^m of each axis, computed on the device in float64
     for (int a = 0; a < 3; ++a) {
         if ((e = launch_axis_twiddles(c->d_tw[a], grid_n[a], c->stream)) != cudaSuccess) {
@@ -416,14 +408,15 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
         }
     }
     if (prm.precision != FTR_PREC_FP32) {
-        if ((e = dalloc(&c->d_tc_table, tc_table_bytes())) != cudaSuccess || (e = dalloc(&c->d_tc_err, 1)) != cudaSuccess) {
+        if ((e = dalloc(&c->d_tc_table, tc_table_bytes())) != cudaSuccess) {
             free_all(c);
             delete c;
             return FTR_ENOMEM;
         }
+        c->d_tc_err = c->h_flags;
         // the split DFT matrices, built on the device from float64 cos / sin
         if ((e = tc_build_table(prm.precision, c->d_tc_table, c->stream)) != cudaSuccess ||
-            (e = cudaMemset(c->d_tc_err, 0, sizeof(int))) != cudaSuccess || (e = tc_prepare(c)) != cudaSuccess) {
+            (e = tc_prepare(c)) != cudaSuccess) {
             free_all(c);
             delete c;
             return FTR_ECUDA;
@@ -439,7 +432,6 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
         cudaEventCreate(&c->ev_start[s]);
         cudaEventCreate(&c->ev_stop[s]);
     }
-    cudaMemsetAsync(c->d_dropped, 0, sizeof(unsigned long long), c->stream);
     // every brick empty (slot -1) until the first splat: the x passes read
     // this table, also when ftr_autotune times the transforms before any frame
     cudaMemsetAsync(c->d_brick_slot, 0xff, sizeof(int) * c->n_bricks, c->stream);
@@ -448,12 +440,8 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
         const int meta0[kMetaInts] = {0, 0, 0, -1};   // and no live rows
         cudaMemcpyAsync(c->d_meta, meta0, sizeof(meta0), cudaMemcpyHostToDevice, c->stream);
     }
-    cudaMemsetAsync(c->d_wild, 0, sizeof(int), c->stream);
-    cudaMemsetAsync(c->d_kerr, 0, sizeof(int), c->stream);
-    c->h_flags[0] = c->h_flags[1] = 0;
     cudaMemsetAsync(c->d_ticket, 0, sizeof(unsigned), c->stream);
-    cudaMemsetAsync(c->d_npts, 0, sizeof(int64_t), c->stream);
-    cudaMemsetAsync(c->d_brick_cnt, 0, sizeof(int) * c->n_bricks, c->stream);
+    cudaMemsetAsync(c->d_brick_cnt, 0, c->reset_bytes, c->stream);
     {
         int wp = 1;
         while (wp < (c->g.n[0] + 31) / 32) wp <<= 1;
@@ -488,11 +476,8 @@ int ftr_reset(ftr_ctx* c) {
     c->v_external = false;
     c->meshed = false;
     c->n_verts = c->n_tris = 0;
-    cudaError_t e = cudaMemsetAsync(c->d_dropped, 0, sizeof(unsigned long long), c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_wild, 0, sizeof(int), c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_npts, 0, sizeof(int64_t), c->stream);
     // the ingest counts each point into the bricks its stencil overlaps
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_brick_cnt, 0, sizeof(int) * c->n_bricks, c->stream);
+    cudaError_t e = cudaMemsetAsync(c->d_brick_cnt, 0, c->reset_bytes, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "ftr_reset");
     return FTR_OK;
 }
@@ -782,12 +767,9 @@ int ftr_solve(ftr_ctx* c, double* iso_level_out) {
     if (e != cudaSuccess) return cuda_fail(c, e, "ftr_solve: level");
     c->solved = true;
     if (iso_level_out) {
-        if ((e = cudaMemcpyAsync(&c->level_host, c->d_level, sizeof(double), cudaMemcpyDeviceToHost, c->stream)) ||
-            (e = launch_flags(c)))
-            return cuda_fail(c, e, "ftr_solve: level copy");
         if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(c, e, "ftr_solve");
         if (int st = tc_check(c, "ftr_solve")) return st;
-        *iso_level_out = c->level_host;
+        *iso_level_out = *static_cast<volatile double*>(c->h_level);   // written by the level kernel
     }
     return FTR_OK;
 }
@@ -838,11 +820,10 @@ int ftr_extract_mesh(ftr_ctx* c, ftr_mesh* out) {
     // counts, offsets and the emission run back to back; the host waits once
     if ((e = launch_mc_count(c)) != cudaSuccess) return cuda_fail(c, e, "ftr_extract_mesh: count");
     if ((e = launch_mc_emit(c)) != cudaSuccess) return cuda_fail(c, e, "ftr_extract_mesh: emit");
-    if ((e = launch_mc_totals(c)) != cudaSuccess || (e = launch_flags(c)) != cudaSuccess)
-        return cuda_fail(c, e, "ftr_extract_mesh: totals");
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(c, e, "ftr_extract_mesh");
     if (int st = tc_check(c, "ftr_extract_mesh")) return st;
-    const int64_t na = c->h_mc_tot[0], nv = c->h_mc_tot[1], nt = c->h_mc_tot[2];
+    const volatile int* tot = c->h_mc_tot;
+    const int64_t na = tot[0], nv = tot[1], nt = tot[2];
     if (na > c->cap_mc_nodes || nv > c->cap_verts || nt > c->cap_tris) {
         // the buffers were too small: the kernels skipped the writes past them
         if ((e = grow_mesh(c, na, nv, nt)) != cudaSuccess) return cuda_fail(c, e, "ftr_extract_mesh: grow");
@@ -860,16 +841,26 @@ int ftr_extract_mesh(ftr_ctx* c, ftr_mesh* out) {
     return FTR_OK;
 }
 
+namespace {
+// Enqueue the copies of the mesh arrays that are asked for: one kernel when
+// every destination is device memory, else a copy per array.
+cudaError_t enqueue_mesh_copy(ftr_ctx* c, float* vertices, float* normals, int32_t* tris) {
+    const size_t vb = sizeof(float) * 3 * (size_t)c->n_verts, tb = sizeof(int32_t) * 3 * (size_t)c->n_tris;
+    const bool v = vertices && vb, n = normals && vb, t = tris && tb;
+    if ((!v || is_device_ptr(vertices)) && (!n || is_device_ptr(normals)) && (!t || is_device_ptr(tris)))
+        return launch_mesh_copy(c, v ? vertices : nullptr, n ? normals : nullptr, t ? tris : nullptr);
+    cudaError_t e = cudaSuccess;
+    if (v) e = cudaMemcpyAsync(vertices, c->d_verts, vb, cudaMemcpyDefault, c->stream);
+    if (e == cudaSuccess && n) e = cudaMemcpyAsync(normals, c->d_vnrm, vb, cudaMemcpyDefault, c->stream);
+    if (e == cudaSuccess && t) e = cudaMemcpyAsync(tris, c->d_tris, tb, cudaMemcpyDefault, c->stream);
+    return e;
+}
+}  // namespace
+
 int ftr_mesh_copy(ftr_ctx* c, float* vertices, float* normals, int32_t* tris) {
     if (!c) return FTR_EINVAL;
     if (!c->meshed) return set_err(c, FTR_ESTATE, "ftr_mesh_copy: no mesh");
-    cudaError_t e = cudaSuccess;
-    if (vertices && c->n_verts)
-        e = cudaMemcpyAsync(vertices, c->d_verts, sizeof(float) * 3 * c->n_verts, cudaMemcpyDefault, c->stream);
-    if (e == cudaSuccess && normals && c->n_verts)
-        e = cudaMemcpyAsync(normals, c->d_vnrm, sizeof(float) * 3 * c->n_verts, cudaMemcpyDefault, c->stream);
-    if (e == cudaSuccess && tris && c->n_tris)
-        e = cudaMemcpyAsync(tris, c->d_tris, sizeof(int32_t) * 3 * c->n_tris, cudaMemcpyDefault, c->stream);
+    cudaError_t e = enqueue_mesh_copy(c, vertices, normals, tris);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "ftr_mesh_copy");
     return FTR_OK;
@@ -878,13 +869,7 @@ int ftr_mesh_copy(ftr_ctx* c, float* vertices, float* normals, int32_t* tris) {
 int ftr_mesh_copy_async(ftr_ctx* c, float* vertices, float* normals, int32_t* tris) {
     if (!c) return FTR_EINVAL;
     if (!c->meshed) return set_err(c, FTR_ESTATE, "ftr_mesh_copy_async: no mesh");
-    cudaError_t e = cudaSuccess;
-    if (vertices && c->n_verts)
-        e = cudaMemcpyAsync(vertices, c->d_verts, sizeof(float) * 3 * c->n_verts, cudaMemcpyDefault, c->stream);
-    if (e == cudaSuccess && normals && c->n_verts)
-        e = cudaMemcpyAsync(normals, c->d_vnrm, sizeof(float) * 3 * c->n_verts, cudaMemcpyDefault, c->stream);
-    if (e == cudaSuccess && tris && c->n_tris)
-        e = cudaMemcpyAsync(tris, c->d_tris, sizeof(int32_t) * 3 * c->n_tris, cudaMemcpyDefault, c->stream);
+    cudaError_t e = enqueue_mesh_copy(c, vertices, normals, tris);
     if (e != cudaSuccess) return cuda_fail(c, e, "ftr_mesh_copy_async");
     return FTR_OK;
 }
@@ -1031,8 +1016,7 @@ cudaError_t enqueue_frame(ftr_ctx* c, const ViewSet& vs, float tol, const ftr_te
                                    out.rgb, out.textured);
         if (e != cudaSuccess) return e;
     }
-    if ((e = launch_mc_totals(c)) != cudaSuccess) return e;
-    return launch_flags(c);
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -1183,8 +1167,6 @@ int ftr_extract_mesh_async(ftr_ctx* c) {
     }
     if ((e = launch_mc_count(c)) != cudaSuccess) return cuda_fail(c, e, "ftr_extract_mesh_async: count");
     if ((e = launch_mc_emit(c)) != cudaSuccess) return cuda_fail(c, e, "ftr_extract_mesh_async: emit");
-    if ((e = launch_mc_totals(c)) != cudaSuccess || (e = launch_flags(c)) != cudaSuccess)
-        return cuda_fail(c, e, "ftr_extract_mesh_async: totals");
     c->meshed = false;
     c->mesh_pending = true;
     c->tex_pending = false;
@@ -1254,7 +1236,8 @@ int ftr_frame_finish(ftr_ctx* c, ftr_mesh* out) {
         c->tex_pending = false;
         return st;
     }
-    const int64_t na = c->h_mc_tot[0], nv = c->h_mc_tot[1], nt = c->h_mc_tot[2];
+    const volatile int* tot = c->h_mc_tot;
+    const int64_t na = tot[0], nv = tot[1], nt = tot[2];
     if (na > c->cap_mc_nodes || nv > c->cap_verts || nt > c->cap_tris) {
         if ((e = grow_mesh(c, na, nv, nt)) != cudaSuccess) return cuda_fail(c, e, "ftr_frame_finish: grow");
         if ((e = launch_mc_emit(c)) != cudaSuccess) return cuda_fail(c, e, "ftr_frame_finish: emit");
@@ -1842,8 +1825,8 @@ int ftr_debug_raise_wait_flag(ftr_ctx* c, int which) {
     if (!c) return FTR_EINVAL;
     int* flag = which == 0 ? c->d_tc_err : (which == 1 ? c->d_kerr : nullptr);
     if (!flag) return set_err(c, FTR_EINVAL, "ftr_debug_raise_wait_flag: no flag %d on this context", which);
-    // the flag's lowest byte to 1: the value a kernel writes when a bounded wait gives up
-    cudaError_t e = cudaMemsetAsync(flag, 1, 1, c->stream);
+    // as a kernel does when a bounded wait gives up
+    cudaError_t e = launch_raise_flag(c, flag);
     if (e != cudaSuccess) return cuda_fail(c, e, "ftr_debug_raise_wait_flag");
     return FTR_OK;
 }

@@ -117,7 +117,8 @@ struct ftr_ctx {
 
     // splat bricks
     int n_bricks = 0;
-    int* d_brick_cnt = nullptr;
+    int* d_brick_cnt = nullptr;   // first of the block that ftr_reset clears (d_npts, d_dropped, d_wild follow)
+    size_t reset_bytes = 0;
     int* d_brick_off = nullptr;
     int* d_brick_cursor = nullptr;
     int* d_brick_slot = nullptr;
@@ -152,8 +153,8 @@ struct ftr_ctx {
     int* d_yz_sync = nullptr;              // its ticket and per-k_x tile counters
     int* occ_query = nullptr;              // set: the pass launchers report occupancy instead of launching
     unsigned char* d_tc_table = nullptr;   // split DFT matrices of the tensor-core passes
-    int* d_tc_err = nullptr;               // set when a tensor-core completion wait gave up
-    int* d_kerr = nullptr;                 // set when a bulk-copy completion wait gave up
+    int* d_tc_err = nullptr;               // set when a tensor-core completion wait gave up (in h_flags)
+    int* d_kerr = nullptr;                 // set when a bulk-copy completion wait gave up (in h_flags)
 
     // raw reconstruction scratch (ftr_splat_depth)
     float* d_raw = nullptr;                // 7 floats per pixel capacity: P (3), N (3), W
@@ -171,7 +172,6 @@ struct ftr_ctx {
     int level_blocks = 0;
     bool solved = false;
     bool v_external = false;   // V was set with ftr_set_field_V: solve skips the splat
-    double level_host = 0.0;
 
     // marching cubes
     int mc_blocks = 0;             // grid rows n_y n_z
@@ -183,8 +183,10 @@ struct ftr_ctx {
     bool rowmm_valid = false;      // d_rowmm belongs to the current A (the fp32 five-pass x inverse wrote it)
     int* d_mc_off = nullptr;       // 3 x (mc_blocks + 1)
     int2* d_mc_word = nullptr;     // per (row, 32-node word) of a tile with surface: first record index, active mask
-    int* h_mc_tot = nullptr;       // pinned: totals (active, verts, tris)
-    int* h_flags = nullptr;        // pinned: the device wait flags (tensor-core, bulk copy) of the last frame
+    void* h_page = nullptr;        // page-locked block of what kernels report to the host:
+    double* h_level = nullptr;     //   the level of the last solve
+    int* h_mc_tot = nullptr;       //   totals of the last mesh (active, verts, tris)
+    int* h_flags = nullptr;        //   the wait flags (tensor-core, bulk copy), raised by the kernels
     int4* d_mc_nodes = nullptr;
     int64_t cap_mc_nodes = 0;
     float* d_verts = nullptr;
@@ -336,8 +338,8 @@ int mc_words_per_row(int nx);                  // padded words per grid row of t
 bool mc_plan_valid(int tile, int tris_per_sm);
 cudaError_t launch_mc_count(ftr_ctx* c);       // inside bits, then tile and group counts
 cudaError_t launch_mc_emit(ftr_ctx* c);        // offsets and node records, then vertices and triangles
-cudaError_t launch_mc_totals(ftr_ctx* c);      // totals (active, verts, tris) to h_mc_tot
-cudaError_t launch_flags(ftr_ctx* c);          // device wait flags to h_flags (api.cu)
+cudaError_t launch_mesh_copy(ftr_ctx* c, float* verts, float* nrm, int32_t* tris);   // to device buffers (null: not)
+cudaError_t launch_raise_flag(ftr_ctx* c, int* flag);
 cudaError_t launch_mc_classes(ftr_ctx* c, uint8_t* out_dev);
 cudaError_t launch_dense_V(ftr_ctx* c, float* out_dev);
 cudaError_t launch_load_dense_V(ftr_ctx* c, const float* V_dev);

@@ -35,7 +35,8 @@ __global__ void __launch_bounds__(kThreads) k_level_partial(GridDev g, const int
                                                             const float4* __restrict__ pfrac,
                                                             const int64_t* __restrict__ npts,
                                                             const float* __restrict__ A, double* part,
-                                                            unsigned* ticket, double* level, float* levelf) {
+                                                            unsigned* ticket, double* level, float* levelf,
+                                                            double* host_level) {
     pdl_wait();
     __shared__ double sh[kThreads / 32];
     __shared__ bool last;
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(kThreads) k_level_partial(GridDev g, const int
         const double L = tc > 0.0 ? ts / tc : 0.0;
         level[0] = L;
         level[1] = tc;
+        *host_level = L;                     // page-locked: no copy follows
         levelf[0] = __double2float_ru(L);   // A >= L (float64) <=> A >= levelf[0] for float32 A
         levelf[1] = __double2float_rn(L);
         *ticket = 0u;                        // ready for the next launch
@@ -95,7 +97,7 @@ __global__ void __launch_bounds__(kThreads) k_level_partial(GridDev g, const int
 cudaError_t launch_level(ftr_ctx* c) {
     launch_pdl(k_level_partial, c->level_blocks, kThreads, 0, c->stream, c->g, c->pts.base, c->pts.frac, c->d_npts, c->d_A,
                                                                  c->d_level_part, c->d_ticket, c->d_level,
-                                                                 c->d_levelf);
+                                                                 c->d_levelf, c->h_level);
     c->launches++;
     return cudaGetLastError();
 }

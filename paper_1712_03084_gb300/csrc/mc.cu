@@ -288,7 +288,8 @@ __global__ void __launch_bounds__(T) k_mc_emit_tiles(GridDev g, const unsigned* 
                                                               const int4* __restrict__ agg,
                                                               const int4* __restrict__ sup, int* __restrict__ off,
                                                               int4* __restrict__ nodes, int cap_nodes,
-                                                              int2* __restrict__ wordinfo) {
+                                                              int2* __restrict__ wordinfo,
+                                                              int* __restrict__ host_totals) {
     pdl_wait();
     __shared__ unsigned char s_ntri[256];
     __shared__ int3 sh[T / 32];
@@ -335,9 +336,12 @@ __global__ void __launch_bounds__(T) k_mc_emit_tiles(GridDev g, const unsigned* 
         off[nrows] = all.x;
         off[(nrows + 1) + nrows] = all.y;
         off[2 * (nrows + 1) + nrows] = all.z;
-        off[3 * (nrows + 1) + 0] = all.x;     // totals for the host
-        off[3 * (nrows + 1) + 1] = all.y;
+        off[3 * (nrows + 1) + 0] = all.x;     // totals for the kernels that follow and, in
+        off[3 * (nrows + 1) + 1] = all.y;     // page-locked memory, for the host
         off[3 * (nrows + 1) + 2] = all.z;
+        host_totals[0] = all.x;
+        host_totals[1] = all.y;
+        host_totals[2] = all.z;
     }
     // the word's first record and its active nodes: the triangle pass finds
     // a corner's owner record from these without scanning the row
@@ -469,6 +473,31 @@ __global__ void __launch_bounds__(256) k_mc_tris(GridDev g, const float* __restr
     }
 }
 
+// n words from src to dst, 16 bytes at a time where both allow it.
+__device__ __forceinline__ void copy_words(const uint32_t* __restrict__ src, uint32_t* __restrict__ dst, int64_t n) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    int64_t done = 0;
+    if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
+        const uint4* s = reinterpret_cast<const uint4*>(src);
+        uint4* d = reinterpret_cast<uint4*>(dst);
+        for (int64_t i = t; i < n / 4; i += step) d[i] = s[i];
+        done = n / 4 * 4;
+    }
+    for (int64_t i = done + t; i < n; i += step) dst[i] = src[i];
+}
+
+// The mesh arrays into caller-owned device buffers: one launch where three
+// device copies cost 2-3 us each.
+__global__ void __launch_bounds__(256) k_mesh_copy(const float* __restrict__ v, const float* __restrict__ nrm,
+                                                   const int32_t* __restrict__ tris, int64_t nv, int64_t nt,
+                                                   float* vo, float* no, int32_t* to) {
+    if (vo) copy_words(reinterpret_cast<const uint32_t*>(v), reinterpret_cast<uint32_t*>(vo), 3 * nv);
+    if (no) copy_words(reinterpret_cast<const uint32_t*>(nrm), reinterpret_cast<uint32_t*>(no), 3 * nv);
+    if (to) copy_words(reinterpret_cast<const uint32_t*>(tris), reinterpret_cast<uint32_t*>(to), 3 * nt);
+}
+
+__global__ void k_raise_flag(int* flag) { atomicExch(flag, 1); }
+
 __global__ void k_mc_classes(GridDev g, const float* __restrict__ A, const float* __restrict__ levelf,
                              uint8_t* out) {
     const int cx = g.n[0] - 1, cy = g.n[1] - 1, cz = g.n[2] - 1;
@@ -564,15 +593,6 @@ cudaError_t launch_mc_count(ftr_ctx* c) {
     return e;
 }
 
-// The three totals (active nodes, vertices, triangles) into pinned host
-// memory; enqueued after the frame's last kernel so that no copy sits between
-// two kernels of the frame.
-cudaError_t launch_mc_totals(ftr_ctx* c) {
-    const int nr = c->mc_blocks;
-    return cudaMemcpyAsync(c->h_mc_tot, c->d_mc_off + 3 * (nr + 1), 3 * sizeof(int), cudaMemcpyDeviceToHost,
-                           c->stream);
-}
-
 // The rows' offsets and the node records, then the vertices and triangles.
 cudaError_t launch_mc_emit(ftr_ctx* c) {
     const int nr = c->mc_blocks;
@@ -582,7 +602,7 @@ cudaError_t launch_mc_emit(ftr_ctx* c) {
     const int4* sup = reinterpret_cast<const int4*>(c->d_mc_blk + 4 * ntiles);
     prof_begin(c, ST_MC_EMIT);
     launch_tiles<EmitK>(c->mc_tile, ntiles, c->stream, c->g, (const unsigned*)c->d_mc_bits, nr, wp, ntiles, agg, sup,
-                        c->d_mc_off, c->d_mc_nodes, (int)c->cap_mc_nodes, c->d_mc_word);
+                        c->d_mc_off, c->d_mc_nodes, (int)c->cap_mc_nodes, c->d_mc_word, c->h_mc_tot);
     c->launches++;
     cudaError_t e = cudaGetLastError();
     prof_end(c, ST_MC_EMIT);
@@ -597,6 +617,22 @@ cudaError_t launch_mc_emit(ftr_ctx* c) {
     e = cudaGetLastError();
     prof_end(c, ST_MC_TRIS);
     return e;
+}
+
+cudaError_t launch_mesh_copy(ftr_ctx* c, float* verts, float* nrm, int32_t* tris) {
+    if (!verts && !nrm && !tris) return cudaSuccess;
+    const int64_t words = 3 * (c->n_verts > c->n_tris ? c->n_verts : c->n_tris);
+    const int64_t blocks = (words / 4 + 255) / 256;
+    k_mesh_copy<<<(unsigned)(blocks < 1 ? 1 : (blocks > 152 * 8 ? 152 * 8 : blocks)), 256, 0, c->stream>>>(
+        c->d_verts, c->d_vnrm, c->d_tris, c->n_verts, c->n_tris, verts, nrm, tris);
+    c->launches++;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_raise_flag(ftr_ctx* c, int* flag) {
+    k_raise_flag<<<1, 1, 0, c->stream>>>(flag);
+    c->launches++;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_mc_classes(ftr_ctx* c, uint8_t* out_dev) {
