@@ -255,7 +255,8 @@ void free_all(ftr_ctx* c) {
     dfree(c->d_mc_bits);
     dfree(c->d_rowmm);
     dfree(c->d_mc_word);
-    dfree(c->d_mc_off);
+    dfree(c->d_mc_cls);
+    dfree(c->d_mc_tot);
     if (c->h_page) cudaFreeHost(c->h_page);
     dfree(c->d_mc_nodes);
     dfree(c->d_verts);
@@ -384,7 +385,8 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
         ALLOC(c->d_mc_bits, (size_t)c->mc_blocks * wp);
         ALLOC(c->d_mc_word, (size_t)c->mc_blocks * wp);
     }
-    ALLOC(c->d_mc_off, 3 * (c->mc_blocks + 1) + 3);
+    ALLOC(c->d_mc_cls, c->mc_blocks);
+    ALLOC(c->d_mc_tot, 4);
     ALLOC(c->d_rowmm, c->mc_blocks);
 #undef ALLOC
     // results that kernels write straight into page-locked memory, so that no
@@ -1012,7 +1014,7 @@ cudaError_t enqueue_frame(ftr_ctx* c, const ViewSet& vs, float tol, const ftr_te
     if ((e = launch_mc_emit(c)) != cudaSuccess) return e;
     if (vs.k > 0) {
         const int64_t limit = out_capacity < c->cap_verts ? out_capacity : c->cap_verts;
-        e = launch_texture_bounded(c, vs, tol, limit, c->d_mc_off + 3 * (c->mc_blocks + 1) + 1, out.weights, out.uv,
+        e = launch_texture_bounded(c, vs, tol, limit, c->d_mc_tot + 1, out.weights, out.uv,
                                    out.rgb, out.textured);
         if (e != cudaSuccess) return e;
     }
@@ -1210,9 +1212,8 @@ int ftr_texture_async(ftr_ctx* c, const ftr_view* views, int k, float depth_tol,
     for (int i = 0; i < 4; ++i)
         if (outs[i] && !is_device_ptr(outs[i]))
             return set_err(c, FTR_EINVAL, "ftr_texture_async: outputs must be device memory");
-    const int nr = c->mc_blocks;
     const int64_t limit = out_capacity < c->cap_verts ? out_capacity : c->cap_verts;
-    cudaError_t e = launch_texture_bounded(c, vs, depth_tol, limit, c->d_mc_off + 3 * (nr + 1) + 1, out->weights,
+    cudaError_t e = launch_texture_bounded(c, vs, depth_tol, limit, c->d_mc_tot + 1, out->weights,
                                            out->uv, out->rgb, out->textured);
     if (e != cudaSuccess) return cuda_fail(c, e, "ftr_texture_async");
     c->tex_pending = true;
@@ -1612,7 +1613,7 @@ int64_t context_bytes(const int n[3], const Caps& k) {
     if (k.yz) b += (int64_t)(yz_ring_elems(n) * sizeof(float2)) + (int64_t)yz_sync_ints(n) * (int64_t)sizeof(int);
     b += k.raw * 7 * (int64_t)sizeof(float) + k.raw_tiles * (int64_t)sizeof(int);
     b += (2 * level_blocks + 8) * (int64_t)sizeof(double);
-    b += (6 * mc_blocks + 16) * (int64_t)sizeof(int);
+    b += (3 * mc_blocks + 16) * (int64_t)sizeof(int) + mc_blocks;   // tile and group sums, row classes
     b += mc_blocks * 16 * (int64_t)sizeof(unsigned);   // inside bits (upper bound)
     b += mc_blocks * (int64_t)sizeof(float2);          // row min / max of A
     b += mc_blocks * 16 * (int64_t)sizeof(int2);       // per-word record index and mask (upper bound)

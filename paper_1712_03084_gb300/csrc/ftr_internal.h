@@ -178,10 +178,11 @@ struct ftr_ctx {
     int mc_tile = 256;             // (row, word) threads per tile of the count and emit passes: 128, 256, 512
     int mc_tris_per_sm = 4;        // CTAs per SM of the triangle pass (256 threads each, grid stride)
     int* d_mc_blk = nullptr;       // 3 x mc_blocks ints: tile and group sums of the marching-cubes count
-    unsigned* d_mc_bits = nullptr; // inside bits, 32 nodes per word, rows padded to a power-of-two word count
+    unsigned* d_mc_bits = nullptr; // inside bits of the mixed rows, 32 nodes per word, rows padded to a power-of-two word count
     float2* d_rowmm = nullptr;     // per grid row (y + n_y z): min and max of A, written with A by the x inverse
     bool rowmm_valid = false;      // d_rowmm belongs to the current A (the fp32 five-pass x inverse wrote it)
-    int* d_mc_off = nullptr;       // 3 x (mc_blocks + 1)
+    unsigned char* d_mc_cls = nullptr;   // per grid row: all outside (0), all inside (1), mixed (2)
+    int* d_mc_tot = nullptr;       // totals of the last mesh (active, verts, tris)
     int2* d_mc_word = nullptr;     // per (row, 32-node word) of a tile with surface: first record index, active mask
     void* h_page = nullptr;        // page-locked block of what kernels report to the host:
     double* h_level = nullptr;     //   the level of the last solve

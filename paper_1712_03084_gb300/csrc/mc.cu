@@ -14,16 +14,16 @@
 // the rows (y+1, z), (y, z+1), (y+1, z+1); XORs give the crossing edges
 // toward +x, +y, +z and AND/OR of the eight corner masks the cells whose
 // corners differ (exactly the cells with triangles).  Launches:
-//   bits   the inside bits of every node
+//   bits   a class per grid row (outside, inside, mixed) and the inside bits
+//          of the mixed rows
 //   count  per tile of (row, word) threads: active nodes (owning a vertex
 //          or lower corner of a cell with triangles), vertices, triangles;
 //          also summed per group of 256 tiles
-//   emit   per tile: its offset from the group and tile sums before it, a
-//          CTA scan of its counts, the rows' offsets, per active node in x
+//   emit   per tile with an active node: its offset from the group and tile
+//          sums before it, a CTA scan of its counts, per active node in x
 //          order one 16-byte record (node, edge bits | class << 8, first
 //          vertex, first triangle), and per word with active nodes its first
-//          record index and active mask (a tile with no active node writes
-//          only its rows' offsets)
+//          record index and active mask
 //   tris   one thread per active node: the vertices of its crossing edges
 //          (t = (L - A0)/(A1 - A0), normal -grad A by central differences,
 //          one-sided at the border, lerped), then its triangles' corners
@@ -69,43 +69,52 @@ __device__ __forceinline__ NodeInfo classify_node(const float* __restrict__ A, i
     return r;
 }
 
-constexpr int kRowsPerCta = kMcThreads / 32;
-
 __device__ __forceinline__ int ntri_of(int cls) { return (cls == 0 || cls == 255) ? 0 : c_ntri[cls]; }
 
 // ---------------------------------------------------------------- bit masks
 // The inside bits (A >= L) of every node, 32 per word: word w of grid row r
 // (y + n_y z) holds x = 32 w .. 32 w + 31 (bit i = node 32 w + i; zero past
 // n_x); rows are `wp` words apart (wp = the words per row rounded up to a
-// power of two).  One warp per row, one ballot per word.
+// power of two).  Per row a class: every node outside (0), every node inside
+// (1) or mixed (2).  Most rows of a grid are not mixed; their words are neither
+// computed nor (unless `all`) written, and the passes below take them from the
+// class.
+// rowmm (nullable): per row the minimum and maximum of A, from which a row
+// whose maximum is below the level, or whose minimum is at or above it, gets
+// its class without reading A (the same bits: every node of the row decides
+// alike); else the class comes from the words.
 // It also zeroes `zero[0 .. nzero)` (the group sums of k_mc_count_tiles).
-// rowmm (nullable): per row the minimum and maximum of A; a row whose maximum
-// is below the level, or whose minimum is at or above it, gets its words
-// without reading A (the same bits: every node of the row decides alike).
+constexpr int kOutside = 0, kInside = 1, kMixed = 2;
+constexpr int kBitRows = 4;          // grid rows per warp: a quarter of the CTAs for rows that end at their class
+
+// Nodes of word w that exist.
+__device__ __forceinline__ unsigned word_valid(int nx, int w) {
+    const int left = nx - 32 * w;
+    return left >= 32 ? 0xffffffffu : (left <= 0 ? 0u : (1u << left) - 1u);
+}
+
 __global__ void __launch_bounds__(kMcThreads) k_mc_bits(GridDev g, const float* __restrict__ A,
                                                         const float* __restrict__ levelf, unsigned* __restrict__ bits,
-                                                        int nrows, int wp, int* __restrict__ zero, int nzero,
-                                                        const float2* __restrict__ rowmm) {
+                                                        unsigned char* __restrict__ cls, int nrows, int wp,
+                                                        int* __restrict__ zero, int nzero,
+                                                        const float2* __restrict__ rowmm, int all) {
     pdl_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nzero; i += gridDim.x * blockDim.x) zero[i] = 0;
     const int lane = threadIdx.x & 31;
     const float L = levelf[0];
     const int nx = g.n[0];
     const int nw = (nx + 31) >> 5;
-    // one warp per row (warp-uniform); the stride covers any grid size
-    for (int row = blockIdx.x * kRowsPerCta + (threadIdx.x >> 5); row < nrows; row += gridDim.x * kRowsPerCta) {
-        const float* a = A + (int64_t)row * nx;
-        if (rowmm) {
-            const float2 mm = rowmm[row];
-            if (mm.y < L || mm.x >= L) {            // false for NaN bounds
-                if (lane < wp) {
-                    unsigned word = 0u;
-                    if (lane < nw && mm.x >= L) word = (32 * (lane + 1) <= nx) ? 0xffffffffu : ((1u << (nx - 32 * lane)) - 1u);
-                    bits[(int64_t)row * wp + lane] = word;
-                }
-                continue;
-            }
-        }
+    const int row0 = (blockIdx.x * (kMcThreads / 32) + (threadIdx.x >> 5)) * kBitRows;
+    if (row0 >= nrows) return;                  // warp-uniform; nrows is a multiple of kBitRows
+    int c = kMixed;
+    if (rowmm && lane < kBitRows) {
+        const float2 mm = rowmm[row0 + lane];
+        c = mm.y < L ? kOutside : (mm.x >= L ? kInside : kMixed);   // mixed for NaN bounds
+    }
+    const unsigned mixed = rowmm ? __ballot_sync(0xffffffffu, lane < kBitRows && c == kMixed) : (1u << kBitRows) - 1u;
+    for (unsigned m = mixed; m; m &= m - 1) {
+        const int r = __ffs(m) - 1;
+        const float* a = A + (int64_t)(row0 + r) * nx;
         unsigned mine = 0u;
         // up to 8 words per batch: all loads are issued before the first ballot
         for (int w0 = 0; w0 < nw; w0 += 8) {
@@ -113,7 +122,7 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_bits(GridDev g, const float* 
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
                 const int x = 32 * (w0 + k) + lane;
-                v[k] = (w0 + k < nw && x < nx) ? a[x] : -INFINITY;
+                v[k] = x < nx ? a[x] : -INFINITY;
             }
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
@@ -121,7 +130,21 @@ __global__ void __launch_bounds__(kMcThreads) k_mc_bits(GridDev g, const float* 
                 if (lane == w0 + k) mine = b;
             }
         }
-        if (lane < wp) bits[(int64_t)row * wp + lane] = lane < nw ? mine : 0u;
+        const unsigned valid = word_valid(nx, lane);
+        mine &= valid;
+        if (!rowmm) {
+            const bool some = __any_sync(0xffffffffu, mine != 0u), every = __all_sync(0xffffffffu, mine == valid);
+            if (lane == r) c = !some ? kOutside : (every ? kInside : kMixed);
+        }
+        if (lane < wp) bits[(int64_t)(row0 + r) * wp + lane] = mine;
+    }
+    if (lane < kBitRows) cls[row0 + lane] = (unsigned char)c;
+    if (all && rowmm) {
+        for (int r = 0; r < kBitRows; ++r) {
+            const int rc = __shfl_sync(0xffffffffu, c, r);
+            if (rc != kMixed && lane < wp)
+                bits[(int64_t)(row0 + r) * wp + lane] = rc == kInside ? word_valid(nx, lane) : 0u;
+        }
     }
 }
 
@@ -134,17 +157,38 @@ struct WordMasks {
     unsigned c[8];   // corner bits of the cells whose lower corner is in the word
 };
 
-__device__ __forceinline__ WordMasks word_masks(const unsigned* __restrict__ bits, int row, int w, int nw, int wp,
-                                                int x_count, bool hy, bool hz, int ny) {
+// Classes of the row, of its +y, +z and +y+z neighbours (the row's own where
+// the grid ends), and whether a surface can pass between them.
+struct RowClasses {
+    int c00, c10, c01, c11;
+    bool live;
+};
+
+__device__ __forceinline__ RowClasses row_classes(const unsigned char* __restrict__ cls, int row, bool hy, bool hz,
+                                                  int ny) {
+    RowClasses r;
+    r.c00 = cls[row];
+    r.c10 = hy ? cls[row + 1] : r.c00;
+    r.c01 = hz ? cls[row + ny] : r.c00;
+    r.c11 = hy && hz ? cls[row + ny + 1] : r.c00;
+    const int any = r.c00 | r.c10 | r.c01 | r.c11;
+    r.live = any > kInside || (any != r.c00 || r.c00 != r.c10 || r.c00 != r.c01 || r.c00 != r.c11);
+    return r;
+}
+
+__device__ __forceinline__ WordMasks word_masks(const unsigned* __restrict__ bits, const RowClasses& rc, int row, int w,
+                                                int nw, int wp, int x_count, bool hy, bool hz, int ny) {
     const int64_t r00 = (int64_t)row * wp, r10 = r00 + wp, r01 = r00 + (int64_t)ny * wp, r11 = r01 + wp;
     const bool more = w + 1 < nw;
-    const unsigned b00 = bits[r00 + w], n00 = more ? bits[r00 + w + 1] : 0u;
-    const unsigned b10 = hy ? bits[r10 + w] : 0u, n10 = (hy && more) ? bits[r10 + w + 1] : 0u;
-    const unsigned b01 = hz ? bits[r01 + w] : 0u, n01 = (hz && more) ? bits[r01 + w + 1] : 0u;
-    const unsigned b11 = (hy && hz) ? bits[r11 + w] : 0u, n11 = (hy && hz && more) ? bits[r11 + w + 1] : 0u;
-    // nodes of the word that exist, and those with a +x neighbour
+    // nodes of the word (and of the next) that exist, and those with a +x neighbour
     const int base = 32 * w;
-    const unsigned valid = x_count - base >= 32 ? 0xffffffffu : ((1u << (x_count - base)) - 1u);
+    const unsigned valid = word_valid(x_count, w), nvalid = word_valid(x_count, w + 1);
+    auto word = [&](int c, int64_t r) { return c == kMixed ? bits[r + w] : (c == kInside ? valid : 0u); };
+    auto next = [&](int c, int64_t r) { return !more ? 0u : (c == kMixed ? bits[r + w + 1] : (c == kInside ? nvalid : 0u)); };
+    const unsigned b00 = word(rc.c00, r00), n00 = next(rc.c00, r00);
+    const unsigned b10 = hy ? word(rc.c10, r10) : 0u, n10 = hy ? next(rc.c10, r10) : 0u;
+    const unsigned b01 = hz ? word(rc.c01, r01) : 0u, n01 = hz ? next(rc.c01, r01) : 0u;
+    const unsigned b11 = (hy && hz) ? word(rc.c11, r11) : 0u, n11 = (hy && hz) ? next(rc.c11, r11) : 0u;
     const unsigned vx = x_count - 1 - base >= 32 ? 0xffffffffu
                         : (x_count - 1 - base <= 0 ? 0u : ((1u << (x_count - 1 - base)) - 1u));
     WordMasks m;
@@ -224,7 +268,7 @@ __device__ __forceinline__ int3 block_scan3(int3 v, int3& total, int3* sh) {
 // per group; integer atomics, so the order does not matter).  The emit
 // kernel's tile gets its offset from the groups before it and the tiles
 // before it in its group (at most 255 + a few loads, spread over the CTA),
-// scans its own counts, and writes its rows' offsets and its node records.
+// scans its own counts, and writes its node records.
 //
 // Tile state (agg) and group sums (sup, zeroed by k_mc_bits) as int4: active
 // nodes, vertices, triangles, unused.
@@ -234,17 +278,17 @@ struct WordCounts {
     int3 c;
 };
 
-__device__ __forceinline__ WordCounts word_counts(const GridDev& g, const unsigned* __restrict__ bits, int64_t t,
-                                                  int nrows, int wp, const unsigned char* s_ntri) {
+__device__ __forceinline__ WordCounts word_counts(const GridDev& g, const unsigned* __restrict__ bits,
+                                                  const RowClasses& rc, int row, int w, int wp,
+                                                  const unsigned char* s_ntri) {
     WordCounts r;
     r.act = 0u;
     r.c = make_int3(0, 0, 0);
-    const int row = (int)(t / wp), w = (int)(t % wp);
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const int nw = (nx + 31) >> 5;
-    if (row < nrows && w < nw) {
+    if (rc.live && w < nw) {
         const int y = row % ny, z = row / ny;
-        r.m = word_masks(bits, row, w, nw, wp, nx, y < ny - 1, z < nz - 1, ny);
+        r.m = word_masks(bits, rc, row, w, nw, wp, nx, y < ny - 1, z < nz - 1, ny);
         r.act = r.m.ex | r.m.ey | r.m.ez | r.m.mixed;
         r.c.x = __popc(r.act);
         r.c.y = __popc(r.m.ex) + __popc(r.m.ey) + __popc(r.m.ez);
@@ -260,20 +304,39 @@ __device__ __forceinline__ WordCounts word_counts(const GridDev& g, const unsign
 
 constexpr int kMcGroup = 256;     // tiles per group sum
 
+// A tile whose rows and their neighbours are all on one side (four fifths of a
+// body's grid) ends after the row classes; 9216 tiles of a 384^3 frame: 33 us
+// when every tile read its words and scanned its counts.
 template <int T>
 __global__ void __launch_bounds__(T) k_mc_count_tiles(GridDev g, const unsigned* __restrict__ bits,
-                                                               int nrows, int wp, int4* __restrict__ agg,
-                                                               int* __restrict__ sup) {
+                                                               const unsigned char* __restrict__ cls, int nrows, int wp,
+                                                               int4* __restrict__ agg, int* __restrict__ sup) {
     pdl_wait();
     __shared__ unsigned char s_ntri[256];
-    __shared__ int3 sh[T / 32];
-    for (int k = threadIdx.x; k < 256; k += blockDim.x) s_ntri[k] = (unsigned char)c_ntri[k];
-    __syncthreads();
+    __shared__ int s_sum[3];
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const WordCounts wc = word_counts(g, bits, t, nrows, wp, s_ntri);
-    int3 tot;
-    block_scan3<T>(wc.c, tot, sh);
+    const int row = (int)(t / wp), w = (int)(t % wp);
+    RowClasses rc;
+    rc.live = false;
+    if (row < nrows) rc = row_classes(cls, row, row % g.n[1] < g.n[1] - 1, row / g.n[1] < g.n[2] - 1, g.n[1]);
+    if (!__syncthreads_or(rc.live)) {
+        if (threadIdx.x == 0) agg[blockIdx.x] = make_int4(0, 0, 0, 0);
+        return;
+    }
+    for (int k = threadIdx.x; k < 256; k += blockDim.x) s_ntri[k] = (unsigned char)c_ntri[k];
+    if (threadIdx.x < 3) s_sum[threadIdx.x] = 0;
+    __syncthreads();
+    const WordCounts wc = word_counts(g, bits, rc, row, w, wp, s_ntri);
+    const int3 sum = make_int3(__reduce_add_sync(0xffffffffu, wc.c.x), __reduce_add_sync(0xffffffffu, wc.c.y),
+                               __reduce_add_sync(0xffffffffu, wc.c.z));
+    if ((threadIdx.x & 31) == 0 && (sum.x | sum.y | sum.z)) {
+        atomicAdd(&s_sum[0], sum.x);
+        atomicAdd(&s_sum[1], sum.y);
+        atomicAdd(&s_sum[2], sum.z);
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
+        const int3 tot = make_int3(s_sum[0], s_sum[1], s_sum[2]);
         agg[blockIdx.x] = make_int4(tot.x, tot.y, tot.z, 0);
         int* s = sup + 4 * (blockIdx.x / kMcGroup);
         if (tot.x) atomicAdd(&s[0], tot.x);
@@ -284,18 +347,23 @@ __global__ void __launch_bounds__(T) k_mc_count_tiles(GridDev g, const unsigned*
 
 template <int T>
 __global__ void __launch_bounds__(T) k_mc_emit_tiles(GridDev g, const unsigned* __restrict__ bits,
-                                                              int nrows, int wp, int ntiles,
-                                                              const int4* __restrict__ agg,
-                                                              const int4* __restrict__ sup, int* __restrict__ off,
+                                                              const unsigned char* __restrict__ cls, int nrows, int wp,
+                                                              int ntiles, const int4* __restrict__ agg,
+                                                              const int4* __restrict__ sup, int* __restrict__ totals,
                                                               int4* __restrict__ nodes, int cap_nodes,
                                                               int2* __restrict__ wordinfo,
                                                               int* __restrict__ host_totals) {
     pdl_wait();
     __shared__ unsigned char s_ntri[256];
     __shared__ int3 sh[T / 32];
+    const int tile = blockIdx.x, grp = tile / kMcGroup;
+    // a tile the count found empty (most of the grid) has nothing to write; the
+    // last one reports the totals
+    const int4 mine = agg[tile];
+    const bool empty = (mine.x | mine.y | mine.z) == 0;
+    if (empty && tile != ntiles - 1) return;
     for (int k = threadIdx.x; k < 256; k += blockDim.x) s_ntri[k] = (unsigned char)c_ntri[k];
     // the sums of every tile before this one: whole groups, then this group's tiles
-    const int tile = blockIdx.x, grp = tile / kMcGroup;
     int3 pre = make_int3(0, 0, 0);
     for (int k = threadIdx.x; k < grp; k += blockDim.x) {
         const int4 v = sup[k];
@@ -312,37 +380,22 @@ __global__ void __launch_bounds__(T) k_mc_emit_tiles(GridDev g, const unsigned* 
     __syncthreads();
     int3 base;
     block_scan3<T>(pre, base, sh);
-    const int64_t t = (int64_t)tile * blockDim.x + threadIdx.x;
-    // a tile the count found empty (most of the grid) has only its rows'
-    // offsets to write
-    const int4 mine = agg[tile];
-    WordCounts wc;
-    int3 tot = make_int3(0, 0, 0), ex = make_int3(0, 0, 0);
-    if ((mine.x | mine.y | mine.z) != 0) {
-        wc = word_counts(g, bits, t, nrows, wp, s_ntri);
-        ex = block_scan3<T>(wc.c, tot, sh);
-    } else {
-        wc.act = 0u;
-    }
-    const int row = (int)(t / wp), w = (int)(t % wp);
-    int ja = base.x + ex.x, jv = base.y + ex.y, jt = base.z + ex.z;
-    if (w == 0 && row < nrows) {
-        off[row] = ja;
-        off[(nrows + 1) + row] = jv;
-        off[2 * (nrows + 1) + row] = jt;
-    }
     if (tile == ntiles - 1 && threadIdx.x == 0) {
-        const int3 all = make_int3(base.x + tot.x, base.y + tot.y, base.z + tot.z);
-        off[nrows] = all.x;
-        off[(nrows + 1) + nrows] = all.y;
-        off[2 * (nrows + 1) + nrows] = all.z;
-        off[3 * (nrows + 1) + 0] = all.x;     // totals for the kernels that follow and, in
-        off[3 * (nrows + 1) + 1] = all.y;     // page-locked memory, for the host
-        off[3 * (nrows + 1) + 2] = all.z;
-        host_totals[0] = all.x;
-        host_totals[1] = all.y;
-        host_totals[2] = all.z;
+        // totals for the kernels that follow and, in page-locked memory, for the host
+        totals[0] = host_totals[0] = base.x + mine.x;
+        totals[1] = host_totals[1] = base.y + mine.y;
+        totals[2] = host_totals[2] = base.z + mine.z;
     }
+    if (empty) return;
+    const int64_t t = (int64_t)tile * blockDim.x + threadIdx.x;
+    const int row = (int)(t / wp), w = (int)(t % wp);
+    RowClasses rc;
+    rc.live = false;
+    if (row < nrows) rc = row_classes(cls, row, row % g.n[1] < g.n[1] - 1, row / g.n[1] < g.n[2] - 1, g.n[1]);
+    const WordCounts wc = word_counts(g, bits, rc, row, w, wp, s_ntri);
+    int3 tot;
+    const int3 ex = block_scan3<T>(wc.c, tot, sh);
+    int ja = base.x + ex.x, jv = base.y + ex.y, jt = base.z + ex.z;
     // the word's first record and its active nodes: the triangle pass finds
     // a corner's owner record from these without scanning the row
     if (wc.act) wordinfo[t] = make_int2(ja, (int)wc.act);
@@ -361,102 +414,135 @@ __global__ void __launch_bounds__(T) k_mc_emit_tiles(GridDev g, const unsigned* 
     }
 }
 
-__device__ __forceinline__ float grad_axis(const float* __restrict__ A, int64_t n, int q, int nq, int64_t stride,
-                                           float inv_h) {
-    if (q == 0) return (A[n + stride] - A[n]) * inv_h;
-    if (q == nq - 1) return (A[n] - A[n - stride]) * inv_h;
-    return (A[n + stride] - A[n - stride]) * (0.5f * inv_h);
-}
-
 // Vertices on the crossing edges of node n: t = (L - A0) / (A1 - A0) and the
 // position p(q) + t h_a e_a, in float32 (no decision depends on them; the
-// error is a few float32 ulps of the coordinates), normal = -grad A lerped.
+// error is a few float32 ulps of the coordinates), normal = -grad A lerped
+// (central differences, one-sided at the border).  All reads (the node's six
+// neighbours, five more per crossing edge) are issued before the first use:
+// edge by edge they were a chain of round trips.
 __device__ __forceinline__ void emit_vertices(const GridDev& g, const float* __restrict__ A, float Ln,
                                               int64_t n, const int q[3], int flags, int vi, int cap_v,
                                               float* __restrict__ verts, float* __restrict__ vnrm) {
     const int nn[3] = {g.n[0], g.n[1], g.n[2]};
     const int64_t st[3] = {1, (int64_t)g.n[0], (int64_t)g.n[0] * g.n[1]};
-    float g0[3];
+    const float a0 = A[n];
+    float fw[3], bw[3];                     // neighbours of the node; itself where the grid ends
 #pragma unroll
-    for (int c = 0; c < 3; ++c) g0[c] = grad_axis(A, n, q[c], nn[c], st[c], g.inv_hf[c]);
+    for (int c = 0; c < 3; ++c) {
+        fw[c] = q[c] < nn[c] - 1 ? A[n + st[c]] : a0;
+        bw[c] = q[c] > 0 ? A[n - st[c]] : a0;
+    }
+    float hi[3][3], lo[3][3];               // per edge: the neighbours of its far node
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
         if (!((flags >> a) & 1)) continue;
         const int64_t n1 = n + st[a];
-        const float a0 = A[n], a1 = A[n1];
-        const float tt = (Ln - a0) / (a1 - a0);
-        int q1[3] = {q[0], q[1], q[2]};
-        q1[a] += 1;
-        float g1[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) g1[c] = grad_axis(A, n1, q1[c], nn[c], st[c], g.inv_hf[c]);
+        for (int c = 0; c < 3; ++c) {
+            const int qc = q[c] + (c == a ? 1 : 0);
+            hi[a][c] = qc < nn[c] - 1 ? A[n1 + st[c]] : fw[a];
+            lo[a][c] = c == a ? a0 : (qc > 0 ? A[n1 - st[c]] : fw[a]);
+        }
+    }
+    float g0[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        g0[c] = (fw[c] - bw[c]) * (q[c] == 0 || q[c] == nn[c] - 1 ? g.inv_hf[c] : 0.5f * g.inv_hf[c]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (!((flags >> a) & 1)) continue;
+        const float tt = (Ln - a0) / (fw[a] - a0);
         float p[3], nv[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
+            const int q1 = q[c] + (c == a ? 1 : 0);
+            const float g1 = (hi[a][c] - lo[a][c]) * (q1 == 0 || q1 == nn[c] - 1 ? g.inv_hf[c] : 0.5f * g.inv_hf[c]);
             const float qc = (float)q[c] + 0.5f + (c == a ? tt : 0.0f);
             p[c] = fmaf(qc, g.hf[c], g.bminf[c]);
-            nv[c] = -((1.0f - tt) * g0[c] + tt * g1[c]);
+            nv[c] = -__fmaf_rn(1.0f - tt, g0[c], __fmul_rn(tt, g1));
         }
-        const float len2 = nv[0] * nv[0] + nv[1] * nv[1] + nv[2] * nv[2];
+        const float len2 = __fmaf_rn(nv[2], nv[2], __fmaf_rn(nv[0], nv[0], __fmul_rn(nv[1], nv[1])));
         const float inv = len2 > 0.f ? rsqrtf(len2) : 0.f;
         if (vi >= cap_v) return;   // buffers too small: the host grows them and runs again
-        verts[3 * (int64_t)vi + 0] = p[0];
-        verts[3 * (int64_t)vi + 1] = p[1];
-        verts[3 * (int64_t)vi + 2] = p[2];
-        vnrm[3 * (int64_t)vi + 0] = nv[0] * inv;
-        vnrm[3 * (int64_t)vi + 1] = nv[1] * inv;
-        vnrm[3 * (int64_t)vi + 2] = nv[2] * inv;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            verts[3 * (int64_t)vi + c] = p[c];
+            vnrm[3 * (int64_t)vi + c] = nv[c] * inv;
+        }
         ++vi;
     }
 }
 
-// The owner of a triangle corner is this node or a node of the same row
-// (+x), of the next row (+y) or of the next plane (+z).  The owner is active
-// (it owns the crossing edge), so its word was written by the emit pass:
-// its record index is the word's first record plus the active nodes before
-// it in the word.
-__device__ __forceinline__ void tris_of_node(const GridDev& g, const int4* __restrict__ nodes, int r,
+constexpr int kTriThreads = 256;
+
+// Triangles of a node's cell.  The owner of a cube edge's vertex is the node at
+// the edge's lower end: this node or a neighbour toward +x, +y, +z.  It is
+// active (it owns the crossing edge), so its word was written by the emit pass:
+// its record index is the word's first record plus the active nodes before it
+// in the word.  The six neighbours' records are looked up together (one round
+// trip for the words, one for the records; corner by corner it was two per
+// corner), the twelve edges' vertex ids go to this thread's column of s_edge
+// and the case table picks from them.
+__device__ __forceinline__ void tris_of_node(const GridDev& g, const int4* __restrict__ nodes, const int4 rec,
                                              const int2* __restrict__ wordinfo, int wp, int n_nodes,
-                                             int32_t* __restrict__ tris) {
-    const int4 rec = nodes[r];
+                                             int32_t* __restrict__ tris, int (*s_edge)[kTriThreads]) {
     const int cls = rec.y >> 8;
     const int nt = ntri_of(cls);
     if (nt == 0) return;
     const int nx = g.n[0], ny = g.n[1];
     const int row = rec.x / nx;
     const int x = rec.x - row * nx;
-    for (int t = 0; t < nt; ++t) {
-        for (int j = 0; j < 3; ++j) {
-            const int e = c_tri[cls][t][j];
-            const int axis = e >> 2;
-            const int cu = e & 1, cv = (e >> 1) & 1;
-            // owner offset: the edge's fixed coordinates on the two other axes
-            const int ox = axis == 0 ? 0 : cu;
-            const int oy = axis == 1 ? 0 : (axis == 0 ? cu : cv);
-            const int oz = axis == 2 ? 0 : cv;
-            int4 orec = rec;
-            if (ox | oy | oz) {
-                const int orow = row + oy + ny * oz;
-                const int ox_node = x + ox;
-                const int2 wi = wordinfo[(int64_t)orow * wp + (ox_node >> 5)];
-                const unsigned before = (unsigned)wi.y & ((1u << (ox_node & 31)) - 1u);
-                // clamped: an inconsistent lookup gives a wrong index, never an access outside the records
-                orec = nodes[min(max(wi.x + __popc(before), 0), n_nodes - 1)];
-            }
-            const int below = (orec.y & 7) & ((1 << axis) - 1);
-            tris[3 * (int64_t)(rec.w + t) + j] = orec.z + __popc(below);
-        }
+    // corner b of the cube at (b & 1, b >> 1 & 1, b >> 2 & 1); owner b is needed
+    // when one of its edges toward +a inside the cube crosses
+    int first[7], below[7];
+    first[0] = rec.z;
+    below[0] = rec.y;
+    int2 wi[7];
+    bool need[7];
+#pragma unroll
+    for (int b = 1; b < 7; ++b) {
+        const int in = (cls >> b) & 1;
+        need[b] = false;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            if (!((b >> a) & 1)) need[b] = need[b] || ((cls >> (b | (1 << a))) & 1) != in;
+        if (need[b])
+            wi[b] = wordinfo[(int64_t)(row + ((b >> 1) & 1) + ny * (b >> 2)) * wp + ((x + (b & 1)) >> 5)];
     }
+#pragma unroll
+    for (int b = 1; b < 7; ++b) {
+        if (!need[b]) continue;
+        const unsigned before = (unsigned)wi[b].y & ((1u << ((x + (b & 1)) & 31)) - 1u);
+        // clamped: an inconsistent lookup gives a wrong index, never an access outside the records
+        const int4 o = nodes[min(max(wi[b].x + __popc(before), 0), n_nodes - 1)];
+        first[b] = o.z;
+        below[b] = o.y;
+    }
+    const int tid = threadIdx.x;
+    // edge 4 a + c_u + 2 c_v: from corner (c_u, c_v) on the two other axes toward +a
+#pragma unroll
+    for (int e = 0; e < 12; ++e) {
+        const int a = e >> 2, cu = e & 1, cv = (e >> 1) & 1;
+        const int b = a == 0 ? (cu << 1) | (cv << 2) : (a == 1 ? cu | (cv << 2) : cu | (cv << 1));
+        if (((cls >> b) & 1) != ((cls >> (b | (1 << a))) & 1))
+            s_edge[e][tid] = first[b] + __popc(below[b] & ((1 << a) - 1));
+    }
+    for (int k = 0; k < nt; ++k)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) tris[3 * (int64_t)(rec.w + k) + j] = s_edge[c_tri[cls][k][j]][tid];
 }
 
 // One thread per node record: the vertices on its crossing edges, then its
 // triangles.
-__global__ void __launch_bounds__(256) k_mc_tris(GridDev g, const float* __restrict__ A,
-                                                 const float* __restrict__ levelf, const int4* __restrict__ nodes,
-                                                 const int* __restrict__ totals, int cap_nodes, int cap_tris,
-                                                 const int2* __restrict__ wordinfo, int wp,
-                                                 int32_t* __restrict__ tris, float* __restrict__ verts,
-                                                 float* __restrict__ vnrm, int cap_v) {
+__global__ void __launch_bounds__(kTriThreads) k_mc_tris(GridDev g, const float* __restrict__ A,
+                                                         const float* __restrict__ levelf,
+                                                         const int4* __restrict__ nodes,
+                                                         const int* __restrict__ totals, int cap_nodes, int cap_tris,
+                                                         const int2* __restrict__ wordinfo, int wp,
+                                                         int32_t* __restrict__ tris, float* __restrict__ verts,
+                                                         float* __restrict__ vnrm, int cap_v) {
     pdl_wait();
+    __shared__ int s_edge[12][kTriThreads];
     const int n_nodes = totals[0];
     if (n_nodes > cap_nodes || totals[2] > cap_tris) return;   // the host grows the buffers and runs again
     const float Ln = levelf[1];
@@ -469,7 +555,7 @@ __global__ void __launch_bounds__(256) k_mc_tris(GridDev g, const float* __restr
             const int q[3] = {rec.x - row * nx, row % ny, row / ny};
             emit_vertices(g, A, Ln, (int64_t)rec.x, q, flags, rec.z, cap_v, verts, vnrm);
         }
-        tris_of_node(g, nodes, r, wordinfo, wp, n_nodes, tris);
+        tris_of_node(g, nodes, rec, wordinfo, wp, n_nodes, tris, s_edge);
     }
 }
 
@@ -542,17 +628,20 @@ static int mc_words(int nx) {
 static int mc_tiles(int nrows, int wp, int t) { return (int)(((int64_t)nrows * wp + t - 1) / t); }
 static int mc_groups(int ntiles) { return (ntiles + kMcGroup - 1) / kMcGroup; }
 
-// CTAs of the inside-bit pass: one warp per row.  (A grid of one resident
+// CTAs of the inside-bit pass: kBitRows rows per warp.  (A grid of one resident
 // wave taking rows in a stride was as fast for one frame and 4-7 % slower
 // when frames of several contexts overlap: short CTAs fill in around other
 // kernels' CTAs.)
-static unsigned mc_bits_grid(int nrows) { return (unsigned)((nrows + kRowsPerCta - 1) / kRowsPerCta); }
+static unsigned mc_bits_grid(int nrows) {
+    constexpr int per = kMcThreads / 32 * kBitRows;
+    return (unsigned)((nrows + per - 1) / per);
+}
 
 cudaError_t launch_mc_bits(ftr_ctx* c) {
     const int nr = c->mc_blocks;
     launch_pdl(k_mc_bits, mc_bits_grid(nr), kMcThreads, 0, c->stream, c->g, c->d_A, c->d_levelf,
-               c->d_mc_bits, nr, mc_words(c->g.n[0]), (int*)nullptr, 0,
-               (const float2*)(c->rowmm_valid ? c->d_rowmm : nullptr));
+               c->d_mc_bits, c->d_mc_cls, nr, mc_words(c->g.n[0]), (int*)nullptr, 0,
+               (const float2*)(c->rowmm_valid ? c->d_rowmm : nullptr), 1);
     c->launches++;
     return cudaGetLastError();
 }
@@ -584,16 +673,17 @@ cudaError_t launch_mc_count(ftr_ctx* c) {
     int* sup = c->d_mc_blk + 4 * ntiles;
     prof_begin(c, ST_MC_COUNT);
     launch_pdl(k_mc_bits, mc_bits_grid(nr), kMcThreads, 0, c->stream, c->g, c->d_A, c->d_levelf,
-               c->d_mc_bits, nr, wp, sup, 4 * mc_groups(ntiles),
-               (const float2*)(c->rowmm_valid ? c->d_rowmm : nullptr));
-    launch_tiles<CountK>(c->mc_tile, ntiles, c->stream, c->g, (const unsigned*)c->d_mc_bits, nr, wp, agg, sup);
+               c->d_mc_bits, c->d_mc_cls, nr, wp, sup, 4 * mc_groups(ntiles),
+               (const float2*)(c->rowmm_valid ? c->d_rowmm : nullptr), 0);
+    launch_tiles<CountK>(c->mc_tile, ntiles, c->stream, c->g, (const unsigned*)c->d_mc_bits,
+                         (const unsigned char*)c->d_mc_cls, nr, wp, agg, sup);
     c->launches += 2;
     cudaError_t e = cudaGetLastError();
     prof_end(c, ST_MC_COUNT);
     return e;
 }
 
-// The rows' offsets and the node records, then the vertices and triangles.
+// The node records, then the vertices and triangles.
 cudaError_t launch_mc_emit(ftr_ctx* c) {
     const int nr = c->mc_blocks;
     const int wp = mc_words(c->g.n[0]);
@@ -601,8 +691,8 @@ cudaError_t launch_mc_emit(ftr_ctx* c) {
     const int4* agg = reinterpret_cast<const int4*>(c->d_mc_blk);
     const int4* sup = reinterpret_cast<const int4*>(c->d_mc_blk + 4 * ntiles);
     prof_begin(c, ST_MC_EMIT);
-    launch_tiles<EmitK>(c->mc_tile, ntiles, c->stream, c->g, (const unsigned*)c->d_mc_bits, nr, wp, ntiles, agg, sup,
-                        c->d_mc_off, c->d_mc_nodes, (int)c->cap_mc_nodes, c->d_mc_word, c->h_mc_tot);
+    launch_tiles<EmitK>(c->mc_tile, ntiles, c->stream, c->g, (const unsigned*)c->d_mc_bits,
+                        (const unsigned char*)c->d_mc_cls, nr, wp, ntiles, agg, sup, c->d_mc_tot, c->d_mc_nodes, (int)c->cap_mc_nodes, c->d_mc_word, c->h_mc_tot);
     c->launches++;
     cudaError_t e = cudaGetLastError();
     prof_end(c, ST_MC_EMIT);
@@ -611,7 +701,7 @@ cudaError_t launch_mc_emit(ftr_ctx* c) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     prof_begin(c, ST_MC_TRIS);
     launch_pdl(k_mc_tris, (sms > 0 ? sms : 152) * c->mc_tris_per_sm, 256, 0, c->stream, c->g, c->d_A, c->d_levelf, c->d_mc_nodes,
-               c->d_mc_off + 3 * (nr + 1), (int)c->cap_mc_nodes, (int)c->cap_tris, (const int2*)c->d_mc_word, wp,
+               (const int*)c->d_mc_tot, (int)c->cap_mc_nodes, (int)c->cap_tris, (const int2*)c->d_mc_word, wp,
                c->d_tris, c->d_verts, c->d_vnrm, (int)c->cap_verts);
     c->launches++;
     e = cudaGetLastError();
