@@ -242,7 +242,7 @@ void free_all(ftr_ctx* c) {
     dfree(c->d_tc_table);
     eval_free(c);
     dfree(c->d_raw);
-    dfree(c->d_raw_tiles);
+    dfree(c->d_raw_masks);
     dfree(c->d_raw_total);
     if (c->h_raw_total) cudaFreeHost(c->h_raw_total);
     dfree(c->d_ring);
@@ -555,7 +555,7 @@ int raw_enqueue(ftr_ctx* c, const char* who, const ftr_view* views, int k, doubl
         pixels += (int64_t)v.w * v.h;
     }
     cudaError_t e;
-    const int tiles = raw_tiles(views, k);
+    const int ints = raw_scratch_ints(views, k);
     if (pixels > c->raw_cap) {
         c->graph_valid = false;
         cudaStreamSynchronize(c->stream);
@@ -563,11 +563,11 @@ int raw_enqueue(ftr_ctx* c, const char* who, const ftr_view* views, int k, doubl
         if ((e = dalloc(&c->d_raw, (size_t)pixels * 7)) != cudaSuccess) return cuda_fail(c, e, who);
         c->raw_cap = pixels;
     }
-    if (tiles > c->raw_tiles_cap) {
+    if (ints > c->raw_masks_cap) {
         cudaStreamSynchronize(c->stream);
-        dfree(c->d_raw_tiles);
-        if ((e = dalloc(&c->d_raw_tiles, (size_t)tiles)) != cudaSuccess) return cuda_fail(c, e, who);
-        c->raw_tiles_cap = tiles;
+        dfree(c->d_raw_masks);
+        if ((e = dalloc(&c->d_raw_masks, (size_t)ints)) != cudaSuccess) return cuda_fail(c, e, who);
+        c->raw_masks_cap = ints;
     }
     if (!c->d_raw_total) {
         if ((e = dalloc(&c->d_raw_total, 1)) != cudaSuccess) return cuda_fail(c, e, who);
@@ -580,7 +580,7 @@ int raw_enqueue(ftr_ctx* c, const char* who, const ftr_view* views, int k, doubl
     rp.noise_f = (float)noise;
     rp.radius = radius;
     float* P = c->d_raw;
-    if ((e = launch_raw(c, rp, views, k, conf_out, P, P + 3 * pixels, P + 6 * pixels, c->d_raw_tiles,
+    if ((e = launch_raw(c, rp, views, k, conf_out, P, P + 3 * pixels, P + 6 * pixels, c->d_raw_masks,
                         c->d_raw_total)) != cudaSuccess)
         return cuda_fail(c, e, who);
     *pixels_out = pixels;
@@ -1587,7 +1587,7 @@ int ftr_autotune(ftr_ctx* c, float* report) {
 namespace {
 // Capacities that decide a context's device memory besides its grid.
 struct Caps {
-    int64_t pts = 0, stage = 0, tex_stage = 0, entries = 0, units = 0, heavy = 0, raw = 0, raw_tiles = 0;
+    int64_t pts = 0, stage = 0, tex_stage = 0, entries = 0, units = 0, heavy = 0, raw = 0, raw_masks = 0;
     int64_t mc_nodes = 0, verts = 0, tris = 0;
     bool tc = false;
     bool yz = false;     // the persistent y+z pass's ring and counters
@@ -1611,7 +1611,7 @@ int64_t context_bytes(const int n[3], const Caps& k) {
     b += 3 * (int64_t)(n[0] + n[1] + n[2]) * (int64_t)sizeof(float2);
     if (k.tc) b += (int64_t)tc_table_bytes() + 16;
     if (k.yz) b += (int64_t)(yz_ring_elems(n) * sizeof(float2)) + (int64_t)yz_sync_ints(n) * (int64_t)sizeof(int);
-    b += k.raw * 7 * (int64_t)sizeof(float) + k.raw_tiles * (int64_t)sizeof(int);
+    b += k.raw * 7 * (int64_t)sizeof(float) + k.raw_masks * (int64_t)sizeof(int);
     b += (2 * level_blocks + 8) * (int64_t)sizeof(double);
     b += (3 * mc_blocks + 16) * (int64_t)sizeof(int) + mc_blocks;   // tile and group sums, row classes
     b += mc_blocks * 16 * (int64_t)sizeof(unsigned);   // inside bits (upper bound)
@@ -1639,7 +1639,7 @@ int64_t ftr_device_bytes(const ftr_ctx* c) {
     k.units = c->cap_units;
     k.heavy = c->cap_heavy;
     k.raw = c->raw_cap;
-    k.raw_tiles = c->raw_tiles_cap;
+    k.raw_masks = c->raw_masks_cap;
     k.mc_nodes = c->cap_mc_nodes;
     k.verts = c->cap_verts;
     k.tris = c->cap_tris;
@@ -1663,7 +1663,9 @@ int64_t ftr_estimate_bytes(const int grid_n[3], int64_t points, int64_t depth_pi
     k.units = nb + k.entries / kSplatChunk + 2;
     k.heavy = heavy_capacity(pts);
     k.raw = depth_pixels;
-    k.raw_tiles = depth_pixels > 0 ? depth_pixels / 128 + 16 * 1024 : 0;
+    // two mask words per 32 pixels of a row and an int per eight: pixels / 16 words, and one per
+    // row of narrow views
+    k.raw_masks = depth_pixels > 0 ? 17 * ((depth_pixels / 16 + 16 * 1024) / 8) : 0;
     // mesh buffers grow to 1.5 x what a frame needs (+1024); active nodes <= vertices
     k.mc_nodes = vertices + vertices / 2 + 1024;
     k.verts = vertices + vertices / 2 + 1024;

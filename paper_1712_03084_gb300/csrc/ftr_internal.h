@@ -159,8 +159,8 @@ struct ftr_ctx {
     // raw reconstruction scratch (ftr_splat_depth)
     float* d_raw = nullptr;                // 7 floats per pixel capacity: P (3), N (3), W
     int64_t raw_cap = 0;                   // pixels
-    int* d_raw_tiles = nullptr;            // per-tile counts / offsets
-    int64_t raw_tiles_cap = 0;
+    int* d_raw_masks = nullptr;            // point and silhouette masks, points before each group of words
+    int64_t raw_masks_cap = 0;
     int* d_raw_total = nullptr;            // device total of the last call
     int* h_raw_total = nullptr;            // pinned copy
 
@@ -324,8 +324,8 @@ struct RawParams {
     int radius;              // W2 window radius
 };
 cudaError_t launch_raw(ftr_ctx* c, const RawParams& rp, const ftr_view* views, int k, float* const* conf_maps,
-                       float* P, float* N, float* W, int* d_tile_cnt, int* d_total);
-int raw_tiles(const ftr_view* views, int k);
+                       float* P, float* N, float* W, int* scratch, int* d_total);
+int raw_scratch_ints(const ftr_view* views, int k);   // two pixel masks and their prefix sums
 int raw_max_radius();
 // tensor-core split-precision passes (fft_tc.cu): pass 0 x fwd, 1 y fwd,
 // 2 z fwd + filter + z inv, 3 y inv, 4 x inv
