@@ -17,12 +17,21 @@
 // (exact).  The twiddles W_N^{j k1} between the two steps, the filter and
 // all other arithmetic stay fp32.
 //
-// One CTA keeps the fp32 passes' tile of F lines.  Step 1: thread (f, j)
-// writes its row x[N2 n1 + j] (n1 < N1) of the operand, one thread issues the
+// One CTA keeps the fp32 passes' tile of F lines.  Step 1: thread t = (f, j)
+// writes row t, x[N2 n1 + j] (n1 < N1), of the operand, one thread issues the
 // MMAs of all 128-row tiles, every thread reads its row back from Tensor
 // Memory (warp w owns lanes 32 (w % 4) ..  of tile w / 4), applies the
 // twiddles and scatters the values into the step-2 operand (the exchange
 // transpose); step 2 the same with the roles of N1 and N2 exchanged.
+//
+// Bound by latency: loads, the two products of a transform and their barriers
+// follow each other within a CTA, so what counts is how many CTAs an SM holds in
+// different phases (the tensor pipe is nearly idle).  Hence rows by whole warps,
+// products read back 16 columns at a time, no staging of whole lines, one DFT sign
+// per kernel, operand buffers without the last tile's padding and conversions two at
+// a time: 384^3 bf16x3, x / y / z / inverse y / inverse x, 211 / 371 / 425 / 164 / 201
+// -> 97 / 158 / 243 / 111 / 157 us; 256^3 fp16x3 57 / 84 / 104 / 41 / 61 -> 38 / 50 /
+// 80 / 38 / 44 us.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math.h>
@@ -77,18 +86,51 @@ template <> struct Half16<FTR_PREC_FP16X3> {
     __device__ static float back(unsigned short b) { return __half2float(__ushort_as_half(b)); }
 };
 
+// Both parts of two values, packed (x in the low half): one conversion for two.
 template <int P>
-__device__ __forceinline__ void split16(float x, unsigned short& hi, unsigned short& lo) {
-    hi = Half16<P>::rn(x);
-    lo = Half16<P>::rn(x - Half16<P>::back(hi));
+__device__ __forceinline__ void split16x2(float x, float y, uint32_t& hi, uint32_t& lo) {
+    if (P == FTR_PREC_BF16X3) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+        hi = reinterpret_cast<const uint32_t&>(h);
+        const __nv_bfloat162 l =
+            __floats2bfloat162_rn(x - __uint_as_float(hi << 16), y - __uint_as_float(hi & 0xffff0000u));
+        lo = reinterpret_cast<const uint32_t&>(l);
+    } else {
+        const __half2 h = __floats2half2_rn(x, y);
+        hi = reinterpret_cast<const uint32_t&>(h);
+        const float2 b = __half22float2(h);
+        const __half2 l = __floats2half2_rn(x - b.x, y - b.y);
+        lo = reinterpret_cast<const uint32_t&>(l);
+    }
+}
+
+// 2^-e for the frexp exponent e of m > 0, which scales m into [1/2, 1), and 2^e.
+__device__ __forceinline__ float line_scale(float m) {
+    const int b = (int)(__float_as_uint(m) >> 23);       // m >= 0; e = b - 126 for a normal m
+    if (b >= 1 && b <= 252) return __uint_as_float((uint32_t)(253 - b) << 23);
+    int e = 0;
+    if (m > 0.f) frexpf(m, &e);
+    return ldexpf(1.f, -e);
+}
+__device__ __forceinline__ float line_unscale(float m) {
+    const int b = (int)(__float_as_uint(m) >> 23);
+    if (b >= 1 && b <= 253) return __uint_as_float((uint32_t)(b + 1) << 23);
+    int e = 0;
+    if (m > 0.f) frexpf(m, &e);
+    return ldexpf(1.f, e);
 }
 
 constexpr int cpow2(int v) { return v <= 32 ? 32 : (v <= 64 ? 64 : (v <= 128 ? 128 : (v <= 256 ? 256 : 512))); }
 constexpr uint32_t kWaitPolls = 1u << 22;
 
 // Per-CTA tensor-core DFT engine for lines of length N, F lines per CTA,
-// F * N1 threads.  FWD / INV: which DFT signs the kernel uses.
-template <int N, int F, int P, bool FWD, bool INV>
+// F * N1 threads, up to DFTS transforms.  INV: the DFT sign of the matrices; the
+// other sign comes from them by conjugating input and output (exact).  TWS: the
+// twiddles are kept in shared memory with the matrices; the z and inverse passes
+// read them through L1 instead, which makes room for another CTA per SM (384 points:
+// z 275 -> 243, inverse x 168 -> 156 us; forward x and y are slower so, 97 -> 114
+// and 158 -> 184 us: their CTAs would not be more).
+template <int N, int F, int P, bool INV, int DFTS, bool TWS>
 struct Tc {
     static constexpr int N1 = Plan<N>::N1, N2 = Plan<N>::N2;
     static_assert(N1 >= N2 && N1 % 8 == 0 && N2 % 8 == 0, "tensor-core plan needs N1 >= N2, both multiples of 8");
@@ -96,69 +138,58 @@ struct Tc {
     static constexpr int tiles(int rows) { return (rows + 127) / 128; }
     static constexpr int TA = tiles(F * N2);   // rows carrying length-N1 vectors
     static constexpr int TB = tiles(F * N1);   // rows carrying length-N2 vectors
-    static constexpr int APART = cmax(TA * 16 * sbo_a(N1), TB * 16 * sbo_a(N2));
+    // The operand parts hold the rows that exist; a last tile of 64 rows reads on
+    // into what follows (its products are not read), so the tables come last.
+    static_assert(F % 8 == 0, "whole 8-row groups");
+    static constexpr int APART = cmax(F * N2 / 8 * sbo_a(N1), F * N1 / 8 * sbo_a(N2));
+    static constexpr int OVER = cmax(TA * 16 * sbo_a(N1), TB * 16 * sbo_a(N2)) - APART;
     static constexpr int COLS = cpow2(cmax(TA * 2 * N1, TB * 2 * N2));
-    static constexpr int NSIGN = (FWD ? 1 : 0) + (INV ? 1 : 0);
     static constexpr int BR1 = 16 * N1 * N1;
     static constexpr int BR2 = (N1 == N2) ? 0 : 16 * N2 * N2;
-    static constexpr int BBYTES = NSIGN * (BR1 + BR2);
-    static constexpr int TWBYTES = 8 * N;                  // W_N^m, m < N
-    static constexpr int HDR = 16 + ((4 * F + 15) / 16) * 16;
-    static constexpr int BYTES = HDR + BBYTES + TWBYTES + 2 * APART;
+    static constexpr int BBYTES = BR1 + BR2;
+    static constexpr int TWBYTES = TWS ? 8 * N : 0;        // W_N^m, m < N
+    static constexpr int HDR = 32 + ((4 * F * DFTS + 15) / 16) * 16;
+    static constexpr int BYTES = HDR + 2 * APART + cmax(BBYTES + TWBYTES, OVER);
 
     unsigned char* base;
-    uint32_t tmem;
     uint32_t phase;
     int* err;
+    const float2* tw_global;
 
     __device__ uint64_t* mbar() const { return (uint64_t*)base; }
-    __device__ unsigned* linemax() const { return (unsigned*)(base + 16); }
-    __device__ unsigned char* bmat(int R, int sign) const {
-        const int s = (FWD && INV && sign > 0) ? 1 : 0;
-        return base + HDR + s * (BR1 + BR2) + (R == N1 ? 0 : BR1);
-    }
-    __device__ const float2* twsm() const { return (const float2*)(base + HDR + BBYTES); }
-    __device__ unsigned char* ahi() const { return base + HDR + BBYTES + TWBYTES; }
-    __device__ unsigned char* alo() const { return base + HDR + BBYTES + TWBYTES + APART; }
-
-    __device__ void copy_b(const unsigned char* __restrict__ table, int R, int sign) {
-        const int bytes = 8 * R * R;
-        unsigned char* dst = bmat(R, sign);
-        for (int part = 0; part < 2; ++part) {
-            const uint4* s = (const uint4*)(table + tc_block(R, sign, part));
-            uint4* d = (uint4*)(dst + part * bytes);
-            for (int i = threadIdx.x; i < bytes / 16; i += blockDim.x) d[i] = s[i];
-        }
+    __device__ uint64_t* tbar() const { return (uint64_t*)(base + 16); }
+    __device__ unsigned* linemax(int k) const { return (unsigned*)(base + 32) + k * F; }
+    __device__ unsigned char* ahi() const { return base + HDR; }
+    __device__ unsigned char* alo() const { return base + HDR + APART; }
+    __device__ unsigned char* bmat(int R) const { return base + HDR + 2 * APART + (R == N1 ? 0 : BR1); }
+    __device__ float2 twiddle(int m) const {
+        return TWS ? ((const float2*)(base + HDR + 2 * APART + BBYTES))[m] : __ldg(tw_global + m);
     }
 
-    // Collective: stage the DFT matrices and the twiddles W_N^m (tw, m < N),
-    // allocate Tensor Memory, set up the completion barrier.
+    // Collective, without a barrier (the first product's makes it good): bulk copies
+    // of the DFT matrices and the twiddles W_N^m (tw, m < N), which arrive while the
+    // CTA loads its lines; Tensor Memory; the completion barrier.
     __device__ void init(unsigned char* smem, const unsigned char* __restrict__ table,
                          const float2* __restrict__ tw, int* err_flag) {
         base = smem;
+        tw_global = tw;
         phase = 0;
         err = err_flag;
-        {
-            float2* t = (float2*)(base + HDR + BBYTES);
-            for (int i = threadIdx.x; i < N; i += blockDim.x) t[i] = tw[i];
-        }
-        if (FWD) {
-            copy_b(table, N1, -1);
-            if (N2 != N1) copy_b(table, N2, -1);
-        }
-        if (INV) {
-            copy_b(table, N1, +1);
-            if (N2 != N1) copy_b(table, N2, +1);
-        }
         if (threadIdx.x < 32) tc::tmem_alloc((uint32_t*)(base + 8), COLS);
         if (threadIdx.x == 0) {
             tc::mbar_init(mbar(), 1);
+            tc::mbar_init(tbar(), 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            tc::fence_async_smem();
+            tc::mbar_expect_tx(tbar(), BBYTES + TWBYTES);
+            constexpr int sign = INV ? 1 : -1;
+            for (int part = 0; part < 2; ++part) {
+                tc::bulk_g2s(bmat(N1) + part * 8 * N1 * N1, table + tc_block(N1, sign, part), 8 * N1 * N1, tbar());
+                if (N2 != N1)
+                    tc::bulk_g2s(bmat(N2) + part * 8 * N2 * N2, table + tc_block(N2, sign, part), 8 * N2 * N2, tbar());
+            }
+            if (TWS) tc::bulk_g2s(base + HDR + 2 * APART + BBYTES, tw, TWBYTES, tbar());
         }
-        tc::fence_before_sync();
-        __syncthreads();
-        tc::fence_after_sync();
-        tmem = *(volatile uint32_t*)(base + 8);
     }
 
     // Collective: release Tensor Memory (every CTA path that called init
@@ -167,56 +198,48 @@ struct Tc {
         tc::fence_before_sync();
         __syncthreads();
         tc::fence_after_sync();
-        if (threadIdx.x < 32) tc::tmem_dealloc(tmem, COLS);
+        if (threadIdx.x < 32) tc::tmem_dealloc(*(volatile uint32_t*)(base + 8), COLS);
     }
 
-    // Row `row` of the length-R operand from R complex values times `scale`.
+    // Complex values 4 q .. 4 q + 3 of row `row` of the length-R operand.
     template <int R>
-    __device__ void put_row(int row, const float2 (&v)[R], float scale) {
-#pragma unroll
-        for (int q = 0; q < R / 4; ++q) {
-            unsigned short h[8], l[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                split16<P>(v[4 * q + i].x * scale, h[2 * i], l[2 * i]);
-                split16<P>(v[4 * q + i].y * scale, h[2 * i + 1], l[2 * i + 1]);
-            }
-            uint4 H, L;
-            H.x = h[0] | ((uint32_t)h[1] << 16); H.y = h[2] | ((uint32_t)h[3] << 16);
-            H.z = h[4] | ((uint32_t)h[5] << 16); H.w = h[6] | ((uint32_t)h[7] << 16);
-            L.x = l[0] | ((uint32_t)l[1] << 16); L.y = l[2] | ((uint32_t)l[3] << 16);
-            L.z = l[4] | ((uint32_t)l[5] << 16); L.w = l[6] | ((uint32_t)l[7] << 16);
-            const int o = a_off(R, row, 8 * q);
-            *(uint4*)(ahi() + o) = H;
-            *(uint4*)(alo() + o) = L;
-        }
+    __device__ void put4(int row, int q, const float2 (&v)[4]) {
+        uint4 H, L;
+        split16x2<P>(v[0].x, v[0].y, H.x, L.x);
+        split16x2<P>(v[1].x, v[1].y, H.y, L.y);
+        split16x2<P>(v[2].x, v[2].y, H.z, L.z);
+        split16x2<P>(v[3].x, v[3].y, H.w, L.w);
+        const int o = a_off(R, row, 8 * q);
+        *(uint4*)(ahi() + o) = H;
+        *(uint4*)(alo() + o) = L;
     }
 
     // Complex value m of row `row` of the length-R operand.
     template <int R>
     __device__ void put1(int row, int m, float2 v) {
-        unsigned short hr, lr, hi, li;
-        split16<P>(v.x, hr, lr);
-        split16<P>(v.y, hi, li);
+        uint32_t h, l;
+        split16x2<P>(v.x, v.y, h, l);
         const int o = a_off(R, row, 2 * m);
-        *(uint32_t*)(ahi() + o) = hr | ((uint32_t)hi << 16);
-        *(uint32_t*)(alo() + o) = lr | ((uint32_t)li << 16);
+        *(uint32_t*)(ahi() + o) = h;
+        *(uint32_t*)(alo() + o) = l;
     }
 
-    // Collective: D_t = A_t D_R (sign) for every 128-row tile t of `rows`
-    // rows, into Tensor Memory columns [t 2R, t 2R + 2R).
-    template <int R, int SIGN>
-    __device__ void run(int rows) {
+    // Collective: D_t = A_t D_R for every 128-row tile t of `rows` rows, into Tensor
+    // Memory columns [t 2R, t 2R + 2R); returns their address.
+    template <int R>
+    __device__ uint32_t run(int rows) {
         tc::fence_async_smem();
         tc::fence_before_sync();
         __syncthreads();
         tc::fence_after_sync();
+        const uint32_t tmem = *(volatile uint32_t*)(base + 8);
+        if (!tc::mbar_wait(tbar(), 0, kWaitPolls)) atomicExch(err, 1);
         if (threadIdx.x == 0) {
             constexpr uint32_t SBO = 32 * R;                 // B: dense
             constexpr uint32_t LA = lbo_a(R), SA = sbo_a(R);  // A: padded
             const uint32_t id = tc::idesc_f16(P == FTR_PREC_BF16X3, 128, 2 * R);
             const uint32_t a0 = tc::smem_u32(ahi()), a1 = tc::smem_u32(alo());
-            const uint32_t b0 = tc::smem_u32(bmat(R, SIGN)), b1 = b0 + 8 * R * R;
+            const uint32_t b0 = tc::smem_u32(bmat(R)), b1 = b0 + 8 * R * R;
             const int nt = tiles(rows);
             for (int t = 0; t < nt; ++t) {
 #pragma unroll
@@ -233,92 +256,114 @@ struct Tc {
         if (!tc::mbar_wait(mbar(), phase, kWaitPolls)) atomicExch(err, 1);
         phase ^= 1u;
         tc::fence_after_sync();
+        const int w = threadIdx.x >> 5;
+        return tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * 2 * R);
     }
 
-    // This thread's row (threadIdx.x) of the last product, 2R floats; false
-    // when the row lies beyond `rows`.
-    template <int R>
-    __device__ bool get(int rows, float (&buf)[2 * R]) {
-        const int w = threadIdx.x >> 5, t = w >> 2;
-        if (t < tiles(rows)) {
-            const uint32_t a = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(t * 2 * R);
-            if ((2 * R) % 32 == 0) {
-#pragma unroll
-                for (int c = 0; c < 2 * R / 32; ++c) tc::tmem_ld32(a + 32 * c, buf + 32 * c);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 2 * R / 16; ++c) tc::tmem_ld16(a + 16 * c, buf + 16 * c);
-            }
-        }
-        return (int)threadIdx.x < rows;
-    }
-
-    // Collective length-R1 R2 transform of F lines.  In: thread with `act`
-    // holds x[R2 n1 + j] (n1 < R1) of line f, j < R2.  Out: thread t < F R1
-    // holds X[k1 + R1 k2] (k2 < R2) of line t / R1 with k1 = t % R1, or (with
-    // LINE_FAST) of line t % F with k1 = t / F.  tw: W_{R1 R2}^m, m < R1 R2.
-    template <int R1, int R2, int SIGN, bool LINE_FAST>
-    __device__ void dft(const float2 (&v)[R1], bool act, int f, int j, float2 (&out)[R2]) {
-        constexpr int NN = R1 * R2;
+    // Collective length-R1 R2 transform number `k` of F lines, sign that of the
+    // matrices or (CONJ) the other one.
+    // In: thread t < F R2 takes x[R2 n1 + j] = ld(n1) (n1 < R1) of line f, with f =
+    // t / R2, j = t % R2 or (IN_FAST) f = t % F, j = t / F: its row of the first
+    // operand, so rows are whole warps.  Out: thread t < F R1 gets st(k2, X[k1 + R1
+    // k2]) for each k2 < R2 of line t / R1 with k1 = t % R1, or (OUT_FAST) of line
+    // t % F with k1 = t / F.  Products are read back 16 columns at a time: a row at a
+    // time (up to 48 registers) kept these passes at one to three CTAs per SM.
+    template <int R1, int R2, bool CONJ, bool IN_FAST, bool OUT_FAST, class Ld, class St>
+    __device__ __forceinline__ void dft(int k, Ld ld, St st) {
+        constexpr int ROWS1 = F * R2, ROWS2 = F * R1;
+        static_assert(ROWS1 % 32 == 0 && ROWS2 % 32 == 0, "whole warps");
         const int tid = threadIdx.x;
-        float scale = 1.f;
+        const int f = IN_FAST ? tid % F : tid / R2, j = IN_FAST ? tid / F : tid % R2;
         if (P == FTR_PREC_FP16X3) {
-            __syncthreads();
-            if (tid < F) linemax()[tid] = 0u;
-            __syncthreads();
-            if (act) {
-                float m = 0.f;
+            float2 v[R1];
+            float m = 0.f;
+            if (tid < ROWS1) {
+#pragma unroll
+                for (int i = 0; i < R1; ++i) v[i] = ld(i);
 #pragma unroll
                 for (int i = 0; i < R1; ++i) m = fmaxf(m, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
-                atomicMax(&linemax()[f], __float_as_uint(m));
-            }
-            __syncthreads();
-            if (act) {
-                int e;
-                const float m = __uint_as_float(linemax()[f]);
-                if (m > 0.f) {
-                    frexpf(m, &e);
-                    scale = ldexpf(1.f, -e);
+                if (!IN_FAST && (R2 & (R2 - 1)) == 0) {         // a line is R2 lanes
+#pragma unroll
+                    for (int o = R2 / 2; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                    if (j == 0) linemax(k)[f] = __float_as_uint(m);
                 }
             }
-        }
-        if (act) put_row<R1>(f * R2 + j, v, scale);
-        run<R1, SIGN>(F * R2);
-        {
-            float buf[2 * R1];
-            if (get<R1>(F * R2, buf)) {
-                const int f1 = tid / R2, j1 = tid % R2;
+            if (IN_FAST || (R2 & (R2 - 1)) != 0) {
+                if (tid < F) linemax(k)[tid] = 0u;
+                __syncthreads();
+                if (tid < ROWS1) atomicMax(&linemax(k)[f], __float_as_uint(m));
+                __syncthreads();
+                m = __uint_as_float(linemax(k)[f]);
+            }
+            if (tid < ROWS1) {
+                const float scale = line_scale(m);
 #pragma unroll
-                for (int k1 = 0; k1 < R1; ++k1) {
-                    float2 y = make_float2(buf[2 * k1], buf[2 * k1 + 1]);
-                    if (k1 != 0 && j1 != 0) {
-                        float2 w = twsm()[(j1 * k1) % NN];
-                        if (SIGN > 0) w.y = -w.y;
+                for (int q = 0; q < R1 / 4; ++q) {
+                    float2 u[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        u[i] = make_float2(v[4 * q + i].x * scale, v[4 * q + i].y * (CONJ ? -scale : scale));
+                    put4<R1>(tid, q, u);
+                }
+            }
+        } else if (tid < ROWS1) {
+#pragma unroll
+            for (int q = 0; q < R1 / 4; ++q) {
+                float2 u[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    u[i] = ld(4 * q + i);
+                    if (CONJ) u[i].y = -u[i].y;
+                }
+                put4<R1>(tid, q, u);
+            }
+        }
+        uint32_t at = run<R1>(ROWS1);
+        if (tid < ROWS1) {
+#pragma unroll
+            for (int c = 0; c < R1 / 8; ++c) {
+                float buf[16];
+                tc::tmem_ld16(at + 16 * c, buf);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int k1 = 8 * c + i;
+                    float2 y = make_float2(buf[2 * i], buf[2 * i + 1]);
+                    if (k1 != 0) {
+                        float2 w = twiddle(j * k1);
+                        if (INV) w.y = -w.y;
                         y = cmul(y, w);
                     }
-                    const int row = LINE_FAST ? k1 * F + f1 : f1 * R1 + k1;
-                    put1<R2>(row, j1, y);
+                    put1<R2>(OUT_FAST ? k1 * F + f : f * R1 + k1, j, y);
                 }
             }
         }
-        run<R2, SIGN>(F * R1);
-        float buf[2 * R2];
-        if (get<R2>(F * R1, buf)) {
+        at = run<R2>(ROWS2);
+        if (tid < ROWS2) {
             float inv = 1.f;
-            if (P == FTR_PREC_FP16X3) {
-                const int fo = LINE_FAST ? tid % F : tid / R1;
-                const float m = __uint_as_float(linemax()[fo]);
-                if (m > 0.f) {
-                    int e;
-                    frexpf(m, &e);
-                    inv = ldexpf(1.f, e);
-                }
-            }
+            if (P == FTR_PREC_FP16X3) inv = line_unscale(__uint_as_float(linemax(k)[OUT_FAST ? tid % F : tid / R1]));
 #pragma unroll
-            for (int k2 = 0; k2 < R2; ++k2) out[k2] = make_float2(buf[2 * k2] * inv, buf[2 * k2 + 1] * inv);
+            for (int c = 0; c < R2 / 8; ++c) {
+                float buf[16];
+                tc::tmem_ld16(at + 16 * c, buf);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    st(8 * c + i, make_float2(buf[2 * i] * inv, buf[2 * i + 1] * (CONJ ? -inv : inv)));
+            }
         }
     }
 };
+
+// The z and inverse-x passes ask for the input of the CTA `ahead` places later in
+// launch order (about the one that takes this CTA's place) to be brought to L2, so
+// that its loads wait for L2 and not for DRAM: 307 -> 270 and 173 -> 163 us at 384^3
+// (bf16x3).  Not where a half spectrum of `elems` fits L2 and mostly is there (256^3:
+// 87 -> 90 us), nor in the y passes (no gain).  Block index, or x = -1: none.
+__device__ __forceinline__ int2 later_block(int ahead, int64_t elems) {
+    if (elems * (int64_t)sizeof(float2) <= (int64_t)128 << 20) return make_int2(-1, -1);
+    const int id = (int)(blockIdx.x + gridDim.x * blockIdx.y) + ahead;
+    if (id >= (int)(gridDim.x * gridDim.y)) return make_int2(-1, -1);
+    return make_int2(id % (int)gridDim.x, id / (int)gridDim.x);
+}
 
 // ---------------------------------------------------------------- x forward
 // Same as the fp32 x pass: 16 rows (y0.., z) of the three components from the
@@ -328,12 +373,12 @@ constexpr int kFxRows = 16;
 constexpr int kFxLines = 24;
 
 template <int N, int P>
-__global__ void __launch_bounds__(kFxLines * Plan<N>::N1)
+__global__ void __launch_bounds__(kFxLines * Plan<N>::N1, N >= 384 ? 2 : 3)
     k_tc_fx(GridDev g, const int* __restrict__ slot_tab, const float* __restrict__ vpool, float2* __restrict__ s0,
             int64_t Mh, const float2* __restrict__ tw, float wx_scale, const int* __restrict__ meta,
             const unsigned char* __restrict__ table, int* err) {
     pdl_wait();
-    using E = Tc<N, kFxLines, P, true, false>;
+    using E = Tc<N, kFxLines, P, false, 1, true>;
     constexpr int N1 = E::N1, N2 = E::N2;
     constexpr int NB = N / kBrick;
     constexpr int NKX = N / 2 + 1;
@@ -376,31 +421,21 @@ __global__ void __launch_bounds__(kFxLines * Plan<N>::N1)
     // once the last product has been read back
     static_assert(sizeof(float2) * ZS * N <= 2 * E::APART, "park fits the operand buffers");
     float2* park = (float2*)e.ahi();
-    const int f = tid / N1, r = tid % N1;
-    const int lz = z & 7;
-    const bool act = r < N2;
-    float2 v[N1];
-    if (act) {
-        const int ra = f < 16 ? f : f - 16;
-        const int rb = f < 16 ? f : f - 8;
-        const int ca = f < 16 ? 0 : 2;
-        const int cb = f < 16 ? 1 : 2;
-#pragma unroll
-        for (int n1 = 0; n1 < N1; ++n1) {
+    const int f = tid / N2, r = tid % N2;             // line and first element in
+    const int ra = f < 16 ? f : f - 16, rb = f < 16 ? f : f - 8;
+    const int la = (f < 16 ? 0 : 2) * kBrickVox + 8 * ((ra & 7) + 8 * (z & 7));
+    const int lb = (f < 16 ? 1 : 2) * kBrickVox + 8 * ((rb & 7) + 8 * (z & 7));
+    const int f2 = tid / N1, r2 = tid % N1;           // line and first bin out
+    e.template dft<N1, N2, false, false, false>(
+        0,
+        [&](int n1) {
             const int x = N2 * n1 + r;
-            const int sa = s_slot[ra >> 3][x >> 3];
-            const int sb = s_slot[rb >> 3][x >> 3];
-            const int la = (x & 7) + 8 * ((ra & 7) + 8 * lz);
-            const int lb = (x & 7) + 8 * ((rb & 7) + 8 * lz);
-            const float a = sa >= 0 ? vpool[(size_t)sa * 3 * kBrickVox + ca * kBrickVox + la] : 0.f;
-            const float b = sb >= 0 ? vpool[(size_t)sb * 3 * kBrickVox + cb * kBrickVox + lb] : 0.f;
-            v[n1] = make_float2(a, b);
-        }
-    }
-    float2 o[N2];
-    e.template dft<N1, N2, -1, false>(v, act, f, r, o);
-#pragma unroll
-    for (int k2 = 0; k2 < N2; ++k2) park[f + ZS * (r + N1 * k2)] = o[k2];
+            const int sa = s_slot[ra >> 3][x >> 3], sb = s_slot[rb >> 3][x >> 3];
+            const float a = sa >= 0 ? vpool[(size_t)sa * 3 * kBrickVox + la + (x & 7)] : 0.f;
+            const float b = sb >= 0 ? vpool[(size_t)sb * 3 * kBrickVox + lb + (x & 7)] : 0.f;
+            return make_float2(a, b);
+        },
+        [&](int k2, float2 y) { park[f2 + ZS * (r2 + N1 * k2)] = y; });
     __syncthreads();
     for (int k = tid; k < kFxRows * NKX; k += blockDim.x) {
         const int row = k & (kFxRows - 1), kx = k >> 4;
@@ -432,8 +467,12 @@ __global__ void __launch_bounds__(kFxLines * Plan<N>::N1)
 
 // Lines per CTA of the y, inverse-y and z passes: 16; the z pass takes 8
 // where the step-1 DFT is longer than 16 (384 points: a CTA of 8 x 24
-// threads, three of which fit an SM; measured faster there, and slower for
-// the y passes).
+// threads, five of which fit an SM; the y passes' strided side needs 16 for
+// whole 128-byte lines).  The minimum CTAs per SM of the launch bounds are the
+// fastest ones measured: a few spilled registers cost less than a CTA less where a
+// pass keeps one component's bins (y 384 bf16x3: 173 us with two, 158 with three), but
+// not in the inverse y pass (111 us with two, 117 with three) nor with the fp16
+// variant's whole lines in registers (z 384: 326 us with five, 303 with four).
 template <int N>
 struct TcLines {
     static constexpr int value = 16;
@@ -448,12 +487,12 @@ struct TcLinesZ {
 // j w_y Y[X V_y] and Y[X V_z] out in [k_x][k_y][z].
 
 template <int N, int P>
-__global__ void __launch_bounds__(TcLines<N>::value * Plan<N>::N1, TcLines<N>::value * Plan<N>::N1 <= 256 ? 2 : 1)
+__global__ void __launch_bounds__(TcLines<N>::value * Plan<N>::N1, N >= 384 ? (P == FTR_PREC_BF16X3 ? 3 : 2) : 4)
     k_tc_fy(GridDev g, const float2* __restrict__ s0, float2* __restrict__ s1, int64_t Mh,
             const float2* __restrict__ tw, float wy_scale, const int* __restrict__ meta,
             const unsigned char* __restrict__ table, int* err) {
     pdl_wait();
-    using E = Tc<N, TcLines<N>::value, P, true, false>;
+    using E = Tc<N, TcLines<N>::value, P, false, 3, true>;
     constexpr int N1 = E::N1, N2 = E::N2;
     constexpr int F = TcLines<N>::value;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -466,49 +505,38 @@ __global__ void __launch_bounds__(TcLines<N>::value * Plan<N>::N1, TcLines<N>::v
     if (z0 < zl || z0 >= zh) return;
     E e;
     e.init(smem_raw, table, tw, err);
-    float2* stash = (float2*)(smem_raw + E::BYTES);
-    const int f1 = tid / N1, r1 = tid % N1;
-    const bool act = r1 < N2;
-    const int f2 = tid % F, i2 = tid / F;
-    const size_t out_base = (size_t)(z0 + f2) + (size_t)nz * ((size_t)N * kx);
-    const float2* line = s0 + (size_t)N * (z0 + f1 + (size_t)nz * kx);
+    const int f1 = tid / N2, r1 = tid % N2;           // line and first element in
+    const int f2 = tid % F, i2 = tid / F;             // line and first bin out
+    const float2* line = s0 + (size_t)N * (z0 + f1 + (size_t)nz * kx) + r1;
+    float2* out = s1 + (size_t)(z0 + f2) + (size_t)nz * ((size_t)N * kx + i2);
     static_assert(16 % N2 == 0, "an element's 16-row group is n1's");
-    const unsigned rows = live_rows(meta, z0 + f1);
-    float2 v[N1], o[N2];
-    for (int c = 0; c < 3; ++c) {
-        if (act) {
-#pragma unroll
-            for (int n1 = 0; n1 < N1; ++n1)
-                v[n1] = (rows >> (N2 * n1 / 16)) & 1u ? line[(size_t)c * Mh + N2 * n1 + r1] : make_float2(0.f, 0.f);
-        }
-        e.template dft<N1, N2, -1, true>(v, act, f1, r1, o);
-        if (c == 0) {
-#pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) stash[f2 + (F + 1) * (i2 + N1 * k2)] = o[k2];
-        } else if (c == 1) {
-#pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) {
-                const int ky = i2 + N1 * k2;
-                const float wy = (ky == N / 2) ? 0.f : wy_scale * (float)signed_bin(ky, N);
-                const float2 w = stash[f2 + (F + 1) * ky];
-                s1[out_base + (size_t)nz * ky] = make_float2(w.x - wy * o[k2].y, w.y + wy * o[k2].x);
-            }
-        } else {
-#pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) s1[Mh + out_base + (size_t)nz * (i2 + N1 * k2)] = o[k2];
-        }
-    }
+    const unsigned rows = tid < F * N2 ? live_rows(meta, z0 + f1) : 0u;
+    const auto in = [&](int n1) {
+        return (rows >> (N2 * n1 / 16)) & 1u ? line[N2 * n1] : make_float2(0.f, 0.f);
+    };
+    // the x component's bins stay in registers until the y component's are there
+    float2 w[N2];
+    e.template dft<N1, N2, false, false, true>(0, in, [&](int k2, float2 y) { w[k2] = y; });
+    line += Mh;
+    e.template dft<N1, N2, false, false, true>(1, in, [&](int k2, float2 y) {
+        const int ky = i2 + N1 * k2;
+        const float wy = (ky == N / 2) ? 0.f : wy_scale * (float)signed_bin(ky, N);
+        out[(size_t)nz * (N1 * k2)] = make_float2(w[k2].x - wy * y.y, w[k2].y + wy * y.x);
+    });
+    line += Mh;
+    out += Mh;
+    e.template dft<N1, N2, false, false, true>(2, in, [&](int k2, float2 y) { out[(size_t)nz * (N1 * k2)] = y; });
     e.finish();
 }
 
 // ------------------------------------------- z forward + filter + z inverse
 template <int N, int P>
-__global__ void __launch_bounds__(TcLinesZ<N>::value * Plan<N>::N1, TcLinesZ<N>::value * Plan<N>::N1 <= 256 ? 3 : 1)
+__global__ void __launch_bounds__(TcLinesZ<N>::value * Plan<N>::N1, N >= 384 && P == FTR_PREC_BF16X3 ? 5 : 4)
     k_tc_fz(GridDev g, float2* __restrict__ s1, int64_t Mh, const float2* __restrict__ tw, float wx_scale,
             float wy_scale, float wz_scale, float inv_m, const int* __restrict__ meta,
             const unsigned char* __restrict__ table, int* err) {
     pdl_wait();
-    using E = Tc<N, TcLinesZ<N>::value, P, true, true>;
+    using E = Tc<N, TcLinesZ<N>::value, P, false, 3, false>;
     constexpr int N1 = E::N1, N2 = E::N2;
     constexpr int F = TcLinesZ<N>::value;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -516,62 +544,53 @@ __global__ void __launch_bounds__(TcLinesZ<N>::value * Plan<N>::N1, TcLinesZ<N>:
     const int ky0 = blockIdx.x * F;
     const int kx = blockIdx.y;
     const int tid = threadIdx.x;
-    const int f = tid / N1, r = tid % N1;
-    const bool act = r < N2;
     int zl, zh;
     live_z_range(meta, zl, zh);
     E e;
     e.init(smem_raw, table, tw, err);
-    const size_t line = (size_t)N * ((size_t)(ky0 + f) + (size_t)ny * kx);
-    float2 v[N1], xw[N2], xh[N2];
-#pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) {
-        const int z = N2 * n1 + r;
-        v[n1] = (act && z >= zl && z < zh) ? s1[line + z] : make_float2(0.f, 0.f);
-    }
-    e.template dft<N1, N2, -1, false>(v, act, f, r, xw);
-#pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) {
-        const int z = N2 * n1 + r;
-        v[n1] = (act && z >= zl && z < zh) ? s1[Mh + line + z] : make_float2(0.f, 0.f);
-    }
-    e.template dft<N1, N2, -1, false>(v, act, f, r, xh);
+    const int2 later = later_block(152 * (P == FTR_PREC_BF16X3 ? 5 : 4), Mh);
+    if (tid < 2 * F && later.x >= 0 && zl < zh)
+        tc::bulk_prefetch_l2(s1 + (tid < F ? 0 : Mh) +
+                                 (size_t)N * ((size_t)(later.x * F + tid % F) + (size_t)ny * later.y) + zl,
+                             (uint32_t)(zh - zl) * (uint32_t)sizeof(float2));
+    float2* lines = s1 + (size_t)N * ((size_t)ky0 + (size_t)ny * kx);
+    const int r1 = tid % N2;                          // first element in, of line tid / N2
+    const float2* line = lines + (size_t)N * (tid / N2) + r1;
+    const auto in = [&](int n1) {
+        const int z = N2 * n1 + r1;
+        return z >= zl && z < zh ? line[N2 * n1] : make_float2(0.f, 0.f);
+    };
+    float2 x[N2];
+    e.template dft<N1, N2, false, false, false>(0, in, [&](int k2, float2 y) { x[k2] = y; });
+    line += Mh;
     // thread (f, r): bins k_z = r + N1 k2 of line f
-    {
-        const int ky = ky0 + f;
-        const float wxd = wx_scale * (float)kx;
-        const float wyd = wy_scale * (float)signed_bin(ky, ny);
-        const float base = wxd * wxd + wyd * wyd;
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) {
-            const int kz = r + N1 * k2;
-            const float wzd = wz_scale * (float)signed_bin(kz, N);
-            const float wzn = (kz == N / 2) ? 0.f : wzd;
-            const float den = base + wzd * wzd;
-            const float s = den > 0.f ? inv_m / den : 0.f;
-            const float2 sv = make_float2(xw[k2].x - wzn * xh[k2].y, xw[k2].y + wzn * xh[k2].x);
-            xw[k2] = make_float2(sv.x * s, sv.y * s);
-        }
-    }
+    const int r = tid % N1;
+    const float wxd = wx_scale * (float)kx;
+    const float wyd = wy_scale * (float)signed_bin(ky0 + tid / N1, ny);
+    const float base = wxd * wxd + wyd * wyd;
+    e.template dft<N1, N2, false, false, false>(1, in, [&](int k2, float2 y) {
+        const int kz = r + N1 * k2;
+        const float wzd = wz_scale * (float)signed_bin(kz, N);
+        const float wzn = (kz == N / 2) ? 0.f : wzd;
+        const float den = base + wzd * wzd;
+        const float s = den > 0.f ? inv_m / den : 0.f;
+        const float2 sv = make_float2(x[k2].x - wzn * y.y, x[k2].y + wzn * y.x);
+        x[k2] = make_float2(sv.x * s, sv.y * s);
+    });
     // inverse along z, N = N2 x N1: thread (f, r) holds x[r + N1 k2]
-    float2 o[N1];
-    e.template dft<N2, N1, +1, false>(xw, true, f, r, o);
-    if (tid < F * N2) {
-        const int fo = tid / N2, ko = tid % N2;
-        float2* dst = s1 + (size_t)N * ((size_t)(ky0 + fo) + (size_t)ny * kx);
-#pragma unroll
-        for (int k2 = 0; k2 < N1; ++k2) dst[ko + N2 * k2] = o[k2];
-    }
+    float2* dst = lines + (size_t)N * (tid / N2) + tid % N2;
+    e.template dft<N2, N1, true, false, false>(
+        2, [&](int n1) { return x[n1]; }, [&](int k2, float2 y) { dst[N2 * k2] = y; });
     e.finish();
 }
 
 // ---------------------------------------------------------------- y inverse
 template <int N, int P>
-__global__ void __launch_bounds__(TcLines<N>::value * Plan<N>::N1)
+__global__ void __launch_bounds__(TcLines<N>::value * Plan<N>::N1, N >= 384 ? 2 : 4)
     k_tc_iy(GridDev g, const float2* __restrict__ src, float2* __restrict__ dst, const float2* __restrict__ tw,
             const unsigned char* __restrict__ table, int* err) {
     pdl_wait();
-    using E = Tc<N, TcLines<N>::value, P, false, true>;
+    using E = Tc<N, TcLines<N>::value, P, true, 1, false>;
     constexpr int N1 = E::N1, N2 = E::N2;
     constexpr int F = TcLines<N>::value;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -581,21 +600,10 @@ __global__ void __launch_bounds__(TcLines<N>::value * Plan<N>::N1)
     const int tid = threadIdx.x;
     E e;
     e.init(smem_raw, table, tw, err);
-    const int f1 = tid % F, j1 = tid / F;
-    const bool act = j1 < N2;
-    float2 v[N1], o[N2];
-    if (act) {
-#pragma unroll
-        for (int n1 = 0; n1 < N1; ++n1) {
-            const int ky = N2 * n1 + j1;
-            v[n1] = src[(size_t)(z0 + f1) + (size_t)nz * ((size_t)ky + (size_t)N * kx)];
-        }
-    }
-    e.template dft<N1, N2, +1, false>(v, act, f1, j1, o);
-    const int f2 = tid / N1, i2 = tid % N1;
-    float2* out = dst + (size_t)N * ((size_t)(z0 + f2) + (size_t)nz * kx);
-#pragma unroll
-    for (int k2 = 0; k2 < N2; ++k2) out[i2 + N1 * k2] = o[k2];
+    const float2* in = src + (size_t)(z0 + tid % F) + (size_t)nz * ((size_t)(tid / F) + (size_t)N * kx);
+    float2* out = dst + (size_t)N * ((size_t)(z0 + tid / N1) + (size_t)nz * kx) + tid % N1;
+    e.template dft<N1, N2, false, true, false>(
+        0, [&](int n1) { return in[(size_t)nz * (N2 * n1)]; }, [&](int k2, float2 y) { out[N1 * k2] = y; });
     e.finish();
 }
 
@@ -605,11 +613,11 @@ constexpr int kIxLines = 8;
 constexpr int kHs = kIxRows + 1;
 
 template <int N, int P>
-__global__ void __launch_bounds__(kIxLines * Plan<N>::N1)
+__global__ void __launch_bounds__(kIxLines * Plan<N>::N1, N >= 384 ? 5 : 9)
     k_tc_ix(GridDev g, const float2* __restrict__ src, float* __restrict__ A, const float2* __restrict__ tw,
             const unsigned char* __restrict__ table, int* err) {
     pdl_wait();
-    using E = Tc<N, kIxLines, P, false, true>;
+    using E = Tc<N, kIxLines, P, true, 1, false>;
     constexpr int N1 = E::N1, N2 = E::N2;
     constexpr int NKX = N / 2 + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -623,6 +631,10 @@ __global__ void __launch_bounds__(kIxLines * Plan<N>::N1)
     // transform fills only after every thread has read its inputs
     static_assert(sizeof(float2) * kHs * (N / 2 + 1) <= 2 * E::APART, "staging fits the operand buffers");
     float2* hs = (float2*)e.ahi();
+    const int2 later = later_block(152 * 5, (int64_t)NKX * ny * nz);
+    if (later.x >= 0)
+        for (int kx = tid; kx < NKX; kx += E::T)
+            prefetch_l2(src + (size_t)(later.x * kIxRows) + (size_t)ny * (later.y + (size_t)nz * kx));
     for (int k = tid; k < kIxRows * NKX; k += blockDim.x) {
         const int row = k & (kIxRows - 1), kx = k >> 4;
         hs[kx * kHs + row] = src[(size_t)(y0 + row) + (size_t)ny * (z + (size_t)nz * kx)];
@@ -630,7 +642,7 @@ __global__ void __launch_bounds__(kIxLines * Plan<N>::N1)
     __syncthreads();
     const int f1 = tid % kIxLines, j1 = tid / kIxLines;
     const bool act = j1 < N2;
-    float2 v[N1], o[N2];
+    float2 v[N1];
     if (act) {
         const int ra = f1, rb = f1 + kIxLines;
 #pragma unroll
@@ -652,15 +664,15 @@ __global__ void __launch_bounds__(kIxLines * Plan<N>::N1)
         }
     }
     __syncthreads();                             // every input is in registers: the staging area becomes the operand
-    e.template dft<N1, N2, +1, false>(v, act, f1, j1, o);
     const int f2 = tid / N1, i2 = tid % N1;
-    float* ra = A + (size_t)N * ((size_t)(y0 + f2) + (size_t)ny * z);
-    float* rb = A + (size_t)N * ((size_t)(y0 + f2 + kIxLines) + (size_t)ny * z);
-#pragma unroll
-    for (int k2 = 0; k2 < N2; ++k2) {
-        ra[i2 + N1 * k2] = o[k2].x;
-        rb[i2 + N1 * k2] = o[k2].y;
-    }
+    float* ra = A + (size_t)N * ((size_t)(y0 + f2) + (size_t)ny * z) + i2;
+    float* rb = ra + (size_t)N * kIxLines;
+    e.template dft<N1, N2, false, true, false>(
+        0, [&](int n1) { return v[n1]; },
+        [&](int k2, float2 y) {
+            ra[N1 * k2] = y.x;
+            rb[N1 * k2] = y.y;
+        });
     e.finish();
 }
 
@@ -687,7 +699,7 @@ cudaError_t run_pass(ftr_ctx* c, int pass, bool launch) {
     cudaError_t e;
     switch (pass) {
         case 0: {
-            using E = Tc<N, kFxLines, P, true, false>;
+            using E = Tc<N, kFxLines, P, false, 1, true>;
             const size_t smem = E::BYTES;
             if ((e = set_smem(k_tc_fx<N, P>, smem, c->device)) != cudaSuccess) return e;
             if (!launch) return cudaSuccess;
@@ -698,8 +710,8 @@ cudaError_t run_pass(ftr_ctx* c, int pass, bool launch) {
             break;
         }
         case 1: {
-            using E = Tc<N, TcLines<N>::value, P, true, false>;
-            const size_t smem = E::BYTES + sizeof(float2) * (TcLines<N>::value + 1) * N;
+            using E = Tc<N, TcLines<N>::value, P, false, 3, true>;
+            const size_t smem = E::BYTES;
             if ((e = set_smem(k_tc_fy<N, P>, smem, c->device)) != cudaSuccess) return e;
             if (!launch) return cudaSuccess;
             dim3 grid(c->g.n[2] / TcLines<N>::value, c->g.n[0] / 2 + 1);
@@ -709,7 +721,7 @@ cudaError_t run_pass(ftr_ctx* c, int pass, bool launch) {
             break;
         }
         case 2: {
-            using E = Tc<N, TcLinesZ<N>::value, P, true, true>;
+            using E = Tc<N, TcLinesZ<N>::value, P, false, 3, false>;
             const size_t smem = E::BYTES;
             if ((e = set_smem(k_tc_fz<N, P>, smem, c->device)) != cudaSuccess) return e;
             if (!launch) return cudaSuccess;
@@ -723,7 +735,7 @@ cudaError_t run_pass(ftr_ctx* c, int pass, bool launch) {
             break;
         }
         case 3: {
-            using E = Tc<N, TcLines<N>::value, P, false, true>;
+            using E = Tc<N, TcLines<N>::value, P, true, 1, false>;
             const size_t smem = E::BYTES;
             if ((e = set_smem(k_tc_iy<N, P>, smem, c->device)) != cudaSuccess) return e;
             if (!launch) return cudaSuccess;
@@ -732,7 +744,7 @@ cudaError_t run_pass(ftr_ctx* c, int pass, bool launch) {
             break;
         }
         default: {
-            using E = Tc<N, kIxLines, P, false, true>;
+            using E = Tc<N, kIxLines, P, true, 1, false>;
             const size_t smem = E::BYTES;
             if ((e = set_smem(k_tc_ix<N, P>, smem, c->device)) != cudaSuccess) return e;
             if (!launch) return cudaSuccess;
