@@ -204,6 +204,13 @@ struct Xchg {
     __device__ __forceinline__ static int idxr(int f, int j, int k1) { return f + P1 * k1 + P2R * j; }
 };
 
+// The threads of step 1 (and of step 2 in swapped roles) are the CTA's first F N2,
+// thread t working on line t / N2 (or t % F), so that the others are whole warps:
+// cut into lines of NT like step 2's, a third to a half of every warp's lanes idled
+// where N1 > N2.  384^3: x 87 -> 75, y 119 -> 109, z 171 -> 152 us.  (Step 2 where N1 <
+// N2 keeps lines of NT: packed lines of N1 = 12 were no faster, 18.3 -> 19.1 us for the
+// inverse x pass of 192^3.)
+//
 // Step 1 of a length-N transform: regs hold x[N2 n1 + j]; afterwards the
 // twiddled step-1 results sit in the exchange buffer.  tw = the axis table
 // (W_N^m, then W_N^(j k1) as [k1 < N1][j < N2], then as [k1 < N2][j < N1]).

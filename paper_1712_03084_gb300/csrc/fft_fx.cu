@@ -66,9 +66,9 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT, N == 256 ? 3 : (
         }
         return;
     }
-    const int f = tid / X::NT, r = tid % X::NT;
     const int lz = z & 7;
-    if (r < X::N2) {
+    if (tid < kLines * X::N2) {
+        const int f = tid / X::N2, r = tid % X::N2;
         const int ra = f < 16 ? f : f - 16;
         const int rb = f < 16 ? f : f - 8;
         const int ca = f < 16 ? 0 : 2;
@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT, N == 256 ? 3 : (
         fft_step1<N, kLines, -1>(v, f, r, smem, tw);
     }
     __syncthreads();
+    const int f = tid / X::NT, r = tid % X::NT;
     float2 o[X::N2];
     if (r < X::N1) fft_step2<N, kLines, -1>(o, f, r, smem);
     __syncthreads();

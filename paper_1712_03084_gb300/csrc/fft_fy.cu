@@ -50,17 +50,18 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
     live_z_range(meta, zl, zh);
     if (z0 + F <= zl || z0 >= zh) return;
     // step-1 mapping: element index fastest (contiguous y lines)
-    const int f1 = tid / X::NT, r1 = tid % X::NT;
+    const int f1 = tid / X::N2, r1 = tid % X::N2;
+    const bool act1 = tid < F * X::N2;
     // step-2 mapping: line index fastest (contiguous z in the output)
     const int f2 = tid % F, i2 = tid / F;
     const size_t out_base = (size_t)(z0 + f2) + (size_t)nz * ((size_t)N * kx);
     // the transformed x component waits in shared memory (line index fastest)
     float2* stash = smem + X::SIZE;
     const float2* line = s0 + (size_t)N * (z0 + f1 + (size_t)nz * kx);
-    const unsigned rows = live_rows(meta, z0 + f1);
+    const unsigned rows = act1 ? live_rows(meta, z0 + f1) : 0u;
     // the y and z components' lines go to L2 while the x component is
     // transformed (one prefetch per 128-byte line per thread)
-    if (r1 < X::N2 && (r1 & 15) == 0) {
+    if ((r1 & 15) == 0) {
 #pragma unroll
         for (int n1 = 0; n1 < X::N1; ++n1) {
             if (!((rows >> (X::N2 * n1 / 16)) & 1u)) continue;
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
     }
     const uint64_t pin = l2_evict_first(), pout = l2_evict_last();
     // x component: transform along y and park it (line index fastest)
-    if (r1 < X::N2) load_step1<N, F>(line, r1, f1, smem, tw, pin, rows);
+    if (act1) load_step1<N, F>(line, r1, f1, smem, tw, pin, rows);
     __syncthreads();
     float2 o[X::N2];
     if (i2 < X::N1) fft_step2<N, F, -1>(o, f2, i2, smem);
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
         for (int k2 = 0; k2 < X::N2; ++k2) stash[f2 + (F + 1) * (i2 + X::N1 * k2)] = o[k2];
     }
     // y component: transform, then W = x + j w_y y goes out as field 0
-    if (r1 < X::N2) load_step1<N, F>(line + Mh, r1, f1, smem, tw, pin, rows);
+    if (act1) load_step1<N, F>(line + Mh, r1, f1, smem, tw, pin, rows);
     __syncthreads();
     if (i2 < X::N1) fft_step2<N, F, -1>(o, f2, i2, smem);
     __syncthreads();
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
         }
     }
     // z component: transform and write as field 1
-    if (r1 < X::N2) load_step1<N, F>(line + 2 * Mh, r1, f1, smem, tw, pin, rows);
+    if (act1) load_step1<N, F>(line + 2 * Mh, r1, f1, smem, tw, pin, rows);
     __syncthreads();
     if (i2 < X::N1) {
         fft_step2<N, F, -1>(o, f2, i2, smem);
@@ -144,23 +145,24 @@ __global__ void __launch_bounds__(16 * Xchg<N, 16>::NT, 2)
                              &mbar[c]);
     }
     __syncthreads();
-    const int f1 = tid / X::NT, r1 = tid % X::NT;
+    const int f1 = tid / X::N2, r1 = tid % X::N2;
+    const bool act1 = tid < F * X::N2;
     const int f2 = tid % F, i2 = tid / F;
     const size_t out_base = (size_t)(z0 + f2) + (size_t)nz * ((size_t)N * kx);
-    const unsigned rows = live_rows(meta, z0 + f1);
+    const unsigned rows = act1 ? live_rows(meta, z0 + f1) : 0u;
     float2* stash = smem;                      // the x component's buffer, once its exchange is done
     float2 o[X::N2];
     for (int c = 0; c < 3; ++c) {
         float2* B = smem + c * BUF;
         if (!tc::mbar_wait(&mbar[c], 0, 1u << 22)) atomicExch(err, 1);
         float2 v[X::N1];
-        if (r1 < X::N2) {
+        if (act1) {
 #pragma unroll
             for (int n1 = 0; n1 < X::N1; ++n1)
                 v[n1] = (rows >> (X::N2 * n1 / 16)) & 1u ? B[f1 * N + X::N2 * n1 + r1] : make_float2(0.f, 0.f);
         }
         __syncthreads();                       // the staged lines are in registers: B becomes the exchange
-        if (r1 < X::N2) fft_step1<N, F, -1>(v, f1, r1, B, tw);
+        if (act1) fft_step1<N, F, -1>(v, f1, r1, B, tw);
         __syncthreads();
         if (i2 < X::N1) fft_step2<N, F, -1>(o, f2, i2, B);
         if (c == 0) {

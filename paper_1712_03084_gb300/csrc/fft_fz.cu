@@ -42,36 +42,38 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
     const int ky0 = blockIdx.x * F;
     const int kx = blockIdx.y;
     const int tid = threadIdx.x;
-    const int f = tid / X::NT, r = tid % X::NT;
+    const int f1 = tid / X::N2, r1 = tid % X::N2;     // elements r1 + N2 n1 in, and out
+    const int f = tid / X::NT, r = tid % X::NT;       // bins r + N1 k2
+    const bool act1 = tid < F * X::N2, act = r < X::N1;
     int zl, zh;
     live_z_range(meta, zl, zh);
-    const size_t line = (size_t)N * ((size_t)(ky0 + f) + (size_t)ny * kx);
+    const size_t line = (size_t)N * ((size_t)(ky0 + f1) + (size_t)ny * kx);
     // field 1 goes to L2 while field 0 is transformed
-    if (r < X::N2 && (r & 15) == 0) {
+    if (act1 && (r1 & 15) == 0) {
 #pragma unroll
         for (int n1 = 0; n1 < X::N1; ++n1) {
-            const int z = X::N2 * n1 + r;
+            const int z = X::N2 * n1 + r1;
             if (z >= zl && z < zh) prefetch_l2(s1 + Mh + line + z);
         }
     }
     // forward z transforms of W (field 0) and of the x/y-transformed V_z (field 1)
-    if (r < X::N2) load_step1<N, F>(s1 + line, r, f, zl, zh, smem, tw);
+    if (act1) load_step1<N, F>(s1 + line, r1, f1, zl, zh, smem, tw);
     __syncthreads();
     // the transformed W waits in shared memory (the same thread reads it back)
     float2* stash = smem + X::SIZE;
     float2 xw[X::N2];
-    if (r < X::N1) {
+    if (act) {
         fft_step2<N, F, -1>(xw, f, r, smem);
 #pragma unroll
         for (int k2 = 0; k2 < X::N2; ++k2) stash[f + (F + 1) * (r + X::N1 * k2)] = xw[k2];
     }
     __syncthreads();
-    if (r < X::N2) load_step1<N, F>(s1 + Mh + line, r, f, zl, zh, smem, tw);
+    if (act1) load_step1<N, F>(s1 + Mh + line, r1, f1, zl, zh, smem, tw);
     __syncthreads();
     float2 xh[X::N2];
-    if (r < X::N1) fft_step2<N, F, -1>(xh, f, r, smem);
+    if (act) fft_step2<N, F, -1>(xh, f, r, smem);
     __syncthreads();
-    if (r < X::N1) {
+    if (act) {
         const int ky = ky0 + f;
         const float wxd = wx_scale * (float)kx;                 // |k_x| <= n_x/2 already
         const float wyd = wy_scale * (float)signed_bin(ky, ny);
@@ -92,12 +94,12 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
         fft_step1_swapped<N, F, +1>(xw, f, r, smem, tw);
     }
     __syncthreads();
-    if (r < X::N2) {
+    if (act1) {
         float2 o[X::N1];
-        fft_step2_swapped<N, F, +1>(o, f, r, smem);
+        fft_step2_swapped<N, F, +1>(o, f1, r1, smem);
         float2* dst = s1 + line;
 #pragma unroll
-        for (int k2 = 0; k2 < X::N1; ++k2) dst[r + X::N2 * k2] = o[k2];
+        for (int k2 = 0; k2 < X::N1; ++k2) dst[r1 + X::N2 * k2] = o[k2];
     }
 }
 
@@ -120,7 +122,9 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
     const int ky0 = blockIdx.x * F;
     const int kx = blockIdx.y;
     const int tid = threadIdx.x;
-    const int f = tid / X::NT, r = tid % X::NT;
+    const int f1 = tid / X::N2, r1 = tid % X::N2;     // elements r1 + N2 n1 in, and out
+    const int f = tid / X::NT, r = tid % X::NT;       // bins r + N1 k2
+    const bool act1 = tid < F * X::N2, act = r < X::N1;
     int zl, zh;
     live_z_range(meta, zl, zh);
     const uint32_t bytes = (uint32_t)(zh - zl) * (uint32_t)sizeof(float2);
@@ -151,25 +155,25 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
     };
     auto staged_step1 = [&](float2* B) {
         float2 v[X::N1];
-        if (r < X::N2) {
+        if (act1) {
 #pragma unroll
             for (int n1 = 0; n1 < X::N1; ++n1) {
-                const int z = X::N2 * n1 + r;
-                v[n1] = (z >= zl && z < zh) ? B[f * N + z] : make_float2(0.f, 0.f);
+                const int z = X::N2 * n1 + r1;
+                v[n1] = (z >= zl && z < zh) ? B[f1 * N + z] : make_float2(0.f, 0.f);
             }
         }
         __syncthreads();                          // the staged lines are in registers: B becomes the exchange
-        if (r < X::N2) fft_step1<N, F, -1>(v, f, r, B, tw);
+        if (act1) fft_step1<N, F, -1>(v, f1, r1, B, tw);
     };
     // forward z transforms of W (field 0) and of the x/y-transformed V_z (field 1)
     wait(&mbar[0]);
     staged_step1(B0);
     __syncthreads();
     float2 xw[X::N2];
-    if (r < X::N1) fft_step2<N, F, -1>(xw, f, r, B0);
+    if (act) fft_step2<N, F, -1>(xw, f, r, B0);
     __syncthreads();                              // every exchange read done: B0 becomes the stash
     float2* stash = B0;
-    if (r < X::N1) {
+    if (act) {
 #pragma unroll
         for (int k2 = 0; k2 < X::N2; ++k2) stash[f + (F + 1) * (r + X::N1 * k2)] = xw[k2];
     }
@@ -177,9 +181,9 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
     staged_step1(B1);
     __syncthreads();
     float2 xh[X::N2];
-    if (r < X::N1) fft_step2<N, F, -1>(xh, f, r, B1);
+    if (act) fft_step2<N, F, -1>(xh, f, r, B1);
     __syncthreads();
-    if (r < X::N1) {
+    if (act) {
         const int ky = ky0 + f;
         const float wxd = wx_scale * (float)kx;                 // |k_x| <= n_x/2 already
         const float wyd = wy_scale * (float)signed_bin(ky, ny);
@@ -198,12 +202,12 @@ __global__ void __launch_bounds__(F * Xchg<N, F>::NT, MinCtasF<N, F>::value)
         fft_step1_swapped<N, F, +1>(xw, f, r, B1, tw);
     }
     __syncthreads();
-    if (r < X::N2) {
+    if (act1) {
         float2 o[X::N1];
-        fft_step2_swapped<N, F, +1>(o, f, r, B1);
-        float2* dst = s1 + tile + (size_t)N * f;
+        fft_step2_swapped<N, F, +1>(o, f1, r1, B1);
+        float2* dst = s1 + tile + (size_t)N * f1;
 #pragma unroll
-        for (int k2 = 0; k2 < X::N1; ++k2) dst[r + X::N2 * k2] = o[k2];
+        for (int k2 = 0; k2 < X::N1; ++k2) dst[r1 + X::N2 * k2] = o[k2];
     }
 }
 
