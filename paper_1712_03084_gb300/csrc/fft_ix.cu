@@ -29,12 +29,19 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
     using X = Xchg<N, kLines>;
     constexpr int NKX = N / 2 + 1;
     extern __shared__ float2 smem[];
-    float2* hs = smem + X::SIZE;            // staged half spectra, [k_x][row]
+    // staged half spectra, [k_x][row]; up to 256 points the exchange reuses their place,
+    // for more CTAs per SM (256^3: 35 -> 32 us; 384^3 was slower so, 117 -> 156)
+    constexpr bool kShare = N <= 256;
+    float2* hs = kShare ? smem : smem + X::SIZE;
     const int ny = g.n[1], nz = g.n[2];
     const int y0 = blockIdx.x * kRows;
     const int z = blockIdx.y;
     const int tid = threadIdx.x;
     const uint64_t pin = l2_evict_first(), pout = l2_evict_last();
+    const int2 later = later_block(152 * 3, (int64_t)NKX * ny * nz);
+    if (later.x >= 0)
+        for (int kx = tid; kx < NKX; kx += (int)blockDim.x)
+            prefetch_l2(src + (size_t)(later.x * kRows) + (size_t)ny * (later.y + (size_t)nz * kx));
     // every load of the staging is issued before the first shared-memory store
     constexpr int kPer = (kRows * NKX + kLines * Xchg<N, kLines>::NT - 1) / (kLines * Xchg<N, kLines>::NT);
     {
@@ -54,9 +61,9 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
     }
     __syncthreads();
     const int f1 = tid % kLines, j1 = tid / kLines;
+    float2 v[X::N1];
     if (j1 < X::N2) {
         const int ra = f1, rb = f1 + kLines;
-        float2 v[X::N1];
 #pragma unroll
         for (int n1 = 0; n1 < X::N1; ++n1) {
             const int k = X::N2 * n1 + j1;
@@ -74,7 +81,11 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
             }
             v[n1] = make_float2(xa.x - xb.y, xa.y + xb.x);
         }
-        fft_step1<N, kLines, +1>(v, f1, j1, smem, tw);
+        if (!kShare) fft_step1<N, kLines, +1>(v, f1, j1, smem, tw);
+    }
+    if (kShare) {
+        __syncthreads();                         // every input is in registers
+        if (j1 < X::N2) fft_step1<N, kLines, +1>(v, f1, j1, smem, tw);
     }
     __syncthreads();
     const int f2 = tid / X::NT, i2 = tid % X::NT;
@@ -117,7 +128,8 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
 template <int N>
 cudaError_t run_ix(ftr_ctx* c) {
     using X = Xchg<N, kLines>;
-    const size_t smem = sizeof(float2) * (X::SIZE + kHs * (N / 2 + 1));
+    constexpr int kStaged = kHs * (N / 2 + 1);
+    const size_t smem = sizeof(float2) * (N <= 256 ? cmax(X::SIZE, kStaged) : X::SIZE + kStaged);
     static bool attr_done[64] = {};
     if (!attr_done[c->device & 63]) {
         cudaError_t e = cudaFuncSetAttribute(k_ix<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -353,18 +353,6 @@ struct Tc {
     }
 };
 
-// The z and inverse-x passes ask for the input of the CTA `ahead` places later in
-// launch order (about the one that takes this CTA's place) to be brought to L2, so
-// that its loads wait for L2 and not for DRAM: 307 -> 270 and 173 -> 163 us at 384^3
-// (bf16x3).  Not where a half spectrum of `elems` fits L2 and mostly is there (256^3:
-// 87 -> 90 us), nor in the y passes (no gain).  Block index, or x = -1: none.
-__device__ __forceinline__ int2 later_block(int ahead, int64_t elems) {
-    if (elems * (int64_t)sizeof(float2) <= (int64_t)128 << 20) return make_int2(-1, -1);
-    const int id = (int)(blockIdx.x + gridDim.x * blockIdx.y) + ahead;
-    if (id >= (int)(gridDim.x * gridDim.y)) return make_int2(-1, -1);
-    return make_int2(id % (int)gridDim.x, id / (int)gridDim.x);
-}
-
 // ---------------------------------------------------------------- x forward
 // Same as the fp32 x pass: 16 rows (y0.., z) of the three components from the
 // brick pool, two real rows per complex line (16 (V_x, V_y) + 8 (V_z, V_z)
