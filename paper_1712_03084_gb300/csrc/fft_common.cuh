@@ -191,13 +191,15 @@ __host__ __device__ constexpr int make_odd(int v) { return (v & 1) ? v : v + 1; 
 
 // Shared-memory exchange layout for F lines of length N: element (f, j, k1)
 // at f + P1 k1 + P2 j.  P1 and P2 are odd so that 16 consecutive lanes that
-// vary any one of f, j or k1 touch 16 different 8-byte bank pairs.
-template <int N, int F>
+// vary any one of f, j or k1 touch 16 different 8-byte bank pairs.  EIGHT: 16 lanes
+// of step 1 are 8 lines x 2 values of j instead (the inverse x pass), and P2 is 8
+// modulo 16 for them.
+template <int N, int F, bool EIGHT = false>
 struct Xchg {
     static constexpr int N1 = Plan<N>::N1, N2 = Plan<N>::N2;
     static constexpr int NT = cmax(N1, N2);               // threads per line
     static constexpr int P1 = make_odd(F + 1);
-    static constexpr int P2 = make_odd(P1 * N1);          // forward layout (j < N2, k1 < N1)
+    static constexpr int P2 = EIGHT ? (P1 * N1 + 7) / 16 * 16 + 8 : make_odd(P1 * N1);   // forward layout (j < N2, k1 < N1)
     static constexpr int P2R = make_odd(P1 * N2);         // swapped layout (j < N1, k1 < N2)
     static constexpr int SIZE = cmax(P2 * N2, P2R * N1);  // float2 elements
     __device__ __forceinline__ static int idx(int f, int j, int k1) { return f + P1 * k1 + P2 * j; }
@@ -214,10 +216,10 @@ struct Xchg {
 // Step 1 of a length-N transform: regs hold x[N2 n1 + j]; afterwards the
 // twiddled step-1 results sit in the exchange buffer.  tw = the axis table
 // (W_N^m, then W_N^(j k1) as [k1 < N1][j < N2], then as [k1 < N2][j < N1]).
-template <int N, int F, int SIGN>
+template <int N, int F, int SIGN, bool EIGHT = false>
 __device__ __forceinline__ void fft_step1(float2 (&v)[Plan<N>::N1], int f, int j, float2* xs,
                                           const float2* __restrict__ tw) {
-    using X = Xchg<N, F>;
+    using X = Xchg<N, F, EIGHT>;
     Dft<X::N1, SIGN>::run(v);
 #pragma unroll
     for (int k1 = 0; k1 < X::N1; ++k1) {
@@ -233,9 +235,9 @@ __device__ __forceinline__ void fft_step1(float2 (&v)[Plan<N>::N1], int f, int j
 
 // Step 2: thread i (< N1) of line f gathers its column and ends with
 // X[i + N1 k2] in out[k2].
-template <int N, int F, int SIGN>
+template <int N, int F, int SIGN, bool EIGHT = false>
 __device__ __forceinline__ void fft_step2(float2 (&out)[Plan<N>::N2], int f, int i, const float2* xs) {
-    using X = Xchg<N, F>;
+    using X = Xchg<N, F, EIGHT>;
 #pragma unroll
     for (int j = 0; j < X::N2; ++j) out[j] = xs[X::idx(f, j, i)];
     Dft<X::N2, SIGN>::run(out);
@@ -308,6 +310,12 @@ __device__ __forceinline__ int2 later_block(int ahead, int64_t elems) {
     if (id >= (int)(gridDim.x * gridDim.y)) return make_int2(-1, -1);
     return make_int2(id % (int)gridDim.x, id / (int)gridDim.x);
 }
+
+// Element of the inverse x passes' staged half spectra, [k_x][16 rows]: the halves of
+// odd k_x are exchanged, so that 16 lanes of 8 rows x 2 consecutive k_x touch 16
+// different bank pairs.  With EIGHT above: half of the pass's shared-memory wavefronts
+// were conflicts; 256^3 32.7 -> 30.7 us, 384^3 110 -> 100 (bf16x3 157 -> 146).
+__device__ __forceinline__ int staged_at(int kx, int row) { return 16 * kx + (row ^ ((kx & 1) << 3)); }
 
 // L2 eviction priorities for the passes' intermediates: a pass reads its
 // input once (evict first: the lines are dead after) and writes the next

@@ -18,19 +18,18 @@ namespace {
 
 constexpr int kRows = 16;
 constexpr int kLines = 8;     // complex transforms per CTA (row pairs r, r + 8)
-constexpr int kHs = kRows + 1;
 
 template <int N>
 __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
     k_ix(GridDev g, const float2* __restrict__ src, float* __restrict__ A, const float2* __restrict__ tw,
          float2* __restrict__ rowmm) {
     pdl_wait();
-    __shared__ float2 s_mm[kRows][Xchg<N, kLines>::NT];
-    using X = Xchg<N, kLines>;
+    using X = Xchg<N, kLines, true>;
+    __shared__ float2 s_mm[kRows][X::NT];
     constexpr int NKX = N / 2 + 1;
     extern __shared__ float2 smem[];
     // staged half spectra, [k_x][row]; up to 256 points the exchange reuses their place,
-    // for more CTAs per SM (256^3: 35 -> 32 us; 384^3 was slower so, 117 -> 156)
+    // for more CTAs per SM (256^3: 35 -> 32.6 us; 384^3 was slower so, 117 -> 156)
     constexpr bool kShare = N <= 256;
     float2* hs = kShare ? smem : smem + X::SIZE;
     const int ny = g.n[1], nz = g.n[2];
@@ -43,7 +42,7 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
         for (int kx = tid; kx < NKX; kx += (int)blockDim.x)
             prefetch_l2(src + (size_t)(later.x * kRows) + (size_t)ny * (later.y + (size_t)nz * kx));
     // every load of the staging is issued before the first shared-memory store
-    constexpr int kPer = (kRows * NKX + kLines * Xchg<N, kLines>::NT - 1) / (kLines * Xchg<N, kLines>::NT);
+    constexpr int kPer = (kRows * NKX + kLines * X::NT - 1) / (kLines * X::NT);
     {
         float2 st[kPer];
 #pragma unroll
@@ -56,7 +55,7 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
             const int k = tid + i * (int)blockDim.x;
-            if (k < kRows * NKX) hs[(k >> 4) * kHs + (k & (kRows - 1))] = st[i];
+            if (k < kRows * NKX) hs[staged_at(k >> 4, k & (kRows - 1))] = st[i];
         }
     }
     __syncthreads();
@@ -69,29 +68,29 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
             const int k = X::N2 * n1 + j1;
             float2 xa, xb;
             if (k <= N / 2) {
-                xa = hs[k * kHs + ra];
-                xb = hs[k * kHs + rb];
+                xa = hs[staged_at(k, ra)];
+                xb = hs[staged_at(k, rb)];
                 if (k == 0 || k == N / 2) {
                     xa.y = 0.f;
                     xb.y = 0.f;
                 }
             } else {
-                xa = cconj(hs[(N - k) * kHs + ra]);
-                xb = cconj(hs[(N - k) * kHs + rb]);
+                xa = cconj(hs[staged_at(N - k, ra)]);
+                xb = cconj(hs[staged_at(N - k, rb)]);
             }
             v[n1] = make_float2(xa.x - xb.y, xa.y + xb.x);
         }
-        if (!kShare) fft_step1<N, kLines, +1>(v, f1, j1, smem, tw);
+        if (!kShare) fft_step1<N, kLines, +1, true>(v, f1, j1, smem, tw);
     }
     if (kShare) {
         __syncthreads();                         // every input is in registers
-        if (j1 < X::N2) fft_step1<N, kLines, +1>(v, f1, j1, smem, tw);
+        if (j1 < X::N2) fft_step1<N, kLines, +1, true>(v, f1, j1, smem, tw);
     }
     __syncthreads();
     const int f2 = tid / X::NT, i2 = tid % X::NT;
     if (i2 < X::N1) {
         float2 o[X::N2];
-        fft_step2<N, kLines, +1>(o, f2, i2, smem);
+        fft_step2<N, kLines, +1, true>(o, f2, i2, smem);
         float* ra = A + (size_t)N * ((size_t)(y0 + f2) + (size_t)ny * z);
         float* rb = A + (size_t)N * ((size_t)(y0 + f2 + kLines) + (size_t)ny * z);
         float mna = INFINITY, mxa = -INFINITY, mnb = INFINITY, mxb = -INFINITY;
@@ -127,8 +126,8 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
 
 template <int N>
 cudaError_t run_ix(ftr_ctx* c) {
-    using X = Xchg<N, kLines>;
-    constexpr int kStaged = kHs * (N / 2 + 1);
+    using X = Xchg<N, kLines, true>;
+    constexpr int kStaged = kRows * (N / 2 + 1);
     const size_t smem = sizeof(float2) * (N <= 256 ? cmax(X::SIZE, kStaged) : X::SIZE + kStaged);
     static bool attr_done[64] = {};
     if (!attr_done[c->device & 63]) {

@@ -598,7 +598,6 @@ __global__ void __launch_bounds__(TcLines<N>::value * Plan<N>::N1, N >= 384 ? 2 
 // ---------------------------------------------------------------- x inverse
 constexpr int kIxRows = 16;
 constexpr int kIxLines = 8;
-constexpr int kHs = kIxRows + 1;
 
 template <int N, int P>
 __global__ void __launch_bounds__(kIxLines * Plan<N>::N1, N >= 384 ? 5 : 9)
@@ -617,7 +616,7 @@ __global__ void __launch_bounds__(kIxLines * Plan<N>::N1, N >= 384 ? 5 : 9)
     e.init(smem_raw, table, tw, err);
     // the half-spectrum rows are staged in the operand buffers, which the
     // transform fills only after every thread has read its inputs
-    static_assert(sizeof(float2) * kHs * (N / 2 + 1) <= 2 * E::APART, "staging fits the operand buffers");
+    static_assert(sizeof(float2) * kIxRows * (N / 2 + 1) <= 2 * E::APART, "staging fits the operand buffers");
     float2* hs = (float2*)e.ahi();
     const int2 later = later_block(152 * 5, (int64_t)NKX * ny * nz);
     if (later.x >= 0)
@@ -625,7 +624,7 @@ __global__ void __launch_bounds__(kIxLines * Plan<N>::N1, N >= 384 ? 5 : 9)
             prefetch_l2(src + (size_t)(later.x * kIxRows) + (size_t)ny * (later.y + (size_t)nz * kx));
     for (int k = tid; k < kIxRows * NKX; k += blockDim.x) {
         const int row = k & (kIxRows - 1), kx = k >> 4;
-        hs[kx * kHs + row] = src[(size_t)(y0 + row) + (size_t)ny * (z + (size_t)nz * kx)];
+        hs[staged_at(kx, row)] = src[(size_t)(y0 + row) + (size_t)ny * (z + (size_t)nz * kx)];
     }
     __syncthreads();
     const int f1 = tid % kIxLines, j1 = tid / kIxLines;
@@ -638,15 +637,15 @@ __global__ void __launch_bounds__(kIxLines * Plan<N>::N1, N >= 384 ? 5 : 9)
             const int k = N2 * n1 + j1;
             float2 xa, xb;
             if (k <= N / 2) {
-                xa = hs[k * kHs + ra];
-                xb = hs[k * kHs + rb];
+                xa = hs[staged_at(k, ra)];
+                xb = hs[staged_at(k, rb)];
                 if (k == 0 || k == N / 2) {
                     xa.y = 0.f;
                     xb.y = 0.f;
                 }
             } else {
-                xa = cconj(hs[(N - k) * kHs + ra]);
-                xb = cconj(hs[(N - k) * kHs + rb]);
+                xa = cconj(hs[staged_at(N - k, ra)]);
+                xb = cconj(hs[staged_at(N - k, rb)]);
             }
             v[n1] = make_float2(xa.x - xb.y, xa.y + xb.x);
         }
