@@ -314,7 +314,7 @@ __device__ __forceinline__ int2 later_block(int ahead, int64_t elems) {
 // Element of the inverse x passes' staged half spectra, [k_x][16 rows]: the halves of
 // odd k_x are exchanged, so that 16 lanes of 8 rows x 2 consecutive k_x touch 16
 // different bank pairs.  With EIGHT above: half of the pass's shared-memory wavefronts
-// were conflicts; 256^3 32.7 -> 30.7 us, 384^3 110 -> 100 (bf16x3 157 -> 146).
+// were conflicts; 256^3 32.7 -> 30.7 us, 384^3 110 -> 99 (bf16x3 157 -> 146).
 __device__ __forceinline__ int staged_at(int kx, int row) { return 16 * kx + (row ^ ((kx & 1) << 3)); }
 
 // L2 eviction priorities for the passes' intermediates: a pass reads its

@@ -28,10 +28,9 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
     __shared__ float2 s_mm[kRows][X::NT];
     constexpr int NKX = N / 2 + 1;
     extern __shared__ float2 smem[];
-    // staged half spectra, [k_x][row]; up to 256 points the exchange reuses their place,
-    // for more CTAs per SM (256^3: 35 -> 32.6 us; 384^3 was slower so, 117 -> 156)
-    constexpr bool kShare = N <= 256;
-    float2* hs = kShare ? smem : smem + X::SIZE;
+    // staged half spectra, [k_x][row]; the exchange reuses their place, for more CTAs
+    // per SM (256^3: 35 -> 32.6 us, 384^3 99 -> 96)
+    float2* hs = smem;
     const int ny = g.n[1], nz = g.n[2];
     const int y0 = blockIdx.x * kRows;
     const int z = blockIdx.y;
@@ -80,12 +79,9 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
             }
             v[n1] = make_float2(xa.x - xb.y, xa.y + xb.x);
         }
-        if (!kShare) fft_step1<N, kLines, +1, true>(v, f1, j1, smem, tw);
     }
-    if (kShare) {
-        __syncthreads();                         // every input is in registers
-        if (j1 < X::N2) fft_step1<N, kLines, +1, true>(v, f1, j1, smem, tw);
-    }
+    __syncthreads();                             // every input is in registers
+    if (j1 < X::N2) fft_step1<N, kLines, +1, true>(v, f1, j1, smem, tw);
     __syncthreads();
     const int f2 = tid / X::NT, i2 = tid % X::NT;
     if (i2 < X::N1) {
@@ -127,8 +123,7 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
 template <int N>
 cudaError_t run_ix(ftr_ctx* c) {
     using X = Xchg<N, kLines, true>;
-    constexpr int kStaged = kRows * (N / 2 + 1);
-    const size_t smem = sizeof(float2) * (N <= 256 ? cmax(X::SIZE, kStaged) : X::SIZE + kStaged);
+    const size_t smem = sizeof(float2) * cmax(X::SIZE, kRows * (N / 2 + 1));
     static bool attr_done[64] = {};
     if (!attr_done[c->device & 63]) {
         cudaError_t e = cudaFuncSetAttribute(k_ix<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
