@@ -354,13 +354,14 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
     }
     // what ftr_reset clears, in one block and one memset: the brick counts, the
     // point count, the dropped points and the wild flags (n_bricks is even)
-    ALLOC(c->d_brick_cnt, c->n_bricks + 6);
-    c->d_npts = reinterpret_cast<int64_t*>(c->d_brick_cnt + c->n_bricks);
+    const size_t counters = (size_t)c->n_bricks << count_shift(c->n_bricks);
+    ALLOC(c->d_brick_cnt, counters + 6);
+    c->d_npts = reinterpret_cast<int64_t*>(c->d_brick_cnt + counters);
     c->d_dropped = reinterpret_cast<unsigned long long*>(c->d_npts + 1);
     c->d_wild = reinterpret_cast<int*>(c->d_dropped + 1);
-    c->reset_bytes = sizeof(int) * ((size_t)c->n_bricks + 6);
+    c->reset_bytes = sizeof(int) * (counters + 6);
     ALLOC(c->d_brick_off, c->n_bricks + 1);
-    ALLOC(c->d_brick_cursor, c->n_bricks);
+    ALLOC(c->d_brick_cursor, counters);
     ALLOC(c->d_brick_slot, c->n_bricks);
     ALLOC(c->d_active, c->n_bricks);
     ALLOC(c->d_meta, kMetaInts);
@@ -1602,7 +1603,7 @@ int64_t context_bytes(const int n[3], const Caps& k) {
     int64_t b = 0;
     b += k.pts * (int64_t)(sizeof(int4) + 2 * sizeof(float4));
     b += k.stage + k.tex_stage;
-    b += nb * (int64_t)sizeof(int) * 5 + (nb / kBrickScanTile + 1) * (int64_t)sizeof(int4) + 64;
+    b += (nb * 3 + 2 * (nb << count_shift((int)nb))) * (int64_t)sizeof(int) + (nb / kBrickScanTile + 1) * (int64_t)sizeof(int4) + 64;
     b += k.entries * (int64_t)sizeof(int);
     b += k.units * (int64_t)sizeof(int4);
     b += k.heavy * (4 * kBrickVox * 8 + 4) + nb * 8;   // heavy-brick accumulators, chunk offsets

@@ -125,6 +125,7 @@ __device__ __forceinline__ void ingest_one(bool live, const float* p, const floa
     // per brick slot k of the at most 2 x 2 x 2 bricks the stencil overlaps, a
     // run of lanes counting into the same brick adds its length with one atomic
     const int lane = threadIdx.x & 31;
+    const int shift = count_shift(g.nb[0] * g.nb[1] * g.nb[2]);
     int lo[3] = {0, 0, 0}, hi[3] = {-1, -1, -1};
     const bool any = stencil_bricks(rec, g.mode, lo, hi);
 #pragma unroll
@@ -133,7 +134,7 @@ __device__ __forceinline__ void ingest_one(bool live, const float* p, const floa
         const bool valid = any && bx <= hi[0] && by <= hi[1] && bz <= hi[2];
         const int b = valid ? bx + g.nb[0] * (by + g.nb[1] * bz) : -1;
         const Run r = run_of(b, lane);
-        if (valid && lane == r.first) atomicAdd(&cnt[b], r.len);
+        if (valid && lane == r.first) atomicAdd(&cnt[b << shift], r.len);
     }
     if (!live) return;
     pbase[dst] = rec;
@@ -188,6 +189,7 @@ __global__ void k_brick_fill(const int4* __restrict__ pbase, const int64_t* __re
     pdl_wait();
     const int64_t n = *npts;
     const int lane = threadIdx.x & 31;
+    const int shift = count_shift(g.nb[0] * g.nb[1] * g.nb[2]);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     // warp-uniform loop: every lane reaches each match below
     for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n; i0 += stride) {
@@ -203,7 +205,7 @@ __global__ void k_brick_fill(const int4* __restrict__ pbase, const int64_t* __re
             const int b = valid ? bx + g.nb[0] * (by + g.nb[1] * bz) : -1;
             run[k] = run_of(b, lane);
             pos[k] = 0;
-            if (valid && lane == run[k].first) pos[k] = atomicAdd(&cursor[b], run[k].len);
+            if (valid && lane == run[k].first) pos[k] = atomicAdd(&cursor[b << shift], run[k].len);
             if (!valid) run[k].len = 0;
         }
 #pragma unroll
@@ -293,7 +295,7 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_sums(const int* __restric
     for (int k = 0; k < kTile / kScanT; ++k) {
         const int b = blockIdx.x * kTile + k * kScanT + threadIdx.x;
         if (b < nb) {
-            const int4 q = brick_counts(cnt[b]);
+            const int4 q = brick_counts(cnt[b << count_shift(nb)]);
             v.x += q.x;
             v.y += q.y;
             v.z += q.z;
@@ -358,9 +360,10 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restri
     }
     static_assert(kTile == kScanT, "a thread per brick");
     int zmin = 0x7fffffff, zmax = -1;
+    const int shift = count_shift(nb);
     {
         const int b = blockIdx.x * kTile + threadIdx.x;
-        const int c = b < nb ? cnt[b] : 0;
+        const int c = b < nb ? cnt[b << shift] : 0;
         const int4 q = brick_counts(c);
         // rank of the brick's full chunks and of its last chunk in their classes
         const int nlast = c - (q.z - 1) * kChunk;
@@ -383,7 +386,7 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restri
         __syncthreads();
         if (b < nb) {
             off[b] = run.x + ex.x;
-            cursor[b] = run.x + ex.x;
+            cursor[b << shift] = run.x + ex.x;
             if (c > 0) {
                 const int s = run.y + ex.y;
                 slot[b] = s;
@@ -399,7 +402,7 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restri
                 zmin = zmax = bz;
                 // its pair of brick rows = 16 grid rows; the first brick of a run along x sets the bit
                 const int by = (b - bz * nbxy) / nbx;
-                if (b % nbx == 0 || cnt[b - 1] == 0) atomicOr(&meta[kMetaRows + bz], 1 << (by >> 1));
+                if (b % nbx == 0 || cnt[(b - 1) << shift] == 0) atomicOr(&meta[kMetaRows + bz], 1 << (by >> 1));
             } else {
                 slot[b] = -1;
             }
