@@ -536,9 +536,17 @@ __device__ __forceinline__ void ssim_terms(float mx, float my, float vx, float v
 // ends after its loads; a tile that touches the image border takes the windows
 // cut at it.  (16 x 16 pixels with direct, bounds-tested 121-tap sums for the
 // means and the moments ran 182 + 137 + 57 us for the three scales of a 1920 x
-// 1080 view whose silhouette covers an eighth of it.)
-__global__ void __launch_bounds__(256) k_ap_ssim(const float* __restrict__ X, const float* __restrict__ Y,
-                                                 const uint8_t* __restrict__ S, int w, int h,
+// 1080 view whose silhouette covers an eighth of it.)  One launch for the tiles of
+// all scales: each scale's last tiles are a dependent chain of some 10 us that the
+// others now cover (26 + 23 + 11 us one after another, now 34).
+struct ApScales {
+    int64_t at[4];            // first tile (= partial of 4 terms) of each scale, and their number
+    int64_t plane[3];         // first pixel of each scale in X, Y and S
+    int w[3], h[3], gx[3];    // pixels, tiles per row
+};
+
+__global__ void __launch_bounds__(256) k_ap_ssim(const float* __restrict__ Xs, const float* __restrict__ Ys,
+                                                 const uint8_t* __restrict__ Ss, const __grid_constant__ ApScales sc,
                                                  const __grid_constant__ Taps tp, double* __restrict__ part) {
     __shared__ float sx[kHaloH][kHaloW];
     __shared__ float sy[kHaloH][kHaloW];
@@ -547,10 +555,16 @@ __global__ void __launch_bounds__(256) k_ap_ssim(const float* __restrict__ X, co
     __shared__ float rowy[kHaloH][kSsimW];
     __shared__ int rown[kHaloH][kSsimW];
     __shared__ double red[4][8];
-    const int bx = blockIdx.x * kSsimW - kR, by = blockIdx.y * kSsimH - kR;
+    const int j3 = (int64_t)blockIdx.x < sc.at[1] ? 0 : ((int64_t)blockIdx.x < sc.at[2] ? 1 : 2);
+    const float* X = Xs + sc.plane[j3];
+    const float* Y = Ys + sc.plane[j3];
+    const uint8_t* S = Ss + sc.plane[j3];
+    const int w = sc.w[j3], h = sc.h[j3];
+    const int tile = (int)(blockIdx.x - sc.at[j3]), tile_y = tile / sc.gx[j3], tile_x = tile - tile_y * sc.gx[j3];
+    const int bx = tile_x * kSsimW - kR, by = tile_y * kSsimH - kR;
     const int tx = threadIdx.x % kSsimW, ty = 2 * (threadIdx.x / kSsimW);
-    const int x = blockIdx.x * kSsimW + tx, y = blockIdx.y * kSsimH + ty;
-    double* out = part + 4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x);
+    const int x = tile_x * kSsimW + tx, y = tile_y * kSsimH + ty;
+    double* out = part + 4 * (int64_t)blockIdx.x;
     const bool in0 = x < w && y < h && S[(int64_t)y * w + x];
     const bool in1 = x < w && y + 1 < h && S[(int64_t)(y + 1) * w + x];
     if (!__syncthreads_or(in0 || in1)) {
@@ -580,7 +594,7 @@ __global__ void __launch_bounds__(256) k_ap_ssim(const float* __restrict__ X, co
                 n += ss[hy][hx + k];
             }
         } else {
-            const int gx = blockIdx.x * kSsimW + hx;
+            const int gx = tile_x * kSsimW + hx;
             for (int k = max(0, kR - gx); k <= min(2 * kR, kR + w - 1 - gx); ++k) {
                 rx += tp.g[k] * sx[hy][hx + k];
                 ry += tp.g[k] * sy[hy][hx + k];
@@ -704,10 +718,6 @@ __global__ void __launch_bounds__(256) k_ap_ssim(const float* __restrict__ X, co
 
 // The twelve sums of the three scales, one CTA each: CTA 4 j + m adds term m of
 // scale j over that scale's tiles in a fixed order.
-struct ApScales {
-    int64_t at[3], n[3];      // first partial (of 4 terms) and number of tiles per scale
-};
-
 __global__ void __launch_bounds__(256) k_ap_final(const double* __restrict__ part, ApScales sc,
                                                   double* __restrict__ out) {
     __shared__ double s[8];
@@ -715,7 +725,7 @@ __global__ void __launch_bounds__(256) k_ap_final(const double* __restrict__ par
     const double* p = part + 4 * sc.at[j] + m;
     double acc = 0.0;
 #pragma unroll 8
-    for (int64_t b = threadIdx.x; b < sc.n[j]; b += 256) acc += p[4 * b];
+    for (int64_t b = threadIdx.x; b < sc.at[j + 1] - sc.at[j]; b += 256) acc += p[4 * b];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = acc;
@@ -947,27 +957,26 @@ int ftr_eval_appearance(ftr_ctx* c, int w, int h, const float* rendered_depth, c
     c->launches++;
     Taps tp;
     for (int i = -kR; i <= kR; ++i) tp.g[i + kR] = (float)exp(-(double)(i * i) / (2.0 * 1.5 * 1.5));
-    for (int j = 0; j < 3; ++j) {
-        if (j) {
-            const int64_t n = (int64_t)ws[j] * hs[j];
-            if (n > 0) {
-                k_ap_down<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(X + off[j - 1], Y + off[j - 1], S + off[j - 1],
-                                                                       ws[j - 1], ws[j], hs[j], X + off[j], Y + off[j],
-                                                                       S + off[j]);
-                c->launches++;
-            }
-        }
-        if ((int64_t)gx[j] * gy[j] > 0) {
-            k_ap_ssim<<<dim3(gx[j], gy[j]), 256, 0, st>>>(X + off[j], Y + off[j], S + off[j], ws[j], hs[j], tp,
-                                                         ev->part + 4 * boff[j]);
+    for (int j = 1; j < 3; ++j) {
+        const int64_t n = (int64_t)ws[j] * hs[j];
+        if (n > 0) {
+            k_ap_down<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(X + off[j - 1], Y + off[j - 1], S + off[j - 1],
+                                                                   ws[j - 1], ws[j], hs[j], X + off[j], Y + off[j],
+                                                                   S + off[j]);
             c->launches++;
         }
     }
     ApScales sc;
     for (int j = 0; j < 3; ++j) {
         sc.at[j] = boff[j];
-        sc.n[j] = boff[j + 1] - boff[j];
+        sc.plane[j] = off[j];
+        sc.w[j] = ws[j];
+        sc.h[j] = hs[j];
+        sc.gx[j] = (int)gx[j];
     }
+    sc.at[3] = boff[3];
+    k_ap_ssim<<<(unsigned)boff[3], 256, 0, st>>>(X, Y, S, sc, tp, ev->part);
+    c->launches++;
     k_ap_final<<<12, 256, 0, st>>>(ev->part, sc, ev->part + 4 * boff[3]);
     c->launches++;
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "ftr_eval_appearance: kernels");
