@@ -312,8 +312,8 @@ int64_t ftr_estimate_bytes(const int grid_n[3], int64_t points, int64_t depth_pi
  * The y, z and inverse-y FFT passes each move F lines per CTA, F in
  * {8, 16, 32}; F = -16 means 16 lines whose input tiles are fetched by bulk
  * asynchronous copies at the CTA's start: the y pass's three component
- * tiles (lines of at most 256), or the z pass's two fields, each line's
- * live z range only.  Every plan computes bit-identical results (each
+ * tiles (lines of at most 256, each line's span of live rows), or the z
+ * pass's two fields, each line's live z range only.  Every plan computes bit-identical results (each
  * line's arithmetic does not depend on the plan), only the speed differs.
  * The plane-fused path's z pass takes 8, 16 or 32 (-16 runs it with 16).
  *
