@@ -161,7 +161,7 @@ __host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 // 16-line passes: what 80 registers per thread allow while the transform still
 // fits in them (a spill of a few values at 384 points): three (24 warps) up to
 // 256, two (24 warps) at 384, where the y and z pass otherwise take 121-145
-// registers and run 12 warps (156 + 204 us, now 119 + 171); one above.
+// registers and run 12 warps (156 + 204 us, with the budget 119 + 171); one above.
 template <int N>
 struct MinCtas {
     static constexpr int value = N <= 256 ? 3 : (N <= 384 ? 2 : 1);
@@ -302,8 +302,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 // the one that takes this CTA's place) to be brought to L2, so that its loads wait for
 // L2 and not for DRAM: inverse x of 384^3 117 -> 108 us; split precision (bf16x3) z 307
 // -> 270, inverse x 173 -> 163.  Not where a half spectrum of `elems` fits L2 and mostly
-// is there (256^3: split-precision z 87 -> 90), nor in the other passes (no gain).  Block
-// index, or x = -1: none.
+// is there (256^3: split-precision z 87 -> 90), nor in the other passes (float32 z of
+// 384^3 152 -> 162, y passes no gain).  Block index, or x = -1: none.
 __device__ __forceinline__ int2 later_block(int ahead, int64_t elems) {
     if (elems * (int64_t)sizeof(float2) <= (int64_t)128 << 20) return make_int2(-1, -1);
     const int id = (int)(blockIdx.x + gridDim.x * blockIdx.y) + ahead;
