@@ -761,7 +761,8 @@ int ftr_solve(ftr_ctx* c, double* iso_level_out) {
     c->solved = false;
     c->meshed = false;
     if (!c->v_external) {
-        if ((e = launch_splat(c)) != cudaSuccess) return cuda_fail(c, e, "ftr_solve: splat");
+        if ((e = clear_classes(c)) != cudaSuccess || (e = launch_splat(c)) != cudaSuccess)
+            return cuda_fail(c, e, "ftr_solve: splat");
     }
     if ((e = launch_transforms(c)) != cudaSuccess) return cuda_fail(c, e, "ftr_solve: transforms");
     prof_begin(c, ST_LEVEL);
@@ -1041,6 +1042,7 @@ int ftr_frame_launch(ftr_ctx* c, const ftr_view* views, int k, float depth_tol, 
     // every buffer the graph captures is sized here, outside the capture
     if ((e = grow_entries(c, 8 * c->n_pts + 1)) != cudaSuccess) return cuda_fail(c, e, "ftr_frame_launch");
     if ((e = grow_heavy(c, c->n_pts)) != cudaSuccess) return cuda_fail(c, e, "ftr_frame_launch");
+    if ((e = clear_classes(c)) != cudaSuccess) return cuda_fail(c, e, "ftr_frame_launch");
     if (c->cap_verts == 0) {
         const int64_t guess = c->M / 256 + 4096;
         if ((e = grow_mesh(c, guess, guess, 2 * guess)) != cudaSuccess) return cuda_fail(c, e, "ftr_frame_launch");

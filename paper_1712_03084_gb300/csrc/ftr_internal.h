@@ -23,7 +23,8 @@ constexpr int kSplatChunk = 1024;          // (point, brick) pairs per accumulat
 // d_meta: the frame's scalars (see ftr_ctx), then per brick layer along z the
 // 16-row groups along y that hold a touched brick (bit y / 16), then the number
 // of accumulation units per size class and the units placed so far (both zero
-// between frames).
+// between frames: the accumulation clears them; after a binning whose
+// accumulation was not enqueued, class_dirty has the next frame clear them).
 constexpr int kSizeClasses = 32;
 constexpr int kMetaRows = 8;
 constexpr int kMetaClasses = kMetaRows + 64;
@@ -136,6 +137,7 @@ struct ftr_ctx {
     int* d_meta = nullptr;     // [0] active bricks, [1] entries, [2] min bz, [3] max bz, [4] accumulation
                                // ticket, [5] accumulation chunks, [6] heavy bricks,
                                // [kMetaRows + bz] live 16-row groups of brick layer bz
+    bool class_dirty = false;  // d_meta's unit counts may be left over from a binning that stopped half way
     int4* d_tile = nullptr;    // per-tile sums / offsets of the brick scan (pairs, touched, chunks, heavy)
     int* d_unit_off = nullptr; // per touched brick: first accumulation chunk; [touched] = all chunks
     int* d_heavy_idx = nullptr;  // per touched brick: index of its global accumulator, -1 for one chunk
@@ -307,6 +309,7 @@ struct IngestSets {
     int k;
 };
 cudaError_t launch_ingest_sets(ftr_ctx* c, const IngestSets& S);
+cudaError_t clear_classes(ftr_ctx* c);         // before launch_splat or a graph that holds it: settles class_dirty
 cudaError_t launch_splat(ftr_ctx* c);          // bin + accumulate into d_vpool
 cudaError_t launch_fx(ftr_ctx* c);
 cudaError_t launch_fy(ftr_ctx* c);

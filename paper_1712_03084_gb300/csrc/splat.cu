@@ -736,8 +736,26 @@ cudaError_t launch_ingest_sets(ftr_ctx* c, const IngestSets& S) {
     return cudaGetLastError();
 }
 
+// The binning adds to the unit counts and the accumulation clears them for the
+// next frame.  A solve that fails between the two (every launch reports errors
+// of the thread, also ones the application left behind) leaves them standing:
+// a frame binned on top of them would place its units at twice their number,
+// past d_units where most bricks are touched.
+cudaError_t clear_classes(ftr_ctx* c) {
+    if (!c->class_dirty) return cudaSuccess;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(c->stream, &cs);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(c->d_meta + kMetaClasses, 0, sizeof(int) * 2 * kSizeClasses, c->stream);
+    // a captured memset has not run yet: the flag stays for the next call
+    if (e == cudaSuccess && cs == cudaStreamCaptureStatusNone) c->class_dirty = false;
+    return e;
+}
+
 cudaError_t launch_splat(ftr_ctx* c) {
     cudaError_t e;
+    const bool dirty = c->class_dirty;
+    c->class_dirty = true;                       // until the accumulation is enqueued
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     if (sms <= 0) sms = 152;
@@ -761,7 +779,8 @@ cudaError_t launch_splat(ftr_ctx* c) {
                c->d_vpool, c->d_unit_off, c->d_heavy_idx, c->d_heavy_acc, c->d_heavy_done);
     c->launches++;
     prof_end(c, ST_SPLAT_ACC);
-    return cudaGetLastError();
+    if ((e = cudaGetLastError()) == cudaSuccess) c->class_dirty = dirty;
+    return e;
 }
 
 cudaError_t launch_load_dense_V(ftr_ctx* c, const float* V_dev) {
