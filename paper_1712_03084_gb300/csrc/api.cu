@@ -353,7 +353,7 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
         return FTR_ENOMEM;                                  \
     }
     // what ftr_reset clears, in one block and one memset: the brick counts, the
-    // point count, the dropped points and the wild flags (n_bricks is even)
+    // point count, the dropped points and the wild flag (n_bricks is even)
     const size_t counters = (size_t)c->n_bricks << count_shift(c->n_bricks);
     ALLOC(c->d_brick_cnt, counters + 6);
     c->d_npts = reinterpret_cast<int64_t*>(c->d_brick_cnt + counters);

@@ -122,7 +122,7 @@ struct ftr_ctx {
     int64_t points_in = 0;             // -1: the count is on the device only (ftr_splat_depth_async)
     bool depth_async = false;          // the frame's points come from ftr_splat_depth_async
     unsigned long long* d_dropped = nullptr;
-    int* d_wild = nullptr;     // bit 0: some accepted weight lies outside [0, 1], bit 1: a normal component beyond 3.9
+    int* d_wild = nullptr;     // set when some accepted weight lies outside [0, 1] or a normal component beyond 1.99
     void* d_stage = nullptr;   // staging for host inputs
     size_t stage_cap = 0;
 

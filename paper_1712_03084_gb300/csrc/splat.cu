@@ -69,6 +69,9 @@ __device__ __forceinline__ Run run_of(int b, int lane) {
     return r;
 }
 
+constexpr float kTameNormal = 1.99f;   // normal components below it: 1024 x (1.99 2^20 + 1/2) < 2^31
+static_assert(kSplatChunk <= 1024, "the sums of one unit fit the 32-bit halves");
+
 // One point: t per axis with every decision equal to the float64 one, the
 // acceptance test, and the point record at slot `dst`.
 // An accepted point also counts itself into every brick its stencil overlaps
@@ -76,7 +79,7 @@ __device__ __forceinline__ Run run_of(int b, int lane) {
 // Called by whole warps; lanes without a point have live = false.
 __device__ __forceinline__ void ingest_one(bool live, const float* p, const float* q, const float* wp, int64_t dst, const GridDev& g,
                                            int4* pbase, float4* pfrac, float4* pnrm, unsigned long long* dropped,
-                                           int* wild_weights, int* cnt) {
+                                           int* wild, int* cnt) {
     bool ok = live;
     int fl[3] = {0, 0, 0};
     float fr[3] = {0.f, 0.f, 0.f};
@@ -138,11 +141,11 @@ __device__ __forceinline__ void ingest_one(bool live, const float* p, const floa
     }
     if (!live) return;
     pbase[dst] = rec;
-    // outside the range of the accumulation's 32-bit halves (bit 0) or of its
-    // conversions by magic addition (bit 1)
-    const bool wild_w = !(wi >= 0.f && wi <= 1.f);
-    const bool wild_n = !(fabsf(q3[0]) < 3.9f && fabsf(q3[1]) < 3.9f && fabsf(q3[2]) < 3.9f);
-    if (ok && (wild_w || wild_n)) atomicOr(wild_weights, (wild_w ? 1 : 0) | (wild_n ? 2 : 0));
+    // outside the range of the accumulation's 32-bit halves: kSplatChunk contributions
+    // of a component below 2 can all fall on one node
+    const bool tame = wi >= 0.f && wi <= 1.f && fabsf(q3[0]) < kTameNormal && fabsf(q3[1]) < kTameNormal &&
+                      fabsf(q3[2]) < kTameNormal;
+    if (ok && !tame) atomicOr(wild, 1);
     pfrac[dst] = make_float4(fr[0], fr[1], fr[2], wi);
     pnrm[dst] = make_float4(q3[0], q3[1], q3[2], 0.f);
 }
@@ -150,7 +153,7 @@ __device__ __forceinline__ void ingest_one(bool live, const float* p, const floa
 // n_dev (nullable): the point count on the device; n then only bounds it.
 __global__ void k_ingest(const float* __restrict__ pts, const float* __restrict__ nrm,
                          const float* __restrict__ w, int64_t n, int64_t base, GridDev g, int4* pbase,
-                         float4* pfrac, float4* pnrm, unsigned long long* dropped, int* wild_weights,
+                         float4* pfrac, float4* pnrm, unsigned long long* dropped, int* wild,
                          int64_t* npts_dev, const int* __restrict__ n_dev, int* cnt) {
     pdl_wait();
     if (n_dev) n = min(n, (int64_t)*n_dev);
@@ -158,14 +161,14 @@ __global__ void k_ingest(const float* __restrict__ pts, const float* __restrict_
     for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n; i0 += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = i0 + threadIdx.x;
         ingest_one(i < n, pts + 3 * i, nrm + 3 * i, w ? w + i : nullptr, base + i, g, pbase, pfrac, pnrm, dropped,
-                   wild_weights, cnt);
+                   wild, cnt);
     }
 }
 
 // Several point sets in one launch: thread i ingests point i of the
 // concatenation of the sets (set order, as separate launches would store them).
 __global__ void k_ingest_sets(IngestSets S, GridDev g, int4* pbase, float4* pfrac, float4* pnrm,
-                              unsigned long long* dropped, int* wild_weights, int64_t* npts_dev, int* cnt) {
+                              unsigned long long* dropped, int* wild, int64_t* npts_dev, int* cnt) {
     pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) *npts_dev = S.base + S.off[S.k];
@@ -173,7 +176,7 @@ __global__ void k_ingest_sets(IngestSets S, GridDev g, int4* pbase, float4* pfra
     while (s + 1 < S.k && i >= S.off[s + 1]) ++s;
     const int64_t j = i - S.off[s];
     ingest_one(i < S.off[S.k], S.pts[s] + 3 * j, S.nrm[s] + 3 * j, S.w[s] ? S.w[s] + j : nullptr, S.base + i, g, pbase, pfrac, pnrm,
-               dropped, wild_weights, cnt);
+               dropped, wild, cnt);
 }
 
 // Grid-stride over the stored points; the count is read on the device, so the
@@ -225,8 +228,8 @@ constexpr int kScanT = 256;
 constexpr int kTile = kBrickScanTile;
 static_assert(kTile % kScanT == 0, "a tile is a whole number of block scans");
 // A brick's pairs are accumulated in chunks of at most kChunk (point, brick)
-// pairs, one chunk per CTA at a time; the 32-bit hi/lo accumulators stay exact
-// for up to 2047 contributions per voxel.
+// pairs, one chunk per CTA at a time; the 32-bit hi/lo accumulators hold that many
+// contributions of weight 1 and a normal component below 1.99 on one voxel.
 constexpr int kChunk = kSplatChunk;
 constexpr int kHeavyUnit = 1 << 30;   // the unit's brick has more than one chunk
 
@@ -439,20 +442,12 @@ __device__ __forceinline__ float fix_to_float(long long v) {
 
 constexpr int kStage = kAccThreads;   // point records staged in shared memory per batch (one per thread)
 
-// Fixed-point contribution round(v * 2^40) = hi 2^20 + lo with two float to
-// int conversions: hi = round(v 2^20); r = v - hi 2^-20 is exact (Sterbenz,
-// or r = v when hi = 0) with |r| <= 2^-21, and lo = round(r 2^40) in
-// [-2^19, 2^19].  Ties go to even as in a direct conversion (hi 2^20 is even).
+// Fixed-point contribution round(v * 2^40) = hi 2^20 + lo of |v| < 4: hi = round(v
+// 2^20); r = v - hi 2^-20 is exact (Sterbenz, or r = v when hi = 0) with |r| <= 2^-21,
+// and lo = round(r 2^40) in [-2^19, 2^19].  Ties go to even as in a direct conversion
+// (hi 2^20 is even).  Adding 1.5 2^23 rounds to an integer and leaves it in the low
+// mantissa bits: conversions run on a unit with a quarter of the rate.
 __device__ __forceinline__ void fix40_split(float v, int& hi, int& lo) {
-    const float hf = rintf(v * 1048576.0f);
-    hi = (int)hf;
-    lo = __float2int_rn(fmaf(hf, -9.5367431640625e-07f, v) * 1099511627776.0f);
-}
-
-// The same for |v| < 4: adding 1.5 2^23 rounds to an integer (ties to even) and
-// leaves it in the low mantissa bits.  The three conversions per component of
-// fix40_split run on a unit with a quarter of the rate; these run at full rate.
-__device__ __forceinline__ void fix40_split_magic(float v, int& hi, int& lo) {
     constexpr float kMagic = 12582912.0f;
     const float f = __fmaf_rn(v, 1048576.0f, kMagic);
     hi = __float_as_int(f) - __float_as_int(kMagic);
@@ -473,10 +468,10 @@ __device__ __forceinline__ int acc_of(int li) { return (li & 63) + kPlane * (li 
 // that fall inside the brick (2.9 of 4 on average), and adds the fixed-point
 // contributions to shared-memory accumulators.  Integer
 // sums are exact and order-independent, so V is bit-reproducible.  32-bit
-// atomics on the (hi, lo) parts, exact while a voxel receives fewer than 2^11
-// contributions of magnitude <= 1 (a chunk has at most kChunk points; weights
-// in [0, 1]: |sum hi| < 2^31, |sum lo| < 2^30); weights outside [0, 1] take
-// 64-bit shared atomics.  A brick of one chunk writes V directly; the chunks
+// atomics on the (hi, lo) parts: a chunk has at most kChunk = 1024 points, so with
+// weights in [0, 1] and normal components below 1.99 |sum hi| < 2^31 and |sum lo| <=
+// 2^29; a frame with a weight or a normal outside takes 64-bit shared atomics
+// throughout.  A brick of one chunk writes V directly; the chunks
 // of a heavier brick add their exact sums into its int64 accumulator in
 // global memory, and the chunk that completes last (a per-brick counter)
 // writes V and clears the accumulator for the next frame.
@@ -495,7 +490,7 @@ __global__ void __launch_bounds__(kAccThreads, 6) k_splat_accum(GridDev g, int* 
                                                                 const int4* __restrict__ pbase,
                                                                 const float4* __restrict__ pfrac,
                                                                 const float4* __restrict__ pnrm,
-                                                                const int* __restrict__ wild_weights,
+                                                                const int* __restrict__ wild,
                                                                 float* __restrict__ vpool,
                                                                 const int* __restrict__ unit_off,
                                                                 const int* __restrict__ heavy_idx,
@@ -515,8 +510,7 @@ __global__ void __launch_bounds__(kAccThreads, 6) k_splat_accum(GridDev g, int* 
     // packed node coordinates: fields at bits 0, 12 and 24, biased by 8, so that
     // a coordinate lies in the brick iff bit 3 is set and bit 4 clear
     const unsigned lane_off = (unsigned)(ox | (oy << 12));
-    const int wild = wild_weights[0];
-    const bool fast = !(wild & 1), magic = wild == 0;                   // block-uniform
+    const bool fast = wild[0] == 0;                                     // block-uniform
     const int nunits = meta[5];
     if (blockIdx.x == 0 && tid < 2 * kSizeClasses) meta[kMetaClasses + tid] = 0;   // for the next frame's binning
     for (int unit = blockIdx.x; unit < nunits;) {
@@ -570,15 +564,7 @@ __global__ void __launch_bounds__(kAccThreads, 6) k_splat_accum(GridDev g, int* 
                         const float e2v = expf(-r2 * g.inv_s2sq) * fr.w;   // sigma2 * g2 * W
                         const int li = lxy + kPlane * (zc + oz);
                         const float val[4] = {e1v * nr.x, e1v * nr.y, e1v * nr.z, e2v};
-                        if (magic) {
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                int hi, lo;
-                                fix40_split_magic(val[c], hi, lo);
-                                atomicAdd(reinterpret_cast<int*>(&acc[c][li]), hi);
-                                atomicAdd(reinterpret_cast<int*>(&acc[4 + c][li]), lo);
-                            }
-                        } else if (fast) {
+                        if (fast) {
 #pragma unroll
                             for (int c = 0; c < 4; ++c) {
                                 int hi, lo;
