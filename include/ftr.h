@@ -442,6 +442,13 @@ int ftr_debug_buffer(ftr_ctx* ctx, int which, void* out, int64_t bytes);
  * without making a GPU wait run out.  FTR_EINVAL if the context has no such
  * flag (which = 0 on an FP32 context). */
 int ftr_debug_raise_wait_flag(ftr_ctx* ctx, int which);
+/* Host arithmetic, no GPU: whether ftr_mesh_copy(_async) may store `bytes` to a
+ * destination with a kernel of the context's device (1) or leaves it to the
+ * driver's copy (0), from what cudaPointerGetAttributes says of it (type,
+ * device), the context's and the calling thread's device, its address and the
+ * bytes from there to the end of its allocation (0: not known). */
+int ftr_debug_mesh_copy_route(int type, int device, int ctx_device, int current_device, uint64_t address,
+                              uint64_t room, uint64_t bytes);
 /* The generated marching-cubes table: ntri[256] and tris[256 * 5 * 3] (-1 padded). */
 int ftr_mc_table(int32_t* ntri, int32_t* tris);
 /* Per-stage device time accounting (CUDA events on the context stream). */

@@ -1,6 +1,7 @@
 // C ABI of the reconstruction library: context lifetime, staging of host
 // inputs, the per-frame call sequence and the inspection hooks.  See
 // include/ftr.h for the contract of every entry point.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdarg.h>
@@ -131,6 +132,26 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+}  // namespace
+
+size_t ftr::room_behind(const void* p) {
+    using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Range range = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return (Range)fn;
+    }();
+    CUdeviceptr base = 0;
+    size_t bytes = 0;
+    if (!range || range(&base, &bytes, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return 0;
+    return bytes - (size_t)((CUdeviceptr)(uintptr_t)p - base);
+}
+
+namespace {
 cudaError_t ensure_stage(ftr_ctx* c, void** buf, size_t* cap, size_t bytes) {
     if (*cap >= bytes) return cudaSuccess;
     if (*buf) cudaFree(*buf);
@@ -845,13 +866,34 @@ int ftr_extract_mesh(ftr_ctx* c, ftr_mesh* out) {
     return FTR_OK;
 }
 
+int ftr_debug_mesh_copy_route(int type, int device, int ctx_device, int current_device, uint64_t address,
+                              uint64_t room, uint64_t bytes) {
+    return type == cudaMemoryTypeDevice && device == ctx_device && current_device == ctx_device &&
+           address % sizeof(uint32_t) == 0 && bytes <= room;
+}
+
 namespace {
-// Enqueue the copies of the mesh arrays that are asked for: one kernel when
-// every destination is device memory, else a copy per array.
+// Whether the copy kernel may store `bytes` at p: to what it may not map, align or
+// hold, the driver's copy goes instead (another GPU's memory, managed memory, an odd
+// address) or refuses (a buffer too small).
+bool kernel_may_store(const ftr_ctx* c, const void* p, size_t bytes) {
+    cudaPointerAttributes a;
+    int current = -1;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&current) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return ftr_debug_mesh_copy_route(a.type, a.device, c->device, current, (uint64_t)(uintptr_t)p, room_behind(p),
+                                     bytes) != 0;
+}
+
+// Enqueue the copies of the mesh arrays that are asked for: one kernel when it
+// may store to every destination, else a copy per array.
 cudaError_t enqueue_mesh_copy(ftr_ctx* c, float* vertices, float* normals, int32_t* tris) {
     const size_t vb = sizeof(float) * 3 * (size_t)c->n_verts, tb = sizeof(int32_t) * 3 * (size_t)c->n_tris;
     const bool v = vertices && vb, n = normals && vb, t = tris && tb;
-    if ((!v || is_device_ptr(vertices)) && (!n || is_device_ptr(normals)) && (!t || is_device_ptr(tris)))
+    if ((!v || kernel_may_store(c, vertices, vb)) && (!n || kernel_may_store(c, normals, vb)) &&
+        (!t || kernel_may_store(c, tris, tb)))
         return launch_mesh_copy(c, v ? vertices : nullptr, n ? normals : nullptr, t ? tris : nullptr);
     cudaError_t e = cudaSuccess;
     if (v) e = cudaMemcpyAsync(vertices, c->d_verts, vb, cudaMemcpyDefault, c->stream);

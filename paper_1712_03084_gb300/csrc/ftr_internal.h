@@ -352,7 +352,8 @@ int mc_words_per_row(int nx);                  // padded words per grid row of t
 bool mc_plan_valid(int tile, int tris_per_sm);
 cudaError_t launch_mc_count(ftr_ctx* c);       // inside bits, then tile and group counts
 cudaError_t launch_mc_emit(ftr_ctx* c);        // offsets and node records, then vertices and triangles
-cudaError_t launch_mesh_copy(ftr_ctx* c, float* verts, float* nrm, int32_t* tris);   // to device buffers (null: not)
+cudaError_t launch_mesh_copy(ftr_ctx* c, float* verts, float* nrm, int32_t* tris);   // to buffers of c->device (null: not)
+size_t room_behind(const void* p);             // bytes from p to the end of its allocation; 0 if not known (api.cu)
 cudaError_t launch_raise_flag(ftr_ctx* c, int* flag);
 cudaError_t launch_mc_classes(ftr_ctx* c, uint8_t* out_dev);
 cudaError_t launch_dense_V(ftr_ctx* c, float* out_dev);

@@ -139,6 +139,7 @@ _SIGNATURES = [
     ("ftr_get_inside_mask", ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
     ("ftr_debug_buffer", ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_int64]),
     ("ftr_debug_raise_wait_flag", ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
+    ("ftr_debug_mesh_copy_route", ctypes.c_int, [ctypes.c_int] * 4 + [ctypes.c_uint64] * 3),
     ("ftr_mc_table", ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
     ("ftr_profile_enable", ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
     ("ftr_profile_read", ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int]),
