@@ -31,7 +31,8 @@
 // (an edge function within its bound of zero), and the float64 work left (a
 // depth per covered pixel that is not behind the surface already there) is
 // queued per CTA so that it runs on full warps.  A triangle projected more
-// than 2^20 pixels away, or not to a number, takes the float64 path throughout.
+// than 2^20 pixels away, or not to a number, takes the float64 path throughout,
+// and so do all triangles where the vertices cannot be projected ahead (see ftr_render).
 // The colours are float32 (they only feed the final rounding to u8).
 #include <cuda_runtime.h>
 #include <math.h>
@@ -301,7 +302,9 @@ __global__ void __launch_bounds__(kRasterThreads) k_raster(
         }
     }
     bool exact = false;
-    if (draw) {
+    if (draw && !xyz) {                              // uniform: nothing is projected
+        exact = true;
+    } else if (draw) {
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
             C[m] = xyz[id[m]];
@@ -618,24 +621,38 @@ int ftr_render(ftr_ctx* c, const ftr_render_src* src, const ftr_camera* cam, flo
         int* nbig = ev->big + src->n_tris;
         if ((e = cudaMemsetAsync(nbig, 0, sizeof(int), c->stream)) != cudaSuccess)
             return cuda_fail(c, e, "ftr_render: clear");
-        // scratch: at, xyz, vd (3 doubles per vertex), slopes (w + h doubles)
+        // scratch: at, xyz, vd (3 doubles per vertex), slopes (w + h doubles).
+        // n_vertices may be no more than a bound: k_project reads every vertex up to
+        // it, so it runs only where they all lie in the array's allocation and where
+        // triangles that share no vertex would name as many; else each triangle reads
+        // its own three.
         const int64_t nv = src->n_vertices, nslope = (int64_t)cam->w + cam->h;
         const size_t need = (size_t)nv * (16 + 16 + 24) + (size_t)nslope * 8;
-        if (need > ev->proj_cap) {
+        bool project = nv <= 3 * src->n_tris && room_behind(src->vertices) >= (size_t)nv * 3 * sizeof(float);
+        if (project && need > ev->proj_cap) {
             cudaStreamSynchronize(c->stream);
             if (ev->proj) cudaFree(ev->proj);
             ev->proj = nullptr;
             ev->proj_cap = 0;
-            if ((e = cudaMalloc(&ev->proj, need)) != cudaSuccess) return cuda_fail(c, e, "ftr_render: vertices");
-            ev->proj_cap = need;
+            if (cudaMalloc(&ev->proj, need) == cudaSuccess) {
+                ev->proj_cap = need;
+            } else {
+                cudaGetLastError();
+                ev->proj = nullptr;
+                project = false;
+            }
         }
-        float4* at = static_cast<float4*>(ev->proj);
-        float4* xyz = at + nv;
-        double* vd = reinterpret_cast<double*>(xyz + nv);
-        double* slope = vd + 3 * nv;
-        k_project<<<(unsigned)((nv + nslope + 255) / 256), 256, 0, c->stream>>>(cd, src->vertices, nv, at, xyz, vd,
-                                                                                          slope);
-        c->launches++;
+        float4 *at = nullptr, *xyz = nullptr;
+        double *vd = nullptr, *slope = nullptr;
+        if (project) {
+            at = static_cast<float4*>(ev->proj);
+            xyz = at + nv;
+            vd = reinterpret_cast<double*>(xyz + nv);
+            slope = vd + 3 * nv;
+            k_project<<<(unsigned)((nv + nslope + 255) / 256), 256, 0, c->stream>>>(cd, src->vertices, nv, at, xyz,
+                                                                                    vd, slope);
+            c->launches++;
+        }
         k_raster<<<(unsigned)((src->n_tris + kRasterThreads - 1) / kRasterThreads), kRasterThreads, 0, c->stream>>>(
             cd, src->vertices, src->tris, src->n_tris, nv, at, xyz, vd, slope, ev->zkey, ev->big, nbig);
         k_raster_big<<<2 * 152, 256, 0, c->stream>>>(cd, src->vertices, src->tris, src->n_vertices, ev->zkey, ev->big,
