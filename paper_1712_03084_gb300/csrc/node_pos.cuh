@@ -27,11 +27,14 @@ __device__ __forceinline__ double node_t(double x, double bmin, double h, double
 
 // The same t without float64 arithmetic: x - b_min exactly as a sum of two
 // floats (two-sum), times 1/h held as a float pair, gives t = th + tl with an
-// error below 1e-11 for t < 2^9 (|tl| stays below ~5e-5).  The fraction
-// r = (th - floor th) + tl is rounded once (error < 6e-8); floor(t), the
-// nearest-node round-up and acceptance (floor(t) in [1, n - 3]) follow from
-// it.  Returns false when r lies within 1e-6 of 0, 1/2 or 1, where node_t
-// decides instead.
+// error below 1e-11 for t < 2^9 (|tl| stays below ~6e-5).  The fraction
+// r = (th - floor th) + tl is rounded once, by at most 2^-25 as the float64 one
+// would be: where t lies past the node that th falls short of, r is formed from
+// the exact difference to that node (1 + 5e-5 would round by 2^-24), and below
+// floor th the small remainder is the only other rounding.  floor(t), the
+// nearest-node round-up and acceptance (floor(t) in [1, n - 3]) follow from it.
+// Returns false when r lies within 1e-6 of 0, 1/2 or 1, where node_t decides
+// instead.
 __device__ __forceinline__ bool node_t_pair(float x, float bmin, float ih, float ih_lo, int& fl, float& fr,
                                             bool& up) {
     const float s = x - bmin;
@@ -50,7 +53,7 @@ __device__ __forceinline__ bool node_t_pair(float x, float bmin, float ih, float
         r += 1.0f;
         fi -= 1;
     } else if (r > 1.0f) {
-        r -= 1.0f;
+        r = (th - f - 1.0f) + tl;                  // th - f - 1 is exact too
         fi += 1;
     }
     fl = fi;
