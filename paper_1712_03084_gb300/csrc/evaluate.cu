@@ -35,6 +35,8 @@
 #include <math.h>
 
 #include <limits>
+#include <mutex>
+#include <set>
 
 #include "ftr_internal.h"
 
@@ -747,6 +749,22 @@ bool dev_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Shared memory of k_ev_cols for an image of h rows.
+size_t col_smem(int h) { return (size_t)((h + 31) / 32) * 64 * sizeof(unsigned); }
+
+// The limit belongs to the function on the device, for every context and host
+// thread: raised once, to the largest image's 128 KB, and never lowered between
+// another thread's check and its launch.
+cudaError_t allow_col_smem(int device) {
+    static std::mutex mu;
+    static std::set<int> done;
+    std::lock_guard<std::mutex> lk(mu);
+    if (done.count(device)) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(k_ev_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)col_smem(16384));
+    if (e == cudaSuccess) done.insert(device);
+    return e;
+}
+
 template <class T>
 cudaError_t grow(T** p, int64_t* cap, int64_t need) {
     if (*cap >= need) return cudaSuccess;
@@ -865,12 +883,10 @@ int ftr_eval_geometry(ftr_ctx* c, const ftr_camera* cam, const float* rendered_d
     if ((e = cudaMemsetAsync(ev->cnt, 0, kCounters * sizeof(unsigned long long), st)) != cudaSuccess)
         return cuda_fail(c, e, "ftr_eval_geometry");
     const int nseg = (h + 31) / 32;
-    const size_t col_smem = (size_t)nseg * 64 * sizeof(unsigned);     // 128 KB at the largest height
-    if (col_smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(k_ev_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)col_smem)) != cudaSuccess)
+    if (col_smem(h) > 48 * 1024 && (e = allow_col_smem(c->device)) != cudaSuccess)
         return cuda_fail(c, e, "ftr_eval_geometry: column masks");
-    k_ev_cols<<<(w + 31) / 32, 32 * (nseg < 16 ? nseg : 16), col_smem, st>>>(rendered_depth, sensor_depth, w, h, nseg,
-                                                                            colG, colR, ev->cnt);
+    k_ev_cols<<<(w + 31) / 32, 32 * (nseg < 16 ? nseg : 16), col_smem(h), st>>>(rendered_depth, sensor_depth, w, h,
+                                                                               nseg, colG, colR, ev->cnt);
     k_ev_rows<<<h, 256, 0, st>>>(rendered_depth, sensor_depth, w, colG, colR, ev->cnt);
     Intr in;
     for (int j = 0; j < 9; ++j) in.K[j] = cam->K[j];
