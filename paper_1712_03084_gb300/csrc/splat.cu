@@ -702,6 +702,7 @@ inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t
 cudaError_t launch_ingest(ftr_ctx* c, const float* pts, const float* nrm, const float* w, int64_t n,
                           const int* n_dev) {
     if (n == 0) return cudaSuccess;
+    if (cudaError_t e = cudaGetLastError()) return e;    // see launch_ingest_sets
     // small CTAs spread the few float64 operations per point over every SM; with
     // the count on the device (n = every depth pixel) they stride over it: a CTA
     // per 32 pixels ran 40,704 CTAs for 65,000 points, 24 us
@@ -713,9 +714,13 @@ cudaError_t launch_ingest(ftr_ctx* c, const float* pts, const float* nrm, const 
     return cudaGetLastError();
 }
 
+// The ingest counts its points into their bricks, which a second call would do
+// again.  So an error that the application left on the thread, which ends the call,
+// is looked for before the launch and not only behind it.
 cudaError_t launch_ingest_sets(ftr_ctx* c, const IngestSets& S) {
     const int64_t n = S.off[S.k];
     if (n == 0) return cudaSuccess;
+    if (cudaError_t e = cudaGetLastError()) return e;
     launch_pdl(k_ingest_sets, blocks_for(n, 32), 32, 0, c->stream, S, c->g, c->pts.base, c->pts.frac, c->pts.nrm,
                c->d_dropped, c->d_wild, c->d_npts, c->d_brick_cnt);
     c->launches++;
