@@ -243,10 +243,8 @@ void free_all(ftr_ctx* c) {
     dfree(c->pts.nrm);
     if (c->d_stage) cudaFree(c->d_stage);
     dfree(c->d_brick_cnt);
-    dfree(c->d_brick_off);
     dfree(c->d_brick_cursor);
     dfree(c->d_brick_slot);
-    dfree(c->d_active);
     dfree(c->d_meta);
     dfree(c->d_tile);
     dfree(c->d_unit_off);
@@ -381,10 +379,8 @@ int ftr_create(const int grid_n[3], const float bbox[6], const ftr_params* p, ft
     c->d_dropped = reinterpret_cast<unsigned long long*>(c->d_npts + 1);
     c->d_wild = reinterpret_cast<int*>(c->d_dropped + 1);
     c->reset_bytes = sizeof(int) * (counters + 6);
-    ALLOC(c->d_brick_off, c->n_bricks + 1);
     ALLOC(c->d_brick_cursor, counters);
     ALLOC(c->d_brick_slot, c->n_bricks);
-    ALLOC(c->d_active, c->n_bricks);
     ALLOC(c->d_meta, kMetaInts);
     ALLOC(c->d_tile, (c->n_bricks + kBrickScanTile - 1) / kBrickScanTile + 1);
     ALLOC(c->d_unit_off, c->n_bricks + 1);
@@ -1647,7 +1643,7 @@ int64_t context_bytes(const int n[3], const Caps& k) {
     int64_t b = 0;
     b += k.pts * (int64_t)(sizeof(int4) + 2 * sizeof(float4));
     b += k.stage + k.tex_stage;
-    b += (nb * 3 + 2 * (nb << count_shift((int)nb))) * (int64_t)sizeof(int) + (nb / kBrickScanTile + 1) * (int64_t)sizeof(int4) + 64;
+    b += (nb + 2 * (nb << count_shift((int)nb))) * (int64_t)sizeof(int) + (nb / kBrickScanTile + 1) * (int64_t)sizeof(int4) + 64;
     b += k.entries * (int64_t)sizeof(int);
     b += k.units * (int64_t)sizeof(int4);
     b += k.heavy * (4 * kBrickVox * 8 + 4) + nb * 8;   // heavy-brick accumulators, chunk offsets

@@ -373,7 +373,6 @@ __global__ void __launch_bounds__(kFxLines * Plan<N>::N1, N >= 384 ? 2 : 3)
     constexpr int ZS = kFxLines + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_slot[2][NB];
-    __shared__ int s_any;
     const int ny = g.n[1], nz = g.n[2];
     const int y0 = blockIdx.x * kFxRows;
     const int z = blockIdx.y;
@@ -382,27 +381,12 @@ __global__ void __launch_bounds__(kFxLines * Plan<N>::N1, N >= 384 ? 2 : 3)
     live_z_range(meta, zl, zh);
     if (z < zl || z >= zh) return;
     if (!((live_rows(meta, z) >> blockIdx.x) & 1u)) return;   // zero rows: the y pass does not read them
-    if (tid == 0) s_any = 0;
-    __syncthreads();
     const int bz = z >> 3;
     for (int k = tid; k < 2 * NB; k += blockDim.x) {
         const int r = k / NB, bx = k % NB;
-        const int s = slot_tab[bx + g.nb[0] * ((y0 >> 3) + r + g.nb[1] * bz)];
-        s_slot[r][bx] = s;
-        if (s >= 0) s_any = 1;
+        s_slot[r][bx] = slot_tab[bx + g.nb[0] * ((y0 >> 3) + r + g.nb[1] * bz)];
     }
     __syncthreads();
-    if (!s_any) {
-        const float2 zero = make_float2(0.f, 0.f);
-        for (int k = tid; k < kFxRows * NKX; k += blockDim.x) {
-            const int r = k & (kFxRows - 1), kx = k >> 4;
-            const size_t o = (size_t)(y0 + r) + (size_t)ny * (z + (size_t)nz * kx);
-            s0[o] = zero;
-            s0[Mh + o] = zero;
-            s0[2 * Mh + o] = zero;
-        }
-        return;
-    }
     E e;
     e.init(smem_raw, table, tw, err);
     // the transformed lines are parked in the operand buffers, which are free

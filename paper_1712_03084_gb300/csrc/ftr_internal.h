@@ -130,10 +130,8 @@ struct ftr_ctx {
     int n_bricks = 0;
     int* d_brick_cnt = nullptr;   // first of the block that ftr_reset clears (d_npts, d_dropped, d_wild follow)
     size_t reset_bytes = 0;
-    int* d_brick_off = nullptr;
     int* d_brick_cursor = nullptr;
     int* d_brick_slot = nullptr;
-    int* d_active = nullptr;
     int* d_meta = nullptr;     // [0] active bricks, [1] entries, [2] min bz, [3] max bz, [4] accumulation
                                // ticket, [5] accumulation chunks, [6] heavy bricks,
                                // [kMetaRows + bz] live 16-row groups of brick layer bz

@@ -222,8 +222,8 @@ __global__ void k_brick_fill(const int4* __restrict__ pbase, const int64_t* __re
 // Exclusive scan of the brick counts in three coalesced launches over tiles
 // of kTile bricks: (1) per-tile sums of the counts and of the touched
 // bricks, (2) each tile adds up the sums before it, rescans itself with
-// that offset and writes the brick offsets, the dense slot of every
-// touched brick (-1 otherwise), the list of touched bricks and the z-range.
+// that offset and writes the fill cursors, the dense slot of every touched
+// brick (-1 otherwise), the accumulation units and the z-range.
 constexpr int kScanT = 256;
 constexpr int kTile = kBrickScanTile;
 static_assert(kTile % kScanT == 0, "a tile is a whole number of block scans");
@@ -325,8 +325,8 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_sums(const int* __restric
 // summed by every CTA itself (no separate scan launch); CTA 0 also writes the
 // totals.  Then the tile's bricks get their offsets, slots and chunk ranges.
 __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restrict__ cnt, int nb, int nbx, int nbxy,
-                                                             const int4* __restrict__ tile_sum, int ntiles, int* off,
-                                                             int* cursor, int* slot, int* active, int* meta,
+                                                             const int4* __restrict__ tile_sum, int ntiles,
+                                                             int* cursor, int* slot, int* meta,
                                                              int* unit_off, int* heavy_idx, int4* units) {
     pdl_wait();
     __shared__ int4 sh[kScanT / 32];
@@ -353,7 +353,6 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restri
     block_scan4(pre, run, sh);
     block_scan4(all, total, sh);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        off[nb] = total.x;
         unit_off[total.y] = total.z;   // end of the last touched brick's chunks
         meta[0] = total.y;
         meta[1] = total.x;
@@ -388,12 +387,10 @@ __global__ void __launch_bounds__(kScanT) k_brick_tile_write(const int* __restri
         }
         __syncthreads();
         if (b < nb) {
-            off[b] = run.x + ex.x;
             cursor[b << shift] = run.x + ex.x;
             if (c > 0) {
                 const int s = run.y + ex.y;
                 slot[b] = s;
-                active[s] = b;
                 unit_off[s] = run.z + ex.z;
                 // per chunk all that its CTA needs: brick, slot, first pair, pairs (| kHeavyUnit)
                 const int hv = q.w ? kHeavyUnit : 0;
@@ -678,7 +675,7 @@ __global__ void k_dense_V(GridDev g, const int* __restrict__ slot, const float* 
         out[c * M + q] = s >= 0 ? vpool[(size_t)s * 3 * kBrickVox + c * kBrickVox + li] : 0.f;
 }
 
-__global__ void k_load_dense_V(GridDev g, const float* __restrict__ V, int64_t M, int* slot, int* active,
+__global__ void k_load_dense_V(GridDev g, const float* __restrict__ V, int64_t M, int* slot,
                                float* vpool) {
     int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= M) return;
@@ -687,10 +684,7 @@ __global__ void k_load_dense_V(GridDev g, const float* __restrict__ V, int64_t M
     const int z = (int)(q / ((int64_t)g.n[0] * g.n[1]));
     const int b = (x >> 3) + g.nb[0] * ((y >> 3) + g.nb[1] * (z >> 3));
     const int li = (x & 7) + 8 * ((y & 7) + 8 * (z & 7));
-    if (li == 0) {
-        slot[b] = b;
-        active[b] = b;
-    }
+    if (li == 0) slot[b] = b;
 #pragma unroll
     for (int c = 0; c < 3; ++c) vpool[(size_t)b * 3 * kBrickVox + c * kBrickVox + li] = V[c * M + q];
 }
@@ -755,7 +749,7 @@ cudaError_t launch_splat(ftr_ctx* c) {
     const int ntiles = (c->n_bricks + kTile - 1) / kTile;
     launch_pdl(k_brick_tile_sums, ntiles, kScanT, 0, c->stream, c->d_brick_cnt, c->n_bricks, c->d_tile, c->d_meta);
     launch_pdl(k_brick_tile_write, ntiles, kScanT, 0, c->stream, c->d_brick_cnt, c->n_bricks, c->g.nb[0], c->g.nb[0] * c->g.nb[1],
-               c->d_tile, ntiles, c->d_brick_off, c->d_brick_cursor, c->d_brick_slot, c->d_active, c->d_meta,
+               c->d_tile, ntiles, c->d_brick_cursor, c->d_brick_slot, c->d_meta,
                c->d_unit_off, c->d_heavy_idx, c->d_units);
     c->launches += 2;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -775,8 +769,7 @@ cudaError_t launch_splat(ftr_ctx* c) {
 }
 
 cudaError_t launch_load_dense_V(ftr_ctx* c, const float* V_dev) {
-    k_load_dense_V<<<blocks_for(c->M, 256), 256, 0, c->stream>>>(c->g, V_dev, c->M, c->d_brick_slot, c->d_active,
-                                                                 c->d_vpool);
+    k_load_dense_V<<<blocks_for(c->M, 256), 256, 0, c->stream>>>(c->g, V_dev, c->M, c->d_brick_slot, c->d_vpool);
     c->launches++;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
