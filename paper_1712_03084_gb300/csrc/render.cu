@@ -197,6 +197,8 @@ __global__ void __launch_bounds__(256) k_project(CamDev cam, const float* __rest
     }
 }
 
+constexpr int kRasterThreads = 128;
+
 // The float64 path of one triangle throughout.
 __device__ __noinline__ void raster_exact(const CamDev& cam, const float* __restrict__ verts,
                                           const int32_t* __restrict__ tris, int64_t t, int64_t nv,
@@ -212,6 +214,15 @@ __device__ __noinline__ void raster_exact(const CamDev& cam, const float* __rest
         const double dy = dd(ds(py, cam.K[5]), cam.K[4]);
         for (double px = s.x0; px <= s.x1; px += 1.0) tri_pixel(cam, s, px, py, dy, (unsigned long long)t, zkey);
     }
+}
+
+// All triangles that way: nothing is projected ahead.
+__global__ void __launch_bounds__(kRasterThreads) k_raster_exact(CamDev cam, const float* __restrict__ verts,
+                                                                 const int32_t* __restrict__ tris, int64_t nt,
+                                                                 int64_t nv, unsigned long long* __restrict__ zkey,
+                                                                 int* __restrict__ big, int* __restrict__ nbig) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < nt) raster_exact(cam, verts, tris, t, nv, zkey, big, nbig);
 }
 
 // Coverage of pixel (px, py) in float64, for a pixel whose float32 edge
@@ -271,7 +282,6 @@ __device__ __forceinline__ void depth_exact(const CamDev& cam, const double n[4]
     atomicMin(zkey + (int64_t)py * cam.w + px, key);
 }
 
-constexpr int kRasterThreads = 128;
 constexpr int kQueue = 2048;        // fragments per CTA that wait for their float64 depth (8 KB)
 
 // Measured on 152,000 triangles of a body-sized mesh: 88 us at 512 x 424 and
@@ -302,9 +312,7 @@ __global__ void __launch_bounds__(kRasterThreads) k_raster(
         }
     }
     bool exact = false;
-    if (draw && !xyz) {                              // uniform: nothing is projected
-        exact = true;
-    } else if (draw) {
+    if (draw) {
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
             C[m] = xyz[id[m]];
@@ -642,19 +650,21 @@ int ftr_render(ftr_ctx* c, const ftr_render_src* src, const ftr_camera* cam, flo
                 project = false;
             }
         }
-        float4 *at = nullptr, *xyz = nullptr;
-        double *vd = nullptr, *slope = nullptr;
+        const unsigned blocks = (unsigned)((src->n_tris + kRasterThreads - 1) / kRasterThreads);
         if (project) {
-            at = static_cast<float4*>(ev->proj);
-            xyz = at + nv;
-            vd = reinterpret_cast<double*>(xyz + nv);
-            slope = vd + 3 * nv;
+            float4* at = static_cast<float4*>(ev->proj);
+            float4* xyz = at + nv;
+            double* vd = reinterpret_cast<double*>(xyz + nv);
+            double* slope = vd + 3 * nv;
             k_project<<<(unsigned)((nv + nslope + 255) / 256), 256, 0, c->stream>>>(cd, src->vertices, nv, at, xyz,
                                                                                     vd, slope);
             c->launches++;
+            k_raster<<<blocks, kRasterThreads, 0, c->stream>>>(cd, src->vertices, src->tris, src->n_tris, nv, at, xyz,
+                                                               vd, slope, ev->zkey, ev->big, nbig);
+        } else {
+            k_raster_exact<<<blocks, kRasterThreads, 0, c->stream>>>(cd, src->vertices, src->tris, src->n_tris, nv,
+                                                                     ev->zkey, ev->big, nbig);
         }
-        k_raster<<<(unsigned)((src->n_tris + kRasterThreads - 1) / kRasterThreads), kRasterThreads, 0, c->stream>>>(
-            cd, src->vertices, src->tris, src->n_tris, nv, at, xyz, vd, slope, ev->zkey, ev->big, nbig);
         k_raster_big<<<2 * 152, 256, 0, c->stream>>>(cd, src->vertices, src->tris, src->n_vertices, ev->zkey, ev->big,
                                                      nbig);
         c->launches += 2;
