@@ -19,10 +19,11 @@ namespace {
 constexpr int kRows = 16;
 constexpr int kLines = 24;
 
-// At most 56 registers per thread up to 384 points: three CTAs per SM, two at 384
-// (there one CTA of 18 warps left its barriers and loads uncovered: 96 us, then 87; at
-// 128 points the allocator otherwise took 76 registers and two CTAs fitted: 11.8 -> 9.8
-// us at 128^3, 15.9 -> 13.9 at 128 x 256 x 128).
+// Three CTAs per SM up to 256 points, two at 384 (there one CTA of 18 warps left its
+// barriers and loads uncovered: 96 us, then 87; at 128 points the allocator otherwise
+// took 76 registers and two CTAs fitted: 11.8 -> 9.8 us at 128^3, 15.9 -> 13.9 at 128 x
+// 256 x 128).  That is at most 56 registers per thread from 128 to 384 points; the
+// shorter lengths have fewer threads and need no limit.  512 points: one CTA, not tuned.
 template <int N>
 __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT, N <= 256 ? 3 : (N == 384 ? 2 : 1))
     k_fx(GridDev g, const int* __restrict__ slot_tab, const float* __restrict__ vpool, float2* __restrict__ s0,

@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(kLines * Xchg<N, kLines>::NT)
     const int z = blockIdx.y;
     const int tid = threadIdx.x;
     const uint64_t pin = l2_evict_first(), pout = l2_evict_last();
-    const int2 later = later_block(152 * 3, (int64_t)NKX * ny * nz);
+    const int2 later = later_block(kSms * 3, (int64_t)NKX * ny * nz);
     if (later.x >= 0)
         for (int kx = tid; kx < NKX; kx += (int)blockDim.x)
             prefetch_l2(src + (size_t)(later.x * kRows) + (size_t)ny * (later.y + (size_t)nz * kx));

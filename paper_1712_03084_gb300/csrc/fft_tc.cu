@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(TcLinesZ<N>::value * Plan<N>::N1, N >= 384 && 
     live_z_range(meta, zl, zh);
     E e;
     e.init(smem_raw, table, tw, err);
-    const int2 later = later_block(152 * (P == FTR_PREC_BF16X3 ? 5 : 4), Mh);
+    const int2 later = later_block(kSms * (P == FTR_PREC_BF16X3 ? 5 : 4), Mh);
     if (tid < 2 * F && later.x >= 0 && zl < zh)
         tc::bulk_prefetch_l2(s1 + (tid < F ? 0 : Mh) +
                                  (size_t)N * ((size_t)(later.x * F + tid % F) + (size_t)ny * later.y) + zl,
@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(kIxLines * Plan<N>::N1, N >= 384 ? 5 : 9)
     // transform fills only after every thread has read its inputs
     static_assert(sizeof(float2) * kIxRows * (N / 2 + 1) <= 2 * E::APART, "staging fits the operand buffers");
     float2* hs = (float2*)e.ahi();
-    const int2 later = later_block(152 * 5, (int64_t)NKX * ny * nz);
+    const int2 later = later_block(kSms * 5, (int64_t)NKX * ny * nz);
     if (later.x >= 0)
         for (int kx = tid; kx < NKX; kx += E::T)
             prefetch_l2(src + (size_t)(later.x * kIxRows) + (size_t)ny * (later.y + (size_t)nz * kx));

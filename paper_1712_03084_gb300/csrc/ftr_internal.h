@@ -16,7 +16,8 @@ constexpr int kBrick = 8;                 // splat accumulation brick edge (node
 constexpr int kBrickVox = kBrick * kBrick * kBrick;
 constexpr int kMaxViews = 8;
 constexpr int kBrickScanTile = 256;   // bricks per tile of the brick-count scan (one block scan per CTA)
-constexpr int kMcThreads = 256;           // CTA size of the inside-bit pass (8 grid rows, a warp each)
+constexpr int kMcThreads = 256;           // CTA size of the inside-bit pass (a warp per four grid rows)
+constexpr int kSms = 152;                 // GB300; only launch shapes and prefetch distances follow from it
 constexpr int kMaxTrisPerCase = 5;
 constexpr int kSplatChunk = 1024;          // (point, brick) pairs per accumulation work unit
 
@@ -97,11 +98,13 @@ struct EvalScratch;
 
 namespace ftr {
 // The per-brick counters that points add to (ingest counts, fill cursors) lie 1 <<
-// count_shift apart: a 32-byte sector each up to 4096 bricks.  Points in no spatial
-// order add one by one, and packed counters of a small grid are a few 128-byte lines,
-// hence a few L2 slices: 20,000 random points on the 512 bricks of 64^3, ingest 15 ->
-// 9 us and scan with fill 20 -> 13.  From 8192 bricks on the packed counters spread by
-// themselves (and would take megabytes to clear and scan).
+// count_shift apart: a 32-byte sector each up to 4096 bricks (131 KB to clear and scan).
+// Points in no spatial order add one by one, and packed counters of a small grid are a
+// few 128-byte lines, hence a few L2 slices.  Ingest with scan and fill, packed -> spread:
+// 20,000 random points on a sphere 36 -> 22 us on the 512 bricks of 64^3, 24 -> 22 on
+// 4096, 23 -> 22 on 6144, 23 -> 23 on 13,824; 100,000 points 108 -> 43, 39 -> 30, 38 ->
+// 28, 32 -> 29; in spatial order 49 -> 28, 30 -> 26, 30 -> 26, 30 -> 28.  So frames of
+// many points would still gain a little past the line, which bounds the clearing.
 __host__ __device__ inline int count_shift(int bricks) { return bricks <= 4096 ? 3 : 0; }
 }  // namespace ftr
 

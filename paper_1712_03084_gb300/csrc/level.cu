@@ -144,7 +144,7 @@ double* g_noalloc_ptr[64] = {};
 // (152 SMs x 8 CTAs of 256 threads), then whole multiples of 256 that keep it
 // to one wave; at the largest n that is 3584 points on 1171 CTAs.
 int noalloc_per_cta(int64_t n) {
-    constexpr int64_t kWave = 152 * 8;
+    constexpr int64_t kWave = kSms * 8;
     const int64_t per = (n + kThreads * kWave - 1) / (kThreads * kWave);
     return kThreads * (int)(per < 1 ? 1 : per);
 }

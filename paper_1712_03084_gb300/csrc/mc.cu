@@ -700,7 +700,7 @@ cudaError_t launch_mc_emit(ftr_ctx* c) {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     prof_begin(c, ST_MC_TRIS);
-    launch_pdl(k_mc_tris, (sms > 0 ? sms : 152) * c->mc_tris_per_sm, 256, 0, c->stream, c->g, c->d_A, c->d_levelf, c->d_mc_nodes,
+    launch_pdl(k_mc_tris, (sms > 0 ? sms : kSms) * c->mc_tris_per_sm, 256, 0, c->stream, c->g, c->d_A, c->d_levelf, c->d_mc_nodes,
                (const int*)c->d_mc_tot, (int)c->cap_mc_nodes, (int)c->cap_tris, (const int2*)c->d_mc_word, wp,
                c->d_tris, c->d_verts, c->d_vnrm, (int)c->cap_verts);
     c->launches++;
@@ -713,7 +713,7 @@ cudaError_t launch_mesh_copy(ftr_ctx* c, float* verts, float* nrm, int32_t* tris
     if (!verts && !nrm && !tris) return cudaSuccess;
     const int64_t words = 3 * (c->n_verts > c->n_tris ? c->n_verts : c->n_tris);
     const int64_t blocks = (words / 4 + 255) / 256;
-    k_mesh_copy<<<(unsigned)(blocks < 1 ? 1 : (blocks > 152 * 8 ? 152 * 8 : blocks)), 256, 0, c->stream>>>(
+    k_mesh_copy<<<(unsigned)(blocks < 1 ? 1 : (blocks > kSms * 8 ? kSms * 8 : blocks)), 256, 0, c->stream>>>(
         c->d_verts, c->d_vnrm, c->d_tris, c->n_verts, c->n_tris, verts, nrm, tris);
     c->launches++;
     return cudaGetLastError();

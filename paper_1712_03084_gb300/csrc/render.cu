@@ -181,8 +181,8 @@ __global__ void __launch_bounds__(256) k_project(CamDev cam, const float* __rest
         const float vl = (e5 + e6) + cam.Kf[4] * br;
         const float ui = rintf(us), vi = rintf(vs);
         // the second terms are below 2^-23 of the sums they belong to, their own
-        // errors below 2^-45: what counts is the rounding of the rest (at most half a
-        // pixel), 2^-25, so 4e-8 covers it while the sums stay below 2^20
+        // errors below 2^-45 of them (2^-25 pixels at the limit of 2^20), and the rest
+        // (half a pixel and a second term) rounds by 2^-25: 6e-8 together
         const float size = fabsf(ua) + fabsf(ub) + fabsf(cam.Kf[2]) + fabsf(va) + fabsf(cam.Kf[5]);
         const float how = !(xc[2] >= kZNear) ? kVertSkip : (size < 1048576.f ? kVertFast : kVertExact);
         at[i] = make_float4(__int_as_float((int)ui), __int_as_float((int)vi), (us - ui) + ul, (vs - vi) + vl);
@@ -338,7 +338,8 @@ __global__ void __launch_bounds__(kRasterThreads) k_raster(
         const float xlo = fminf(fminf(X[0], X[1]), X[2]), xhi = fmaxf(fmaxf(X[0], X[1]), X[2]);
         const float ylo = fminf(fminf(Y[0], Y[1]), Y[2]), yhi = fmaxf(fmaxf(Y[0], Y[1]), Y[2]);
         const float D = fmaxf(fmaxf(xhi, yhi), -fminf(xlo, ylo)) + 1.f;      // > every coordinate used below
-        const float e = 1e-7f * D;          // > the error of X, Y: 4e-8 of the vertex + 2^-24 D of the sum
+        // > the error of X, Y: 6e-8 of the vertex and 2^-24 (D - 1) of the sum
+        const float e = 1e-7f * D;
         // pixel centres the box can hold, widened by that error
         const int x0 = max(ox + (int)ceilf(xlo - 2.f * e), 0), x1 = min(ox + (int)floorf(xhi + 2.f * e), cam.w - 1);
         const int y0 = max(oy + (int)ceilf(ylo - 2.f * e), 0), y1 = min(oy + (int)floorf(yhi + 2.f * e), cam.h - 1);
@@ -665,7 +666,7 @@ int ftr_render(ftr_ctx* c, const ftr_render_src* src, const ftr_camera* cam, flo
             k_raster_exact<<<blocks, kRasterThreads, 0, c->stream>>>(cd, src->vertices, src->tris, src->n_tris, nv,
                                                                      ev->zkey, ev->big, nbig);
         }
-        k_raster_big<<<2 * 152, 256, 0, c->stream>>>(cd, src->vertices, src->tris, src->n_vertices, ev->zkey, ev->big,
+        k_raster_big<<<2 * kSms, 256, 0, c->stream>>>(cd, src->vertices, src->tris, src->n_vertices, ev->zkey, ev->big,
                                                      nbig);
         c->launches += 2;
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "ftr_render: raster");

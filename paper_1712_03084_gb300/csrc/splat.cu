@@ -15,11 +15,11 @@
 //           brick and the accumulation chunks (no single-CTA scan)
 //   fill    per point, append its index to each overlapped brick's list
 //   accum   persistent CTAs take work units (up to 1024 (point, brick) pairs
-//           of one touched brick): 64 lanes per point
-//           evaluate the stencil nodes inside the brick and add the
-//           contributions to shared-memory fixed-point accumulators (value *
-//           2^40 as 32-bit hi/lo halves, exact and order-independent, so the
-//           result is bit-reproducible); a brick of several units adds each
+//           of one touched brick): a warp per pair evaluates the stencil nodes
+//           inside the brick and adds the contributions to shared-memory
+//           fixed-point accumulators (value * 2^40 as 32-bit hi/lo halves, exact
+//           and order-independent, so the result is bit-reproducible; 64-bit in
+//           a frame with weights or normals beyond their range); a brick of several units adds each
 //           unit's exact sums into an int64 global accumulator and its last
 //           unit writes V = (sigma2 / sigma1) U / d to the brick's slot.
 // The simple variant (nearest node floor(t + 1/2), V = mean N) uses the same
@@ -700,7 +700,7 @@ cudaError_t launch_ingest(ftr_ctx* c, const float* pts, const float* nrm, const 
     // small CTAs spread the few float64 operations per point over every SM; with
     // the count on the device (n = every depth pixel) they stride over it: a CTA
     // per 32 pixels ran 40,704 CTAs for 65,000 points, 24 us
-    const unsigned blocks = n_dev ? (unsigned)min((int64_t)152 * 32, (int64_t)blocks_for(n, 32)) : blocks_for(n, 32);
+    const unsigned blocks = n_dev ? (unsigned)min((int64_t)kSms * 32, (int64_t)blocks_for(n, 32)) : blocks_for(n, 32);
     launch_pdl(k_ingest, blocks, 32, 0, c->stream, pts, nrm, w, n, c->n_pts, c->g, c->pts.base, c->pts.frac,
                                                        c->pts.nrm, c->d_dropped, c->d_wild, c->d_npts, n_dev,
                                                        c->d_brick_cnt);
@@ -743,7 +743,7 @@ cudaError_t launch_splat(ftr_ctx* c) {
     c->class_dirty = true;                       // until the accumulation is enqueued
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    if (sms <= 0) sms = 152;
+    if (sms <= 0) sms = kSms;
     prof_begin(c, ST_SPLAT_BIN);
     // the per-brick point counts were taken by the ingest
     const int ntiles = (c->n_bricks + kTile - 1) / kTile;

@@ -208,9 +208,10 @@ __device__ __forceinline__ bool eval_camera_mixed(const ViewDev& vw, const float
 // warp-uniform constant reads and the vertices' projections fall on
 // neighbouring pixels.  (With the camera varying by lane, as before, each of
 // the ~40 parameter reads was serialised over the cameras: 300,000 vertices x
-// 6 cameras took 112 us a call, now 71 with the host's part of it showing.)  The per-camera results meet in shared memory: the
-// weights and UVs leave as one contiguous block per CTA, and a thread per
-// vertex blends in the fixed order of a binary tree over the cameras.
+// 6 cameras took 112 us a call, then 71; now 54, see pixel_of.)  The per-camera
+// results meet in shared memory: the weights and UVs leave as one contiguous block per
+// CTA, and a thread per vertex blends in the fixed order of a binary tree over the
+// cameras.
 // nv_dev (optional): the vertex count on the device; nv then bounds it.
 template <int G>
 __global__ void __launch_bounds__(256) k_texture(ViewSet vs, const float* __restrict__ verts, int64_t nv,
