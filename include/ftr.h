@@ -504,7 +504,8 @@ typedef struct {
  * floor(c + 1/2), black where nothing is drawn or no view applies.
  * Returns FTR_EINVAL for bad sizes, host pointers, n_tris >= 2^31 or a
  * colour source without rgb_out.  Triangle indices are checked on the device:
- * a triangle with an index outside [0, n_vertices) is not drawn.
+ * a triangle with an index outside [0, n_vertices) is not drawn.  n_vertices
+ * may be a loose bound: memory past the vertices' allocation is not touched.
  */
 int ftr_render(ftr_ctx* ctx, const ftr_render_src* src, const ftr_camera* cam, float* depth_out,
                uint8_t* rgb_out);
