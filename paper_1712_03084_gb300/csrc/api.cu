@@ -196,23 +196,28 @@ int64_t heavy_capacity(int64_t points) {
     return cap;
 }
 
+// A buffer that is freed to grow has no capacity until its successor is there: an
+// allocation that fails must not leave the old size standing for smaller frames.
+template <class T>
+cudaError_t regrow(T*& p, int64_t& cap, int64_t count, int64_t elems) {
+    dfree(p);
+    cap = 0;
+    const cudaError_t e = dalloc(&p, (size_t)elems);
+    if (e == cudaSuccess) cap = count;
+    return e;
+}
+
 cudaError_t grow_entries(ftr_ctx* c, int64_t need) {
-    if (need <= c->cap_entries) return cudaSuccess;
-    c->graph_valid = false;
     int64_t cap = c->cap_entries ? c->cap_entries : 1 << 18;
     while (cap < need) cap *= 2;
-    cudaStreamSynchronize(c->stream);
-    dfree(c->d_entries);
-    cudaError_t e = dalloc(&c->d_entries, cap);
-    if (e != cudaSuccess) return e;
-    c->cap_entries = cap;
     // chunks: one per touched brick plus at most cap / chunk more
     const int64_t units = (int64_t)c->n_bricks + cap / kSplatChunk + 2;
-    if (units > c->cap_units) {
-        dfree(c->d_units);
-        if ((e = dalloc(&c->d_units, (size_t)units)) != cudaSuccess) return e;
-        c->cap_units = units;
-    }
+    if (cap <= c->cap_entries && units <= c->cap_units) return cudaSuccess;
+    c->graph_valid = false;
+    cudaStreamSynchronize(c->stream);
+    cudaError_t e = cudaSuccess;
+    if (units > c->cap_units && (e = regrow(c->d_units, c->cap_units, units, units)) != cudaSuccess) return e;
+    if (cap > c->cap_entries) e = regrow(c->d_entries, c->cap_entries, cap, cap);
     return e;
 }
 
@@ -227,6 +232,7 @@ cudaError_t grow_heavy(ftr_ctx* c, int64_t points) {
         cudaStreamSynchronize(c->stream);
         dfree(c->d_heavy_acc);
         dfree(c->d_heavy_done);
+        c->cap_heavy = 0;
         if ((e = dalloc(&c->d_heavy_acc, (size_t)heavy * 4 * kBrickVox)) != cudaSuccess) return e;
         if ((e = dalloc(&c->d_heavy_done, (size_t)heavy)) != cudaSuccess) return e;
         if ((e = cudaMemset(c->d_heavy_acc, 0, sizeof(unsigned long long) * heavy * 4 * kBrickVox)) != cudaSuccess)
@@ -577,17 +583,14 @@ int raw_enqueue(ftr_ctx* c, const char* who, const ftr_view* views, int k, doubl
     if (pixels > c->raw_cap) {
         c->graph_valid = false;
         cudaStreamSynchronize(c->stream);
-        dfree(c->d_raw);
-        if ((e = dalloc(&c->d_raw, (size_t)pixels * 7)) != cudaSuccess) return cuda_fail(c, e, who);
-        c->raw_cap = pixels;
+        if ((e = regrow(c->d_raw, c->raw_cap, pixels, pixels * 7)) != cudaSuccess) return cuda_fail(c, e, who);
     }
     if (ints > c->raw_masks_cap) {
         cudaStreamSynchronize(c->stream);
-        dfree(c->d_raw_masks);
-        if ((e = dalloc(&c->d_raw_masks, (size_t)ints)) != cudaSuccess) return cuda_fail(c, e, who);
-        c->raw_masks_cap = ints;
+        if ((e = regrow(c->d_raw_masks, c->raw_masks_cap, ints, ints)) != cudaSuccess) return cuda_fail(c, e, who);
     }
-    if (!c->d_raw_total) {
+    if (!c->h_raw_total) {
+        dfree(c->d_raw_total);
         if ((e = dalloc(&c->d_raw_total, 1)) != cudaSuccess) return cuda_fail(c, e, who);
         if ((e = cudaMallocHost((void**)&c->h_raw_total, sizeof(int))) != cudaSuccess) return cuda_fail(c, e, who);
     }
@@ -799,30 +802,26 @@ namespace {
 
 // Grow the mesh buffers to hold at least (na, nv, nt) with 50 % headroom.
 cudaError_t grow_mesh(ftr_ctx* c, int64_t na, int64_t nv, int64_t nt) {
+    const auto headroom = [](int64_t n) { return n + n / 2 + 1024; };
     cudaError_t e = cudaSuccess;
-    if (na > c->cap_mc_nodes || nv > c->cap_verts || nt > c->cap_tris) c->graph_valid = false;
+    if (na <= c->cap_mc_nodes && nv <= c->cap_verts && nt <= c->cap_tris) return e;
+    c->graph_valid = false;
+    cudaStreamSynchronize(c->stream);
     if (na > c->cap_mc_nodes) {
-        cudaStreamSynchronize(c->stream);
-        dfree(c->d_mc_nodes);
-        const int64_t cap = na + na / 2 + 1024;
-        if ((e = dalloc(&c->d_mc_nodes, cap)) != cudaSuccess) return e;
-        c->cap_mc_nodes = cap;
+        const int64_t cap = headroom(na);
+        if ((e = regrow(c->d_mc_nodes, c->cap_mc_nodes, cap, cap)) != cudaSuccess) return e;
     }
     if (nv > c->cap_verts) {
-        cudaStreamSynchronize(c->stream);
+        const int64_t cap = headroom(nv);
+        c->cap_verts = 0;
         dfree(c->d_verts);
         dfree(c->d_vnrm);
-        const int64_t cap = nv + nv / 2 + 1024;
         if ((e = dalloc(&c->d_verts, 3 * cap)) != cudaSuccess) return e;
-        if ((e = dalloc(&c->d_vnrm, 3 * cap)) != cudaSuccess) return e;
-        c->cap_verts = cap;
+        if ((e = regrow(c->d_vnrm, c->cap_verts, cap, 3 * cap)) != cudaSuccess) return e;
     }
     if (nt > c->cap_tris) {
-        cudaStreamSynchronize(c->stream);
-        dfree(c->d_tris);
-        const int64_t cap = nt + nt / 2 + 1024;
-        if ((e = dalloc(&c->d_tris, 3 * cap)) != cudaSuccess) return e;
-        c->cap_tris = cap;
+        const int64_t cap = headroom(nt);
+        if ((e = regrow(c->d_tris, c->cap_tris, cap, 3 * cap)) != cudaSuccess) return e;
     }
     return e;
 }
